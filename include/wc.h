@@ -307,10 +307,9 @@ wc_status wc_count_noalloc(const uint8_t *d_text, uint64_t nbytes, uint64_t *d_k
 /* The paper's numeric MapReduce (Sec. 4.2): *d_out (one device double) =
  * sum_{i=1}^{n} term(i) with term(i) = sqrt(i) (WC_SERIES_SQRT) or
  * (-1)^(i+1) / i (WC_SERIES_ALT_HARMONIC, whose limit is ln 2).  Each term is
- * an IEEE double (correctly rounded sqrt and division); the terms are summed
- * with Neumaier-compensated additions, per thread over a strided share of one
- * block's contiguous range, then over warps and blocks in a fixed order, so a
- * given GPU always returns the same value (no atomics).  n = 0 gives 0.
+ * an IEEE double (correctly rounded sqrt and division); the terms are added
+ * exactly in 128-bit integers and the sum is rounded once, so the result is
+ * the double nearest to the exact sum of the terms on any GPU.  n = 0 gives 0.
  * Asynchronous on `stream`; scratch (16 bytes a block) comes from the
  * context's pool.  Errors: WC_ERR_INVALID_ARG (unknown series, null
  * pointer), WC_ERR_UNSUPPORTED (n >= 2^53: indices no longer exact in

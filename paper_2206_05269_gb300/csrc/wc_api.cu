@@ -261,10 +261,10 @@ wc_status wc_series_sum(wc_ctx *ctx, int series, uint64_t n, double *d_out, cuda
     cudaSetDevice(ctx->device);
     const int nb = series_blocks(n);
     void *part = nullptr;
-    wc_status st = ctx->alloc(&part, sizeof(double2) * (size_t)nb, stream);
+    wc_status st = ctx->alloc(&part, sizeof(ulonglong2) * (size_t)nb, stream);
     if (st != WC_OK) return st;
-    const cudaError_t e = launch_series(series, n, static_cast<double2 *>(part), nb, d_out, stream);
-    ctx->release(part, sizeof(double2) * (size_t)nb, stream);
+    const cudaError_t e = launch_series(series, n, static_cast<ulonglong2 *>(part), nb, d_out, stream);
+    ctx->release(part, sizeof(ulonglong2) * (size_t)nb, stream);
     if (e != cudaSuccess) return ctx->cuda_fail(e, "series sum");
     ctx->launches += 2;
     return WC_OK;

@@ -68,10 +68,10 @@ cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
 }
 
 // ---------------------------------------------------------------- numeric MapReduce
-// Blocks of the series sum for n terms, and its two launches (per-block
-// compensated partial sums into part[nb], then their fixed-order sum).
+// Blocks of the series sum for n terms, and its two launches (exact per-block
+// sums into part[nb], then their sum rounded once).
 int series_blocks(unsigned long long n);
-cudaError_t launch_series(int series, unsigned long long n, double2 *part, int nb, double *d_out, cudaStream_t s);
+cudaError_t launch_series(int series, unsigned long long n, ulonglong2 *part, int nb, double *d_out, cudaStream_t s);
 
 // Row sums of a row-major uint32 matrix (the hybrid pipeline's reduce).
 cudaError_t launch_row_sums(const uint32_t *m, unsigned long long rows, unsigned long long cols,
