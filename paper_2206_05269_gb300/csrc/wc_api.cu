@@ -594,7 +594,7 @@ CapPlan plan_capacity(const wc_ctx *ctx, uint64_t nbytes, const wc_count_opts *o
 }
 
 // Allocates the hash tables (+ head-selection scratch) + sort scratch in one block.
-wc_status scratch_create(wc_ctx *ctx, const CapPlan &p, bool head, cudaStream_t s, CountScratch &cs) {
+wc_status scratch_create(wc_ctx *ctx, const CapPlan &p, bool head, cudaStream_t s, CountScratch &cs, bool radix) {
     cs.gcap8 = p.cap8;
     cs.gcap = p.cap16;
     cs.glcap = p.caplong;
@@ -602,7 +602,8 @@ wc_status scratch_create(wc_ctx *ctx, const CapPlan &p, bool head, cudaStream_t 
     const size_t b8 = r(p.cap8 * sizeof(G8Slot)), b16 = r(p.cap16 * sizeof(GSlot)), bl = r(p.caplong * sizeof(LSlot));
     const size_t hb = b8 + b16 + bl;
     const size_t bh = head ? r(head_scratch_bytes()) : 0;
-    cs.bytes = hb + bh + sort_scratch_bytes(cs.entries(), true) + 512;
+    if (cs.entries() > kBktMaxCap) radix = true;
+    cs.bytes = hb + bh + (radix ? sort_scratch_bytes(cs.entries()) : bucket_scratch_bytes(cs.entries())) + 512;
     wc_status st = ctx->alloc(&cs.mem, cs.bytes, s);
     if (st != WC_OK) return st;
     uint8_t *q = static_cast<uint8_t *>(cs.mem);
@@ -610,7 +611,8 @@ wc_status scratch_create(wc_ctx *ctx, const CapPlan &p, bool head, cudaStream_t 
     cs.slots = reinterpret_cast<GSlot *>(q + b8);
     cs.lslots = reinterpret_cast<LSlot *>(q + b8 + b16);
     cs.head = head ? q + hb : nullptr;
-    sort_scratch_carve(cs.ss, q + hb + bh, cs.entries(), true);
+    if (radix) sort_scratch_carve(cs.ss, q + hb + bh, cs.entries());
+    else bucket_scratch_carve(cs.bs, q + hb + bh, cs.entries());
     cudaMemsetAsync(cs.mem, 0, hb, s);
     return WC_OK;
 }
@@ -633,6 +635,7 @@ wc_status wc_count_ex(wc_ctx *ctx, const uint8_t *d_text, uint64_t nbytes, const
     st = table_create(ctx, cs.entries(), plan.caplong, plan.arena, ctx->count_bits, stream, &t);
     if (st != WC_OK) { ctx->release(cs.mem, cs.bytes, stream); return st; }
     t->src_bytes = nbytes;
+    t->max_tokens = nbytes / 2 + 1;
     const GTable g = cs.gtable(t->dt.d_status);
     CountLaunch cl{d_text, 0, nbytes, g, 0, cs.head, {nullptr, nullptr}};
     cl.no_level1 = opts && opts->no_level1 ? 1 : 0;
@@ -645,9 +648,9 @@ wc_status wc_count_ex(wc_ctx *ctx, const uint8_t *d_text, uint64_t nbytes, const
     ctx->launches += count_global_launches(nbytes, !cl.no_level1, cs.head != nullptr);
     ctx->prof_mark(ctx->ev_finish, stream);
     const uint32_t skip = sort_skip_mask(nbytes / 2 + 1, 0);  // no count exceeds the token bound
-    if (e == cudaSuccess) e = finish_table(g, cs.gcap8, cs.gcap, cs.glcap, cs.ss, t->dt, stream, skip);
+    if (e == cudaSuccess) e = finish_table(g, cs.gcap8, cs.gcap, cs.glcap, cs.ss, cs.bs, t->dt, stream, skip);
     ctx->prof_mark(ctx->ev_finish, stream);
-    ctx->launches += finish_table_launches(cs.ss, skip);
+    ctx->launches += finish_table_launches(cs.ss, cs.bs, skip);
     ctx->release(cs.mem, cs.bytes, stream);
     table_mark_done(t, stream);
     if (e != cudaSuccess) {
@@ -706,6 +709,7 @@ wc_status wc_count_host(wc_ctx *ctx, const uint8_t *h_text, uint64_t nbytes, uin
         return st;
     }
     t->src_bytes = nbytes;
+    t->max_tokens = nbytes / 2 + 1;
     const GTable g = cs.gtable(t->dt.d_status);
     // copies on the copy stream (after the caller's earlier work); each piece
     // is counted on the caller's stream once it has landed, so later copies
@@ -730,8 +734,8 @@ wc_status wc_count_host(wc_ctx *ctx, const uint8_t *h_text, uint64_t nbytes, uin
         ctx->launches += count_global_launches(cut[i + 1] - cut[i], i == 0 && head && !cl.no_level1, cs.head != nullptr);
     }
     const uint32_t skip = sort_skip_mask(nbytes / 2 + 1, 0);  // no count exceeds the token bound
-    if (e == cudaSuccess) e = finish_table(g, cs.gcap8, cs.gcap, cs.glcap, cs.ss, t->dt, stream, skip);
-    ctx->launches += finish_table_launches(cs.ss, skip);
+    if (e == cudaSuccess) e = finish_table(g, cs.gcap8, cs.gcap, cs.glcap, cs.ss, cs.bs, t->dt, stream, skip);
+    ctx->launches += finish_table_launches(cs.ss, cs.bs, skip);
     for (auto x : ev)
         if (x) cudaEventDestroy(x);  // released once their work completes
     ctx->release(cs.mem, cs.bytes, stream);
@@ -750,7 +754,7 @@ wc_status wc_merge(wc_ctx *ctx, const wc_table *const *in, uint32_t n, cudaStrea
     if (!ctx || !out || (n && !in)) return WC_ERR_INVALID_ARG;
     *out = nullptr;
     cudaSetDevice(ctx->device);
-    uint64_t sum_cap = 0, sum_lcap = 0, sum_arena = 0, chunks = 0;
+    uint64_t sum_cap = 0, sum_lcap = 0, sum_arena = 0, chunks = 0, max_tokens = 0;
     std::vector<MergeSrc> src(n);
     std::vector<uint64_t> cstart(n + 1, 0);
     for (uint32_t i = 0; i < n; i++) {
@@ -763,6 +767,8 @@ wc_status wc_merge(wc_ctx *ctx, const wc_table *const *in, uint32_t n, cudaStrea
         sum_cap += known ? in[i]->n : d.cap;
         sum_lcap += known ? in[i]->nlong : d.lcap;
         sum_arena += known ? in[i]->word_bytes + in[i]->nlong : d.arena_cap;
+        const uint64_t tok = known ? in[i]->tokens : in[i]->max_tokens;
+        max_tokens = tok > UINT64_MAX - max_tokens ? UINT64_MAX : max_tokens + tok;
         cstart[i] = chunks;
         chunks += (d.cap + kMergeChunk - 1) / kMergeChunk;
         cudaStreamWaitEvent(stream, in[i]->done, 0);
@@ -774,11 +780,13 @@ wc_status wc_merge(wc_ctx *ctx, const wc_table *const *in, uint32_t n, cudaStrea
     plan.caplong = pow2_at_least(std::max<uint64_t>(256, 2 * sum_lcap));
     plan.arena = std::max<uint64_t>(4096, sum_arena);
     CountScratch cs;
-    wc_status st = scratch_create(ctx, plan, false, stream, cs);
+    const uint32_t skip = sort_skip_mask(max_tokens, 0);  // no count exceeds the inputs' tokens
+    wc_status st = scratch_create(ctx, plan, false, stream, cs, max_tokens >= (1ull << 48));
     if (st != WC_OK) return st;
     wc_table *t = nullptr;
     st = table_create(ctx, cs.entries(), plan.caplong, plan.arena, ctx->count_bits, stream, &t);
     if (st != WC_OK) { ctx->release(cs.mem, cs.bytes, stream); return st; }
+    t->max_tokens = max_tokens;
     void *dsrc = nullptr;
     size_t sb = sizeof(MergeSrc) * std::max<uint32_t>(n, 1) + 8 * (n + 1);
     if ((st = ctx->alloc(&dsrc, sb, stream)) != WC_OK) {
@@ -798,9 +806,9 @@ wc_status wc_merge(wc_ctx *ctx, const wc_table *const *in, uint32_t n, cudaStrea
                                 n, chunks, g, stream);
     ctx->launches += chunks ? 1 : 0;
     ctx->prof_mark(ctx->ev_finish, stream);
-    if (e == cudaSuccess) e = finish_table(g, cs.gcap8, cs.gcap, cs.glcap, cs.ss, t->dt, stream);
+    if (e == cudaSuccess) e = finish_table(g, cs.gcap8, cs.gcap, cs.glcap, cs.ss, cs.bs, t->dt, stream, skip);
     ctx->prof_mark(ctx->ev_finish, stream);
-    ctx->launches += finish_table_launches(cs.ss);
+    ctx->launches += finish_table_launches(cs.ss, cs.bs, skip);
     ctx->release(dsrc, sb, stream);
     ctx->release(cs.mem, cs.bytes, stream);
     table_mark_done(t, stream);
@@ -893,6 +901,7 @@ wc_status wc_topk(wc_ctx *ctx, const wc_table *in, uint32_t k, cudaStream_t stre
     wc_status st = table_create(ctx, cap, std::max<uint64_t>(1, d.lcap), std::max<uint64_t>(16, d.arena_cap),
                                 d.count_bits, stream, &t);
     if (st != WC_OK) return st;
+    t->max_tokens = in->max_tokens;
     cudaStreamWaitEvent(stream, in->done, 0);
     cudaError_t e = launch_topk_copy(d, k, t->dt, stream);
     ctx->launches += 1;

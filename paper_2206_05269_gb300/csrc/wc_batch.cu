@@ -13,9 +13,15 @@
 //    global tables keyed by (document, word).
 // A whole document whose shared table fills up spills the rest of its words
 // (and, at the end, its shared table) to the same global tables.  Documents
-// counted there are finished by a segmented pass: compaction, a radix sort
-// with the document as most significant key, and a CSR write.
+// counted there are finished by a segmented pass: the bucket sort (wc_bucket.cuh) with the
+// document ordering first, straight into the CSR output; where the document and
+// count need more than 48 bits or the tables more than 2^24 slots, compaction, a
+// radix sort with the document as most significant key, and a CSR write.
 #include "wc_batch.h"
+
+#include <algorithm>
+
+#include "wc_bucket.cuh"
 
 namespace wc {
 
@@ -676,12 +682,12 @@ __global__ void k_bcompact16(const GSlot *slots, unsigned long long cap, SortScr
     }
 }
 
-// One lane per long slot, a warp's slots reserving entries, long indices
-// and arena bytes with one atomic each: document from the representative's
-// position, bytes copied (lowercased, 0-terminated) into the batch arena by
-// the slot's lane up to 64 bytes and by the whole warp beyond.
-__global__ void k_bcompact_long(const LSlot *ls, unsigned long long lcap, SortScratch ss, BatchArgs a,
-                                unsigned long long *meta) {
+// One lane per long slot, a warp's slots reserving long indices and arena
+// bytes with one atomic each; bytes copied (lowercased, 0-terminated) into the
+// batch arena by the slot's lane up to 64 bytes and by the whole warp beyond.
+// Then emit(slot, occupied, word, count, lref, rank, nocc) runs in every lane.
+template <class Emit>
+__device__ __forceinline__ void long_rows_body(const LSlot *ls, unsigned long long lcap, const BatchArgs &a, Emit &&emit) {
     const int lane = threadIdx.x & 31;
     const unsigned long long nw = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
     for (unsigned long long w0 = (((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; w0 < lcap;
@@ -705,16 +711,13 @@ __global__ void k_bcompact_long(const LSlot *ls, unsigned long long lcap, SortSc
             if (lane >= dd) incl += t;
         }
         const unsigned long long total = __shfl_sync(kFull, incl, 31);
-        unsigned long long boff = 0, blidx = 0, bpos = 0;
+        unsigned long long boff = 0, blidx = 0;
         if (lane == 0) {
             boff = atomicAdd(&a.meta[2], total);
             blidx = atomicAdd(&a.meta[1], nocc);
-            bpos = atomicAdd(&meta[0], nocc);
-            atomicAdd(&meta[1], nocc);  // long entries present: the sort orders shared prefixes by full bytes
         }
         const unsigned long long off = __shfl_sync(kFull, boff, 0) + incl - bytes;
         const unsigned long long lidx = __shfl_sync(kFull, blidx, 0) + rank;
-        const unsigned long long pos = __shfl_sync(kFull, bpos, 0) + rank;
         const bool fits = off + len + 1 <= a.arena_cap && lidx < a.lcap;
         const uint8_t *src = reinterpret_cast<const uint8_t *>(addr);
         if (occ && fits && len <= 64)
@@ -734,13 +737,28 @@ __global__ void k_bcompact_long(const LSlot *ls, unsigned long long lcap, SortSc
                 a.loff[lidx] = off;
                 a.llen[lidx] = len;
             }
-            ss.khi[pos] = be_bytes16(src, 0);
-            ss.klo[pos] = be_bytes16(src, 8);
-            ss.cnt[pos] = c;
-            ss.lref[pos] = fits ? (uint32_t)(lidx + 1) : 0u;
-            ss.doc[pos] = doc_of_pos(a.doc_off, a.ndocs, addr - reinterpret_cast<uintptr_t>(a.text));
         }
+        emit(w, occ, src, c, fits ? (uint32_t)(lidx + 1) : 0u, (uint32_t)rank, (uint32_t)nocc);
     }
+}
+__global__ void k_bcompact_long(const LSlot *ls, unsigned long long lcap, SortScratch ss, BatchArgs a,
+                                unsigned long long *meta) {
+    const int lane = threadIdx.x & 31;
+    long_rows_body(ls, lcap, a, [&](unsigned long long, bool occ, const uint8_t *src, unsigned long long c, uint32_t lref,
+                                    uint32_t rank, uint32_t nocc) {
+        unsigned long long pos = 0;
+        if (lane == 0) {
+            pos = atomicAdd(&meta[0], (unsigned long long)nocc);
+            atomicAdd(&meta[1], (unsigned long long)nocc);  // long entries present: the sort orders shared prefixes by full bytes
+        }
+        pos = __shfl_sync(kFull, pos, 0) + rank;
+        if (!occ) return;
+        ss.khi[pos] = be_bytes16(src, 0);
+        ss.klo[pos] = be_bytes16(src, 8);
+        ss.cnt[pos] = c;
+        ss.lref[pos] = lref;
+        ss.doc[pos] = doc_of_pos(a.doc_off, a.ndocs, (unsigned long long)(src - a.text));
+    });
 }
 
 __global__ void k_seg_base(BatchArgs a, unsigned long long *meta) {
@@ -823,13 +841,253 @@ static int gridn(unsigned long long n, int t, int maxb) {
     return (int)g;
 }
 
+// ---- by buckets
+struct SegJob {
+    GTable g;
+    unsigned long long cap8, cap16, lcap;
+    BucketScratch s;
+    BatchArgs a;
+    unsigned long long *meta;  // [0] entries, [1] long ones
+    int count_bits;
+    // the 48 bits that order first: document, then the count complemented
+    __device__ __forceinline__ unsigned long long first(uint32_t d, unsigned long long cnt) const {
+        const unsigned long long mask = (1ull << count_bits) - 1ull;
+        return ((unsigned long long)d << count_bits) | (mask - cnt);
+    }
+    __device__ __forceinline__ uint32_t doc(const Key128 &k) const { return (uint32_t)((k.hi >> 16) >> count_bits); }
+    __device__ __forceinline__ uint32_t cnt(const Key128 &k) const {
+        const unsigned long long mask = (1ull << count_bits) - 1ull;
+        return (uint32_t)(mask - ((k.hi >> 16) & mask));
+    }
+    __device__ __forceinline__ Key128 key8(unsigned long long k, unsigned long long c) const {
+        const unsigned long long w = restore_letters(k);
+        return bucket_key(first(gather_doc(k), c), be_half((uint32_t)w, (uint32_t)(w >> 32)), 0ull);
+    }
+    __device__ __forceinline__ Key128 key16(uint4 k, unsigned long long c) const {
+        const unsigned long long lo = ((unsigned long long)k.y << 32) | k.x, hi = ((unsigned long long)k.w << 32) | k.z;
+        const unsigned long long wl = restore_letters(lo), wh = restore_letters(hi);
+        return bucket_key(first(gather_doc(lo) | (gather_doc(hi) << 24), c), be_half((uint32_t)wl, (uint32_t)(wl >> 32)),
+                          be_half((uint32_t)wh, (uint32_t)(wh >> 32)));
+    }
+    __device__ __forceinline__ Key128 keylong(const uint8_t *src, unsigned long long c) const {
+        const uint32_t d = doc_of_pos(a.doc_off, a.ndocs, (unsigned long long)(src - a.text));
+        return bucket_key(first(d, c), be_bytes16(src, 0), be_bytes16(src, 8));
+    }
+};
+struct SegSource {
+    const SegJob &j;
+    __device__ __forceinline__ unsigned long long cap() const { return j.cap8 + j.cap16 + j.lcap; }
+    __device__ __forceinline__ bool get(unsigned long long i, Key128 &k, uint32_t &tie) const {
+        tie = 0u;
+        if (i < j.cap8) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(&j.g.slots8[i]);
+            if (v.x) k = j.key8(v.x, v.y);
+            return v.x != 0ull;
+        }
+        i -= j.cap8;
+        if (i < j.cap16) {
+            const uint4 w = j.g.slots[i].key;
+            if (!key_zero(w)) k = j.key16(w, j.g.slots[i].cnt);
+            return !key_zero(w);
+        }
+        i -= j.cap16;
+        const LSlot &l = j.g.lslots[i];
+        if (l.h == 0ull && l.addr == 0ull) return false;
+        k = j.keylong(reinterpret_cast<const uint8_t *>(l.addr), l.cnt);
+        tie = (uint32_t)i;
+        return true;
+    }
+};
+
+// (also: documents counted in the global tables start with no rows)
+__global__ void __launch_bounds__(kBktThreads) k_seg_sample(SegJob j) {
+    for (uint32_t d = blockIdx.x * kBktThreads + threadIdx.x; d < j.a.ndocs; d += gridDim.x * kBktThreads)
+        if (j.a.doc_flags[d]) {
+            j.a.doc_start[d] = ~0ull;
+            j.a.doc_n[d] = 0u;
+        }
+    grid_dependency_trigger();
+    bucket_sample(j.s, SegSource{j});
+}
+__global__ void __launch_bounds__(kRankThreads) k_seg_rank(SegJob j) {
+    extern __shared__ __align__(16) uint8_t bsm[];
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    bucket_rank(j.s, bsm, SegSource{j}.cap());
+}
+
+constexpr int kSegThreads = 512;
+__global__ void __launch_bounds__(kSegThreads, 2) k_seg_scatter(SegJob j) {
+    extern __shared__ __align__(16) uint8_t bsm[];
+    __shared__ uint32_t tot[2];
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    if (threadIdx.x < 2) tot[threadIdx.x] = 0u;
+    SlotQueue q = slot_queue(bsm);
+    const Splitters sp = load_splitters(j.s, bsm + slot_queue_smem(kSegThreads));
+    const unsigned long long step = (unsigned long long)gridDim.x * kSegThreads * kScanUnroll;
+    const unsigned long long b0 = (unsigned long long)blockIdx.x * kSegThreads * kScanUnroll;
+    uint32_t n = 0, nl = 0;
+    auto make = [&](const uint4 &k, unsigned long long c) -> Key128 {
+        n++;
+        return (k.z | k.w) ? j.key16(k, c) : j.key8(((unsigned long long)k.y << 32) | k.x, c);
+    };
+    for (unsigned long long b = b0; b < j.cap8; b += step) {  // block-uniform
+        ulonglong2 v[kScanUnroll];
+#pragma unroll
+        for (int u = 0; u < kScanUnroll; u++) {
+            const unsigned long long i = b + (unsigned long long)u * kSegThreads + threadIdx.x;
+            v[u] = i < j.cap8 ? *reinterpret_cast<const ulonglong2 *>(&j.g.slots8[i]) : make_ulonglong2(0ull, 0ull);
+        }
+#pragma unroll
+        for (int u = 0; u < kScanUnroll; u++)
+            q.push(j.s, sp, v[u].x != 0ull, make_uint4((uint32_t)v[u].x, (uint32_t)(v[u].x >> 32), 0u, 0u), v[u].y, make);
+    }
+    for (unsigned long long b = b0; b < j.cap16; b += step) {
+        uint4 k[kScanUnroll];
+        unsigned long long c[kScanUnroll];
+#pragma unroll
+        for (int u = 0; u < kScanUnroll; u++) {
+            const unsigned long long i = b + (unsigned long long)u * kSegThreads + threadIdx.x;
+            k[u] = make_uint4(0, 0, 0, 0);
+            c[u] = 0;
+            if (i < j.cap16) {
+                k[u] = j.g.slots[i].key;
+                c[u] = j.g.slots[i].cnt;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kScanUnroll; u++) q.push(j.s, sp, !key_zero(k[u]), k[u], c[u], make);
+    }
+    q.flush(j.s, sp, make);
+    long_rows_body(j.g.lslots, j.lcap, j.a, [&](unsigned long long slot, bool occ, const uint8_t *src, unsigned long long c,
+                                                uint32_t lref, uint32_t, uint32_t) {
+        if (!occ) return;
+        n++;
+        nl++;
+        bucket_put(j.s, sp, j.keylong(src, c), (uint32_t)slot, lref);
+    });
+    n = __reduce_add_sync(kFull, n);
+    nl = __reduce_add_sync(kFull, nl);
+    if ((threadIdx.x & 31) == 0 && n) {
+        atomicAdd(&tot[0], n);
+        atomicAdd(&tot[1], nl);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && tot[0]) {
+        atomicAdd(&j.meta[0], (unsigned long long)tot[0]);
+        if (tot[1]) atomicAdd(&j.meta[1], (unsigned long long)tot[1]);
+    }
+    bucket_close(j.s);
+}
+
+// The rows follow those of the documents counted in shared memory: a.meta[0] is
+// theirs until k_seg_close adds these.
+__global__ void __launch_bounds__(kBktSortThreads, kBktSortPerSm) k_seg_sort(SegJob j) {
+    extern __shared__ __align__(16) uint8_t bsm[];
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    const unsigned long long out0 = j.a.meta[0];
+    if (out0 + j.meta[0] > j.a.out_cap) return;
+    auto put = [&](unsigned long long row, const Key128 &k, uint32_t r) {
+        unsigned long long khi, klo;
+        key_prefix(k, khi, klo);
+        j.a.out_khi[row] = khi;
+        j.a.out_klo[row] = klo;
+        j.a.out_cnt[row] = j.cnt(k);
+        j.a.out_lref[row] = r;
+    };
+    bucket_sort(
+        j.s, *reinterpret_cast<BucketShared *>(bsm),
+        [&](unsigned long long base, uint32_t m, auto &&row) {
+            for (uint32_t i = threadIdx.x; i < m; i += kBktSortThreads) {
+                Key128 k, o;
+                uint32_t r, x;
+                row(i, k, r);
+                put(out0 + base + i, k, r);
+                // a document's rows in this bucket: [first, last]
+                const uint32_t d = j.doc(k);
+                if (i > 0) row(i - 1, o, x);
+                if (i == 0 || j.doc(o) != d) {
+                    atomicMin(&j.a.doc_start[d], out0 + base + i);
+                    atomicAdd(&j.a.doc_n[d], 0u - i);
+                }
+                if (i + 1 < m) row(i + 1, o, x);
+                if (i + 1 == m || j.doc(o) != d) atomicAdd(&j.a.doc_n[d], i + 1u);
+            }
+        },
+        [&](unsigned long long row, const Key128 &k, uint32_t r) {
+            put(out0 + row, k, r);
+            atomicMin(&j.a.doc_start[j.doc(k)], out0 + row);
+            atomicAdd(&j.a.doc_n[j.doc(k)], 1u);
+        });
+}
+
+// Adds the rows to the output's total, gives documents without a word their
+// empty range, and orders words of equal count and prefix by their remaining bytes (one
+// warp a document, only when the sort saw equal keys).
+__global__ void __launch_bounds__(256) k_seg_close(SegJob j) {
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    const BatchArgs &a = j.a;
+    const bool tied = j.s.state[kBktTied] != 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (a.meta[0] + j.meta[0] > a.out_cap) atomicOr(a.status, ST_OUT_FULL);
+        a.meta[0] += j.meta[0];
+    }
+    const int lane = threadIdx.x & 31;
+    const LongView v{a.out_lref, a.loff, a.llen, a.arena};
+    for (uint32_t d = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; d < a.ndocs; d += (gridDim.x * blockDim.x) >> 5) {
+        if (!a.doc_flags[d]) continue;
+        const uint32_t n = a.doc_n[d];
+        if (n == 0u) {
+            if (lane == 0) a.doc_start[d] = 0ull;
+            continue;
+        }
+        if (!tied) continue;
+        const unsigned long long s = a.doc_start[d];
+        uint32_t *lr = a.out_lref + s;
+        auto same = [&](uint32_t x, uint32_t y) {
+            return a.out_cnt[s + x] == a.out_cnt[s + y] && a.out_khi[s + x] == a.out_khi[s + y] &&
+                   a.out_klo[s + x] == a.out_klo[s + y];
+        };
+        for (uint32_t i = 1u + lane; i < n; i += 32) {  // the last row of a run sorts it
+            if ((i + 1 < n && same(i, i + 1)) || !same(i - 1, i)) continue;
+            uint32_t lo = i - 1;
+            while (lo > 0 && same(lo - 1, i)) lo--;
+            for (uint32_t p = lo + 1; p <= i; p++) {
+                const uint32_t x = lr[p];
+                uint32_t q = p;
+                while (q > lo && lref_less(v, x, lr[q - 1])) { lr[q] = lr[q - 1]; q--; }
+                lr[q] = x;
+            }
+        }
+    }
+}
+
+static cudaError_t finish_seg_by_buckets(const SegJob &j, int sms, cudaStream_t s) {
+    const size_t smem = splitters_smem(j.s);
+    cudaError_t e = ensure_smem_limit((const void *)k_seg_rank, (int)kept_smem(kBktGroups));
+    if (e == cudaSuccess) e = ensure_smem_limit((const void *)k_seg_scatter, (int)(kSplittersMax + slot_queue_smem(kSegThreads)));
+    if (e == cudaSuccess) e = ensure_smem_limit((const void *)k_seg_sort, (int)sizeof(BucketShared));
+    if (e != cudaSuccess) return e;
+    k_seg_sample<<<j.s.groups, kBktThreads, 0, s>>>(j);
+    launch_dependent(k_seg_rank, dim3(j.s.groups), dim3(kRankThreads), kept_smem(j.s.groups), s, j);
+    launch_dependent(k_seg_scatter, dim3(gridn(j.cap8 + j.cap16 + j.lcap, kSegThreads * kScanUnroll, sms * 2)),
+                     dim3(kSegThreads), smem + slot_queue_smem(kSegThreads), s, j);
+    launch_dependent(k_seg_sort, dim3(j.s.buckets()), dim3(kBktSortThreads), sizeof(BucketShared), s, j);
+    launch_dependent(k_seg_close, dim3(gridn((unsigned long long)j.a.ndocs * 32, 256, sms * 4)), dim3(256), 0, s, j);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_segmented_finish(const BatchArgs &a, const GTable &g, uint64_t cap8, uint64_t cap16,
-                                    uint64_t caplong, SortScratch &ss, unsigned long long *smeta, cudaStream_t s,
-                                    uint32_t skip) {
+                                    uint64_t caplong, SortScratch &ss, const BucketScratch &bs, int count_bits,
+                                    unsigned long long *smeta, cudaStream_t s, uint32_t skip) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaMemsetAsync(smeta, 0, 16 * 8, s);
+    if (bs.key) return finish_seg_by_buckets(SegJob{g, cap8, cap16, caplong, bs, a, smeta, count_bits}, sms, s);
     sort_state_reset(ss, s);
     k_bcompact8<<<gridn(cap8, 256 * kScanUnroll, sms * 8), 256, 0, s>>>(g.slots8, cap8, ss, smeta);
     k_bcompact16<<<gridn(cap16, 256 * kScanUnroll, sms * 8), 256, 0, s>>>(g.slots, cap16, ss, smeta);
@@ -842,8 +1100,8 @@ cudaError_t launch_segmented_finish(const BatchArgs &a, const GTable &g, uint64_
     k_seg_ends<<<gridn(ss.cap, 256 * kScanUnroll, sms * 8), 256, 0, s>>>(ss, a, smeta, kSortPassesSeg);
     return cudaGetLastError();
 }
-int segmented_finish_launches(uint64_t cap, uint32_t skip) {
-    return 4 + sort_entries_launches(kSortPassesSeg, cap, skip) + 3;
+int segmented_finish_launches(const SortScratch &ss, const BucketScratch &bs, uint32_t skip) {
+    return bs.key ? 5 : 4 + sort_entries_launches(kSortPassesSeg, ss.cap, skip) + 3;
 }
 
 }  // namespace wc

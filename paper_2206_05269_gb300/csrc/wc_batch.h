@@ -45,9 +45,12 @@ extern const int kNumDocShapes;
 // class's kernel in the stream (independent work; it waits for that kernel
 // only at its end).
 cudaError_t launch_docs(const BatchArgs &a, int shape, cudaStream_t s, bool dependent = false);
+// The (document, word) tables' rows sorted into the output.  By the bucket sort when
+// `bs` is carved (count_bits: bits of the largest count, with the documents' bits at most 48), else
+// by the radix sort of `ss`.
 cudaError_t launch_segmented_finish(const BatchArgs &a, const GTable &g, uint64_t cap8, uint64_t cap16,
-                                    uint64_t caplong, SortScratch &ss, unsigned long long *smeta, cudaStream_t s,
-                                    uint32_t skip = 0);
-int segmented_finish_launches(uint64_t cap, uint32_t skip = 0);
+                                    uint64_t caplong, SortScratch &ss, const BucketScratch &bs, int count_bits,
+                                    unsigned long long *smeta, cudaStream_t s, uint32_t skip = 0);
+int segmented_finish_launches(const SortScratch &ss, const BucketScratch &bs, uint32_t skip = 0);
 
 }  // namespace wc

@@ -8,6 +8,7 @@
 
 #include "../../include/wc.h"
 #include "wc_batch.h"
+#include "wc_bucket.cuh"
 #include "wc_host.h"
 
 using namespace wc;
@@ -72,6 +73,12 @@ struct wc_batch {
     bool tables_built = false;
     bool exact = false;  // capacities at the exact bounds
     uint64_t max_doc_bytes = 0, total_bytes = 0;  // bounds on counts: no count exceeds half of these
+    int count_bits() const {  // bits of the largest count of a document
+        return 64 - __builtin_clzll(max_doc_bytes / 2 + 1);
+    }
+    bool seg_radix() const {  // (document, count) keys past the bucket sort's 48 bits
+        return count_bits() + (ndocs > 1 ? 64 - __builtin_clzll((uint64_t)ndocs - 1) : 0) > 48;
+    }
     std::vector<wc_table *> class_tables;
     wc_table *global = nullptr;
     CountScratch gscratch;        // global hash tables kept for ratio lookups
@@ -275,7 +282,7 @@ static wc_status batch_alloc(wc_batch *b, cudaStream_t stream) {
     a.ndocs = b->ndocs;
     // scratch: items + queue cursors, (document, word) tables, sort scratch
     CapPlan plan{b->cap8, b->cap16, b->caplong, 0};
-    st = scratch_create(ctx, plan, false, stream, b->scr.cs);
+    st = scratch_create(ctx, plan, false, stream, b->scr.cs, b->seg_radix());
     b->scr.ibytes = sizeof(DocItem) * std::max<size_t>(b->items.size(), 1) + 256 + 16 * 8;
     void *ib = nullptr;
     if (st == WC_OK) st = ctx->alloc(&ib, b->scr.ibytes, stream);
@@ -348,8 +355,9 @@ static cudaError_t batch_enqueue(wc_batch *b, const uint8_t *d_text, const uint6
     }
     if (e == cudaSuccess) {
         const uint32_t skip = sort_skip_mask(b->max_doc_bytes / 2 + 1, b->ndocs);
-        e = launch_segmented_finish(a, a.g, cs.gcap8, cs.gcap, cs.glcap, cs.ss, b->scr.smeta, stream, skip);
-        n += segmented_finish_launches(cs.ss.cap, skip);
+        e = launch_segmented_finish(a, a.g, cs.gcap8, cs.gcap, cs.glcap, cs.ss, cs.bs, b->count_bits(), b->scr.smeta,
+                                    stream, skip);
+        n += segmented_finish_launches(cs.ss, cs.bs, skip);
     }
     if (launches) *launches = n;
     return e;
@@ -631,6 +639,7 @@ static wc_status build_tables_at(wc_batch *b, const std::vector<uint64_t> &est, 
                                s, &tabs[c])) != WC_OK)
             break;
         tabs[c]->owner = b;
+        tabs[c]->max_tokens = b->total_bytes / 2 + b->ndocs + 1;
     }
     if (st != WC_OK) {
         cleanup(nt);
@@ -657,13 +666,11 @@ static wc_status build_tables_at(wc_batch *b, const std::vector<uint64_t> &est, 
     std::vector<FinishSpec> spec(nt);
     for (uint32_t c = 0; c < nt; c++) {
         CountScratch &cs = c < b->nclasses ? scr[c] : b->gscratch;
-        spec[c] = FinishSpec{c < b->nclasses ? g[c] : gg, cs.gcap8, cs.gcap, cs.glcap, &cs.ss, &tabs[c]->dt};
+        spec[c] = FinishSpec{c < b->nclasses ? g[c] : gg, cs.gcap8, cs.gcap, cs.glcap, &cs.ss, &cs.bs, &tabs[c]->dt};
     }
     const uint32_t skip = sort_skip_mask(b->total_bytes / 2 + 1, 0);
     if (e == cudaSuccess) e = finish_tables(spec.data(), (int)nt, static_cast<uint8_t *>(dg) + gbytes, s, skip);
-    uint64_t capmax = 0;
-    for (uint32_t c = 0; c < nt; c++) capmax = std::max<uint64_t>(capmax, spec[c].ss->cap);
-    ctx->launches += 1 + (uint64_t)finish_tables_launches((int)nt, capmax, skip);
+    ctx->launches += 1 + (uint64_t)finish_tables_launches(spec.data(), (int)nt, skip);
     cleanup(nt);
     ctx->release(dg, dbytes, s);
     for (auto *t : tabs) table_mark_done(t, s);
@@ -1220,8 +1227,8 @@ __device__ __forceinline__ uint4 entry_key(unsigned long long hi8, unsigned long
     return k;
 }
 
-// Sort input: the global table's entries with every count zero, so that the
-// stable (count desc, word asc) sort orders them by word alone.
+// The global table's entries with every count taken as zero, so that the
+// (count desc, word asc) sorts order them by word alone: as the radix sort's input...
 __global__ void k_vocab_prep(DevTable G, SortScratch ss, unsigned long long *meta) {
     const unsigned long long n = G.d_meta[0];
     if (blockIdx.x == 0 && threadIdx.x == 0) meta[0] = n;
@@ -1233,13 +1240,102 @@ __global__ void k_vocab_prep(DevTable G, SortScratch ss, unsigned long long *met
         ss.lref[i] = G.lref[i];
     }
 }
+// ...and as the bucket sort's; perm[i] = the row of G with the i-th word.
+struct VocabJob {
+    DevTable G;
+    unsigned long long n;
+    BucketScratch s;
+    uint32_t *perm;
+};
+struct VocabSource {
+    const VocabJob &j;
+    __device__ __forceinline__ unsigned long long cap() const { return j.n; }
+    __device__ __forceinline__ bool get(unsigned long long i, Key128 &k, uint32_t &tie) const {
+        k = bucket_key(0ull, j.G.khi[i], j.G.klo[i]);
+        tie = (uint32_t)i;
+        return true;
+    }
+};
+__global__ void __launch_bounds__(kBktThreads) k_vocab_sample(VocabJob j) {
+    grid_dependency_trigger();
+    bucket_sample(j.s, VocabSource{j});
+}
+__global__ void __launch_bounds__(kRankThreads) k_vocab_rank(VocabJob j) {
+    extern __shared__ __align__(16) uint8_t bsm[];
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    bucket_rank(j.s, bsm, j.n);
+}
+__global__ void __launch_bounds__(kBktThreads) k_vocab_scatter(VocabJob j) {
+    extern __shared__ __align__(16) uint8_t bsm[];
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    const Splitters sp = load_splitters(j.s, bsm);
+    for (unsigned long long i = (unsigned long long)blockIdx.x * kBktThreads + threadIdx.x; i < j.n;
+         i += (unsigned long long)gridDim.x * kBktThreads)
+        bucket_put(j.s, sp, bucket_key(0ull, j.G.khi[i], j.G.klo[i]), (uint32_t)i, (uint32_t)i);
+    bucket_close(j.s);
+}
+__global__ void __launch_bounds__(kBktSortThreads, kBktSortPerSm) k_vocab_sort(VocabJob j) {
+    extern __shared__ __align__(16) uint8_t bsm[];
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    bucket_sort(
+        j.s, *reinterpret_cast<BucketShared *>(bsm),
+        [&](unsigned long long base, uint32_t m, auto &&row) {
+            for (uint32_t i = threadIdx.x; i < m; i += kBktSortThreads) {
+                Key128 k;
+                uint32_t r;
+                row(i, k, r);
+                j.perm[base + i] = r;
+            }
+        },
+        [&](unsigned long long row, const Key128 &, uint32_t r) { j.perm[row] = r; });
+}
+// Words of one prefix (17+ letters, and at most one of 16) ordered by their remaining bytes.
+__global__ void k_vocab_fix(VocabJob j) {
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    if (!j.s.state[kBktTied]) return;
+    const LongView v{j.G.lref, j.G.loff, j.G.llen, j.G.arena};
+    uint32_t *perm = j.perm;
+    auto same = [&](unsigned long long a, unsigned long long b) {
+        return j.G.khi[perm[a]] == j.G.khi[perm[b]] && j.G.klo[perm[a]] == j.G.klo[perm[b]];
+    };
+    for (unsigned long long i = 1ull + (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < j.n;
+         i += (unsigned long long)gridDim.x * blockDim.x) {
+        if ((i + 1 < j.n && same(i, i + 1)) || !same(i - 1, i)) continue;  // the last of a run sorts it
+        unsigned long long lo = i - 1;
+        while (lo > 0 && same(lo - 1, i)) lo--;
+        for (unsigned long long a = lo + 1; a <= i; a++) {
+            const uint32_t x = perm[a];
+            unsigned long long b = a;
+            while (b > lo && lref_less(v, j.G.lref[x], j.G.lref[perm[b - 1]])) { perm[b] = perm[b - 1]; b--; }
+            perm[b] = x;
+        }
+    }
+}
+static cudaError_t launch_vocab_sort(const VocabJob &j, int sms, cudaStream_t s) {
+    const size_t smem = splitters_smem(j.s);
+    cudaError_t e = ensure_smem_limit((const void *)k_vocab_rank, (int)kept_smem(kBktGroups));
+    if (e == cudaSuccess) e = ensure_smem_limit((const void *)k_vocab_scatter, (int)kSplittersMax);
+    if (e == cudaSuccess) e = ensure_smem_limit((const void *)k_vocab_sort, (int)sizeof(BucketShared));
+    if (e != cudaSuccess) return e;
+    const int grid = (int)std::max<uint64_t>(1, std::min<uint64_t>((j.n + kBktThreads - 1) / kBktThreads, 4ull * sms));
+    k_vocab_sample<<<j.s.groups, kBktThreads, 0, s>>>(j);
+    launch_dependent(k_vocab_rank, dim3(j.s.groups), dim3(kRankThreads), kept_smem(j.s.groups), s, j);
+    launch_dependent(k_vocab_scatter, dim3(grid), dim3(kBktThreads), smem, s, j);
+    launch_dependent(k_vocab_sort, dim3(j.s.buckets()), dim3(kBktSortThreads), sizeof(BucketShared), s, j);
+    launch_dependent(k_vocab_fix, dim3(grid), dim3(256), 0, s, j);
+    return cudaGetLastError();
+}
 
 // Row i of the vocabulary = the i-th word in word order (with its global
 // count and the global table's long-word bytes); the id table maps each
-// word to i + 1.
-__global__ void k_vocab_place(DevTable G, SortScratch ss, DevTable V, GTable vg) {
+// word to i + 1.  perm: the order, or null for the radix sort's.
+__global__ void k_vocab_place(DevTable G, SortScratch ss, const uint32_t *perm, DevTable V, GTable vg) {
     const unsigned long long n = G.d_meta[0];
-    const uint32_t *perm = ss.perm_buf(ss.cur[kCurFinal]);
+    if (!perm) perm = ss.perm_buf(ss.cur[kCurFinal]);
     if (blockIdx.x == 0 && threadIdx.x < 8) V.d_meta[threadIdx.x] = G.d_meta[threadIdx.x];
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (unsigned long long)gridDim.x * blockDim.x) {
@@ -1304,30 +1400,41 @@ static wc_status build_vocab(wc_batch *b) {
         ctx->release(cs.mem, cs.bytes, s);
         return st;
     }
+    // radix sort metadata, or the bucket sort's order
     void *dmeta = nullptr;
-    if ((st = ctx->alloc(&dmeta, 64, s)) != WC_OK) {
+    const size_t mb = cs.bs.key ? 4 * std::max<uint64_t>(1, n) : 64;
+    if ((st = ctx->alloc(&dmeta, mb, s)) != WC_OK) {
         ctx->release(ids, ib, s);
         free_owned_table(V);
         ctx->release(cs.mem, cs.bytes, s);
         return st;
     }
-    unsigned long long *smeta = static_cast<unsigned long long *>(dmeta);
-    cudaMemsetAsync(smeta, 0, 64, s);
     const GTable vg = cs.gtable(V->dt.d_status);
     const int grid = std::max(1, std::min(ctx->sms * 8, (int)((std::max<uint64_t>(n, b->entries) + 255) / 256)));
     cudaStreamWaitEvent(s, G->done, 0);
-    sort_state_reset(cs.ss, s);
-    k_vocab_prep<<<grid, 256, 0, s>>>(G->dt, cs.ss, smeta);
-    const LongView lv{G->dt.lref, G->dt.loff, G->dt.llen, G->dt.arena};
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = sort_entries(cs.ss, smeta, lv, kSortPasses, s, sort_skip_mask(0, 0));
+    cudaError_t e = cudaSuccess;
+    const uint32_t *perm = nullptr;
+    if (cs.bs.key) {
+        perm = static_cast<uint32_t *>(dmeta);
+        if (n) e = launch_vocab_sort(VocabJob{G->dt, n, cs.bs, static_cast<uint32_t *>(dmeta)}, ctx->sms, s);
+        ctx->launches += 5;
+    } else {
+        unsigned long long *smeta = static_cast<unsigned long long *>(dmeta);
+        cudaMemsetAsync(smeta, 0, 64, s);
+        sort_state_reset(cs.ss, s);
+        k_vocab_prep<<<grid, 256, 0, s>>>(G->dt, cs.ss, smeta);
+        const LongView lv{G->dt.lref, G->dt.loff, G->dt.llen, G->dt.arena};
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = sort_entries(cs.ss, smeta, lv, kSortPasses, s, sort_skip_mask(0, 0));
+        ctx->launches += 2 + (uint64_t)sort_entries_launches(kSortPasses, cs.ss.cap, sort_skip_mask(0, 0));
+    }
     if (e == cudaSuccess) {
-        k_vocab_place<<<grid, 256, 0, s>>>(G->dt, cs.ss, V->dt, vg);
+        k_vocab_place<<<grid, 256, 0, s>>>(G->dt, cs.ss, perm, V->dt, vg);
         k_vocab_ids<<<grid, 256, 0, s>>>(b->args, vg, static_cast<uint32_t *>(ids), b->entries);
         e = cudaGetLastError();
+        ctx->launches += 2;
     }
-    ctx->launches += 4 + (uint64_t)sort_entries_launches(kSortPasses, cs.ss.cap, sort_skip_mask(0, 0));
-    ctx->release(dmeta, 64, s);
+    ctx->release(dmeta, mb, s);
     ctx->release(cs.mem, cs.bytes, s);
     table_mark_done(V, s);
     if (e != cudaSuccess) {

@@ -91,25 +91,21 @@ __device__ __forceinline__ uint4 load_key16(const uint8_t *win, uint32_t p, uint
 
 // 8 big-endian key bytes (0, or a letter) -> 8 five-bit codes (0 for
 // padding, 1..26 for a..z), the first byte in the highest code (40 bits):
-// integer order on codes is byte order on lowercase words.
+// integer order on codes is byte order on lowercase words.  A letter's code is
+// its low five bits; neighbouring codes are joined 8 -> 16 -> 32 -> 64 bits.
 __device__ __forceinline__ unsigned long long pack5(unsigned long long be) {
-    unsigned long long r = 0;
-#pragma unroll
-    for (int i = 0; i < 8; i++) {
-        const uint32_t b = (uint32_t)(be >> (56 - 8 * i)) & 0xFFu;
-        r = (r << 5) | (b ? ((b | 0x20u) - 0x60u) & 31u : 0u);
-    }
-    return r;
+    unsigned long long r = be & 0x1F1F1F1F1F1F1F1Full;
+    r = (r & 0x001F001F001F001Full) | ((r >> 3) & 0x03E003E003E003E0ull);
+    r = (r & 0x000003FF000003FFull) | ((r >> 6) & 0x000FFC00000FFC00ull);
+    return (r & 0xFFFFFull) | ((r >> 12) & 0xFFFFF00000ull);
 }
 // The inverse of pack5: 40 bits of codes -> 8 big-endian lowercase bytes.
 __device__ __forceinline__ unsigned long long unpack5(unsigned long long c) {
-    unsigned long long r = 0;
-#pragma unroll
-    for (int i = 0; i < 8; i++) {
-        const uint32_t v = (uint32_t)(c >> (35 - 5 * i)) & 31u;
-        r = (r << 8) | (v ? v + 0x60u : 0u);
-    }
-    return r;
+    unsigned long long r = (c & 0xFFFFFull) | ((c & 0xFFFFF00000ull) << 12);
+    r = (r & 0x000003FF000003FFull) | ((r & 0x000FFC00000FFC00ull) << 6);
+    r = (r & 0x001F001F001F001Full) | ((r & 0x03E003E003E003E0ull) << 3);
+    const unsigned long long nz = (r + 0x7F7F7F7F7F7F7F7Full) & 0x8080808080808080ull;  // 0x80 where the code is not 0
+    return r | (nz >> 1) | (nz >> 2);
 }
 
 __device__ __forceinline__ bool key_eq(uint4 a, uint4 b) {

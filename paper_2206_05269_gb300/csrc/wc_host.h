@@ -67,6 +67,7 @@ struct wc_table {
     wc_status sync_status = WC_OK;
     uint64_t n = 0, nlong = 0, tokens = 0, word_bytes = 0;
     uint32_t status_bits = 0;
+    uint64_t max_tokens = UINT64_MAX;  // no count of this table, nor their sum, exceeds it
     uint64_t src_bytes = 0;  // input size of a single-document count (capacity hints)
     int meta_slot = -1;      // pinned slot of wc_ctx::meta_host, or -1
 };
@@ -80,7 +81,8 @@ struct CountScratch {
     wc::GSlot *slots = nullptr;
     wc::LSlot *lslots = nullptr;
     void *head = nullptr;
-    wc::SortScratch ss{};
+    wc::SortScratch ss{};    // radix sort (carved only when the bucket sort's scratch is not)
+    wc::BucketScratch bs{};
     wc::GTable gtable(uint32_t *status) const {
         return wc::GTable{slots, gcap - 1, lslots, glcap - 1, status, slots8, gcap8 - 1};
     }
@@ -97,4 +99,5 @@ wc_status table_create(wc_ctx *ctx, uint64_t cap, uint64_t lcap, uint64_t arena,
 void table_mark_done(wc_table *t, cudaStream_t s);
 wc_status table_sync(const wc_table *t);
 CapPlan plan_capacity(const wc_ctx *ctx, uint64_t nbytes, const wc_count_opts *o);
-wc_status scratch_create(wc_ctx *ctx, const CapPlan &p, bool head, cudaStream_t s, CountScratch &cs);
+// radix: sort scratch for the radix sort even where the bucket sort would serve.
+wc_status scratch_create(wc_ctx *ctx, const CapPlan &p, bool head, cudaStream_t s, CountScratch &cs, bool radix = false);

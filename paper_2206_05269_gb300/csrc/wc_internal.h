@@ -138,10 +138,6 @@ struct SortScratch {
     uint32_t group_stride;
     uint32_t *look[2];       // 256 x ntiles each: per-tile digit counts published for the look-back, by pass parity
     uint32_t *tile_ctr;      // [2]: tiles taken in launch order, by pass parity
-    // merge sort of a single table (null when the scratch was carved without
-    // it): 128-bit keys, the high and low words of buffer 0, then of buffer 1
-    // (the indices travel in perm[0] and perm[1])
-    unsigned long long *mk[4];
     // permutation buffer c (0 or 1), selected without indexing the parameter array
     __device__ __forceinline__ uint32_t *perm_buf(uint32_t c) const { return c ? perm[1] : perm[0]; }
     __device__ __forceinline__ uint32_t *group_buf(uint32_t c) const { return c ? group_hist[1] : group_hist[0]; }
@@ -150,10 +146,8 @@ struct SortScratch {
 // Slot of SortScratch::cur where a radix pass records a look-back that gave
 // up waiting (the finish then reports WC_ERR_TIMEOUT).
 constexpr int kCurSortError = 30;
-// with_msort: also the merge sort's key buffers (32 bytes an entry), which a
-// single table's finish then uses (see finish_table).
-size_t sort_scratch_bytes(uint64_t cap, bool with_msort = false);
-void sort_scratch_carve(SortScratch &s, void *base, uint64_t cap, bool with_msort = false);
+size_t sort_scratch_bytes(uint64_t cap);
+void sort_scratch_carve(SortScratch &s, void *base, uint64_t cap);
 // Zeroes what a sort accumulates into (digit histograms, pass cursors, group
 // counts, the first pass's look-back buffer and the tile counters): every
 // sort of a scratch starts with this (stream-ordered memsets).
@@ -179,14 +173,49 @@ cudaError_t sort_entries(SortScratch &ss, const unsigned long long *meta, const 
                          cudaStream_t st, uint32_t skip = 0);
 int sort_entries_launches(int passes, uint64_t cap, uint32_t skip = 0);
 
-// Compacts the global hash tables into unsorted scratch arrays and copies
-// the long words into out.arena; then sorts and writes `out`.  The sort is a
-// merge sort when ss has its key buffers and `skip` shows every count below
-// 2^32 (the radix sort's count digits 4..7 skipped), else the radix sort.
-// finish_table_launches(ss, skip) kernels are launched.
-int finish_table_launches(const SortScratch &ss, uint32_t skip = 0);
+// Scratch of the bucket sort (wc_bucket.cuh) of up to `cap` entries: about 84
+// bytes an entry.
+constexpr int kBktGroups = 128;  // sample blocks at most
+constexpr int kBktKeep = 64;     // sampled keys a sample block keeps at most
+constexpr int kBktApart = 3;     // sampled keys between two splitters at least
+constexpr int kBktMean = 384;    // entries a bucket is meant to hold
+constexpr int kBktStride = 8;    // words between two buckets' counters
+constexpr int kBktSplits = 0, kBktRoom = 1, kBktSpilled = 2, kBktTied = 3, kBktBig = 4, kBktTicket = 5;  // BucketScratch::state
+// Tables of more slots are radix sorted: there are at most 2,730 splitters (54 KB
+// of shared memory in the scatter kernels), and 8M entries would put 3,000 in a
+// bucket; from 2,560 on a block sorts in global memory.
+constexpr uint64_t kBktMaxCap = 1ull << 24;
+struct BucketScratch {
+    uint32_t groups;              // sample blocks
+    unsigned long long slots;     // entries `key` and `lref` hold, shared out evenly to the buckets
+    ulonglong2 *kept, *split;     // sampled keys, splitters in order (high and low halves)
+    uint32_t *kept_tie, *split_tie;
+    uint2 *found;                 // per sample block: entries found, keys kept
+    uint32_t rank_blocks;         // blocks of the rank kernel
+    uint32_t tree;                // words of the scatter kernels' search tree: a power of two above splits()
+    uint32_t *count;              // entries a bucket got, kBktStride words apart
+    uint32_t *first;              // a bucket's first row
+    uint32_t *state;
+    ulonglong2 *key;              // null: no bucket scratch
+    uint32_t *lref;
+    ulonglong2 *spill_key;        // entries past their bucket's room
+    uint32_t *spill_lref, *spill_bucket;
+    ulonglong2 *big_key;          // buckets too large for shared memory are sorted here
+    uint32_t *big_lref;
+    __host__ __device__ __forceinline__ uint32_t splits() const { return groups * kBktKeep / kBktApart; }
+    __host__ __device__ __forceinline__ uint32_t buckets() const { return splits() + 1; }
+};
+size_t bucket_scratch_bytes(uint64_t cap);
+void bucket_scratch_carve(BucketScratch &s, void *base, uint64_t cap);
+
+// Turns the global hash tables into the sorted table `out` (long words copied
+// into out.arena): by the bucket sort when `bs` is carved and `skip` shows every
+// count below 2^48 (the count's two high digits skipped), else compaction
+// into `ss` and the radix sort.  finish_table_launches(...) kernels are launched.
+bool finish_by_buckets(const BucketScratch &bs, uint32_t skip);
+int finish_table_launches(const SortScratch &ss, const BucketScratch &bs, uint32_t skip = 0);
 cudaError_t finish_table(const GTable &g, uint64_t gcap8, uint64_t gcap, uint64_t glcap, SortScratch &ss,
-                         DevTable &out, cudaStream_t s, uint32_t skip = 0);
+                         const BucketScratch &bs, DevTable &out, cudaStream_t s, uint32_t skip = 0);
 
 // Compaction scans read kScanUnroll slots a thread per step (independent
 // loads in flight) and reserve output positions with one atomic per block
@@ -234,25 +263,26 @@ __device__ __forceinline__ unsigned long long block_take(BlockTake &sh, uint32_t
     return pos;
 }
 
-// One table's sort arguments (device copies of them for finish_tables).
+// One radix sort's arguments.
 struct SortJob {
     SortScratch s;
     const unsigned long long *meta;
     LongView v;
     DevTable out;
 };
-// finish_table for n tables at once: each table's compaction, then every
-// sort pass and the final gather as one launch over all n tables (grid.y).
-// d_jobs: device memory of finish_tables_job_bytes(n), alive until the
-// stream has run the launches.  finish_tables_launches(n, largest cap) kernels.
+// finish_table for n tables at once by the bucket sort: every step as one launch over all
+// n tables (grid.y).  d_jobs: device memory of finish_tables_job_bytes(n), alive
+// until the stream has run the launches.  Tables without bucket scratch are
+// finished one by one.
 struct FinishSpec {
     GTable g;
     uint64_t gcap8, gcap, glcap;
     SortScratch *ss;
+    BucketScratch *bs;
     DevTable *out;
 };
 size_t finish_tables_job_bytes(int n);
-int finish_tables_launches(int n, uint64_t cap, uint32_t skip = 0);
+int finish_tables_launches(const FinishSpec *spec, int n, uint32_t skip = 0);
 cudaError_t finish_tables(const FinishSpec *spec, int n, void *d_jobs, cudaStream_t s, uint32_t skip = 0);
 
 // Entries of finished tables re-inserted into a global hash table (merge).

@@ -2,23 +2,22 @@
 //
 // After the counting kernel the global hash tables hold each distinct word
 // once with its exact count (Sec. 3.3's reduced dictionary).  This file turns
-// them into the sorted output: compact the occupied slots, copy long words
-// into the table's own byte arena, then sort.  A single table whose counts
-// are below 2^32 is merge-sorted by one 128-bit key per entry (the
-// complemented count, then the 16-letter prefix packed 5 bits a letter: 0 for
-// padding, 1..26 for a..z, so integer order is lexicographic order and a
-// proper prefix sorts first).  Other sorts (batched, merged and allocation-
-// free tables) are an LSD radix sort over a permutation: 10 byte-digits of
-// the packed prefix and up to 8 digits of the complemented count (count
-// descending).  Either is followed by a fix-up that orders long words sharing
-// count and 16-letter prefix by their remaining bytes; every radix pass is
-// stable, so the final order is (count desc, word asc).  Digits that are equal for every
-// element are skipped, detected on the device from one histogram pass; those
-// the host's bounds already show constant (count bytes above the token bound,
-// document bytes above the document count) are not launched at all.
+// them into the sorted output.  A table of at most kBktMaxCap slots whose counts
+// are below 2^48 goes through the bucket sort of wc_bucket.cuh, straight from the
+// hash tables.  Other tables (and the allocation-free entry point, whose fixed
+// scratch has no room for it) are compacted and then sorted by an LSD radix sort over a
+// permutation: 10 byte-digits of the packed prefix and up to 8 digits of the
+// complemented count (count descending).  Either is followed by a fix-up that
+// orders long words sharing count and 16-letter prefix by their remaining
+// bytes, so the final order is (count desc, word asc).  Radix digits that are
+// equal for every element are skipped, detected on the device from one
+// histogram pass; those the host's bounds already show constant (count bytes
+// above the token bound, document bytes above the document count) are not
+// launched at all.
 #include <algorithm>
 #include <vector>
 
+#include "wc_bucket.cuh"
 #include "wc_internal.h"
 
 namespace wc {
@@ -38,14 +37,14 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
     return m;
 }
 
-size_t sort_scratch_bytes(uint64_t cap, bool with_msort) {
+size_t sort_scratch_bytes(uint64_t cap) {
     uint64_t ntiles = (cap + kSortTile - 1) / kSortTile;
     return cap * (8 + 8 + 8 + 8 + 4 + 4 + 4 + 4 + 4) + 4 * kPassesSeg * 256 + 4 * 256 * ntiles + 4 * 32 +
            2 * 4 * 256 * (ntiles <= kSortFusedMaxTiles ? sort_group_stride(ntiles) : 1) + 4096 +
-           2 * (4 * 256 * ntiles + 256) + 256 + (with_msort ? 4 * (cap * 8 + 256) : 0);
+           2 * (4 * 256 * ntiles + 256) + 256;
 }
 
-void sort_scratch_carve(SortScratch &s, void *base, uint64_t cap, bool with_msort) {
+void sort_scratch_carve(SortScratch &s, void *base, uint64_t cap) {
     uint64_t ntiles = (cap + kSortTile - 1) / kSortTile;
     uint8_t *p = static_cast<uint8_t *>(base);
     auto take = [&](size_t n) { uint8_t *r = p; p += (n + 255) & ~(size_t)255; return r; };
@@ -68,8 +67,6 @@ void sort_scratch_carve(SortScratch &s, void *base, uint64_t cap, bool with_msor
     s.look[0] = reinterpret_cast<uint32_t *>(take(4 * 256 * ntiles));
     s.look[1] = reinterpret_cast<uint32_t *>(take(4 * 256 * ntiles));
     s.tile_ctr = reinterpret_cast<uint32_t *>(take(4 * 2));
-    for (int i = 0; i < 4; i++)
-        s.mk[i] = with_msort ? reinterpret_cast<unsigned long long *>(take(cap * 8)) : nullptr;
 }
 
 // ---------------------------------------------------------------- compaction
@@ -94,39 +91,20 @@ __device__ __forceinline__ void sort_key_prep(const SortScratch &s, unsigned lon
     atomicAdd(&h[9 * 256 + ((hi >> 8) & 0xFF)], 1u);
 }
 
-// The merge sort's 128-bit key of an entry (counts below 2^32): the count
-// inverted in the high 32 bits (count descending), then the 80-bit packed
-// prefix, then 16 zero bits.  A count of at least 1 keeps the high word below
-// all ones, the key of the sort's padding.
-__device__ __forceinline__ void ms_key_prep(const SortScratch &s, unsigned long long i, unsigned long long khi,
-                                            unsigned long long klo, unsigned long long cnt) {
-    const unsigned long long ph = pack5(khi), pl = pack5(klo);
-    const unsigned long long lo = (ph << 40) | pl, hi16 = ph >> 24;  // the 80-bit code: hi16:lo
-    s.mk[0][i] = ((unsigned long long)(~(uint32_t)cnt) << 32) | (hi16 << 16) | (lo >> 48);
-    s.mk[1][i] = lo << 16;
-}
-
-// How a compaction prepares the sort: nothing (the sort packs its own keys),
-// the radix sort's keys and digit counts (into the block histogram h), or the
-// merge sort's keys.
-enum KeyPrep : int { kPrepNone = 0, kPrepRadix = 1, kPrepMerge = 2 };
-
-// One entry of a compaction, with the sort keys `prep` asks for.
+// One entry of a compaction, with its sort keys (digit counts into the block histogram h).
 __device__ __forceinline__ void emit_entry(const SortScratch &ss, unsigned long long pos, unsigned long long khi,
-                                           unsigned long long klo, unsigned long long cnt, uint32_t lref, uint32_t *h,
-                                           int prep) {
+                                           unsigned long long klo, unsigned long long cnt, uint32_t lref, uint32_t *h) {
     ss.khi[pos] = khi;
     ss.klo[pos] = klo;
     ss.cnt[pos] = cnt;
     ss.lref[pos] = lref;
-    if (prep == kPrepRadix) sort_key_prep(ss, pos, khi, klo, cnt, h);
-    else if (prep == kPrepMerge) ms_key_prep(ss, pos, khi, klo, cnt);
+    sort_key_prep(ss, pos, khi, klo, cnt, h);
 }
 
 // Occupied 16-byte-key slots -> entries (big-endian key halves); block bid of nb.
 __device__ __forceinline__ void compact_short_body(const GSlot *slots, unsigned long long cap, const SortScratch &ss,
-                                                   unsigned long long *meta, unsigned bid, unsigned nb, uint32_t *h,
-                                                   int prep) {
+                                                   unsigned long long *meta, unsigned bid, unsigned nb,
+                                                   uint32_t *h) {
     __shared__ BlockTake sh;
     const unsigned long long step = (unsigned long long)nb * blockDim.x * kScanUnroll;
     for (unsigned long long b = (unsigned long long)bid * blockDim.x * kScanUnroll; b < cap; b += step) {
@@ -151,7 +129,7 @@ __device__ __forceinline__ void compact_short_body(const GSlot *slots, unsigned 
 #pragma unroll
         for (int u = 0; u < kScanUnroll; u++) {
             if (key_zero(k[u])) continue;
-            emit_entry(ss, pos, be64(k[u].x, k[u].y), be64(k[u].z, k[u].w), c[u], 0u, h, prep);
+            emit_entry(ss, pos, be64(k[u].x, k[u].y), be64(k[u].z, k[u].w), c[u], 0u, h);
             pos++;
         }
     }
@@ -159,8 +137,8 @@ __device__ __forceinline__ void compact_short_body(const GSlot *slots, unsigned 
 
 // Occupied 8-byte-key slots -> entries; block bid of nb.
 __device__ __forceinline__ void compact8_body(const G8Slot *slots, unsigned long long cap, const SortScratch &ss,
-                                              unsigned long long *meta, unsigned bid, unsigned nb, uint32_t *h,
-                                              int prep) {
+                                              unsigned long long *meta, unsigned bid, unsigned nb,
+                                              uint32_t *h) {
     __shared__ BlockTake sh;
     const unsigned long long step = (unsigned long long)nb * blockDim.x * kScanUnroll;
     for (unsigned long long b = (unsigned long long)bid * blockDim.x * kScanUnroll; b < cap; b += step) {
@@ -181,7 +159,7 @@ __device__ __forceinline__ void compact8_body(const G8Slot *slots, unsigned long
         for (int u = 0; u < kScanUnroll; u++) {
             const unsigned long long key = v[u].x;
             if (!key) continue;
-            emit_entry(ss, pos, be64((uint32_t)key, (uint32_t)(key >> 32)), 0ull, v[u].y, 0u, h, prep);
+            emit_entry(ss, pos, be64((uint32_t)key, (uint32_t)(key >> 32)), 0ull, v[u].y, 0u, h);
             pos++;
         }
     }
@@ -193,16 +171,17 @@ __device__ __forceinline__ uint32_t byte16(uint4 v, uint32_t i) {
     return (w >> (8u * (i & 3u))) & 0xFFu;
 }
 
-// One lane per long-word slot: a warp's occupied slots take their entry
-// positions, long-word indices and arena bytes with one atomic each.  Each
-// word is copied (lowercased, followed by one 0 byte so a run in the arena
-// ends where the word ends) into the arena, by its own lane up to 64 bytes
-// and by the whole warp beyond, and emits an entry.  A word of at most 32
-// letters whose slot holds its first and last 16 letters (kLongReady) is
-// written from the slot, without reading its occurrence in the text.
-__device__ __forceinline__ void compact_long_body(const LSlot *ls, unsigned long long lcap, const SortScratch &ss,
-                                                  const DevTable &out, unsigned bid, unsigned nb, uint32_t *hist,
-                                                  int prep) {
+// One lane per long-word slot: a warp's occupied slots take their long-word
+// indices and arena bytes with one atomic each.  Each word is copied
+// (lowercased, followed by one 0 byte so a run in the arena ends where the word
+// ends) into the arena, by its own lane up to 64 bytes and by the whole warp
+// beyond; then emit(slot, rank, occupied, khi, klo, count, lref, nocc, length) runs in every lane
+// (rank: among the warp's nocc occupied slots).  A word of at most 32 letters
+// whose slot holds its first and last 16 letters (kLongReady) is written from
+// the slot, without reading its occurrence in the text.
+template <class Emit>
+__device__ __forceinline__ void long_slots_body(const LSlot *ls, unsigned long long lcap, const DevTable &out,
+                                                unsigned bid, unsigned nb, Emit &&emit) {
     const int lane = threadIdx.x & 31;
     const unsigned long long nw = ((unsigned long long)nb * blockDim.x) >> 5;
     unsigned long long *meta = out.d_meta;
@@ -228,23 +207,19 @@ __device__ __forceinline__ void compact_long_body(const LSlot *ls, unsigned long
         }
         const unsigned long long rank = __popc(m & lanemask_lt()), nocc = __popc(m);
         const unsigned long long bytes = occ ? len + 1 : 0ull;
-        unsigned long long incl = bytes, tok = occ ? c : 0ull;
+        unsigned long long incl = bytes;
         for (int d = 1; d < 32; d <<= 1) {
             const unsigned long long t = __shfl_up_sync(kFull, incl, d);
             if (lane >= d) incl += t;
         }
-        for (int d = 16; d; d >>= 1) tok += __shfl_xor_sync(kFull, tok, d);
         const unsigned long long total = __shfl_sync(kFull, incl, 31);
-        unsigned long long boff = 0, blidx = 0, bpos = 0;
+        unsigned long long boff = 0, blidx = 0;
         if (lane == 0) {
             boff = atomicAdd(&meta[2], total);
             blidx = atomicAdd(&meta[1], nocc);
-            bpos = atomicAdd(&meta[0], nocc);
-            atomicAdd(&meta[3], tok);
         }
         const unsigned long long off = __shfl_sync(kFull, boff, 0) + incl - bytes;
         const unsigned long long lidx = __shfl_sync(kFull, blidx, 0) + rank;
-        const unsigned long long pos = __shfl_sync(kFull, bpos, 0) + rank;
         // The arena or the long index is full: the table fails (status), but
         // the entry slot taken above is still filled (prefix key, no long
         // reference) so that the sort that follows reads only valid entries.
@@ -263,6 +238,7 @@ __device__ __forceinline__ void compact_long_body(const LSlot *ls, unsigned long
             const unsigned long long bo = __shfl_sync(kFull, off, l), bl = __shfl_sync(kFull, len, l);
             for (unsigned long long j = lane; j < bl; j += 32) out.arena[bo + j] = (uint8_t)(bs[j] | 0x20u);
         }
+        unsigned long long hi = 0, lo = 0;
         if (occ) {
             if (full) {
                 atomicOr(out.d_status, ST_ARENA_FULL);
@@ -271,7 +247,6 @@ __device__ __forceinline__ void compact_long_body(const LSlot *ls, unsigned long
                 out.loff[lidx] = off;
                 out.llen[lidx] = len;
             }
-            unsigned long long hi = 0, lo = 0;
             if (from_slot) {  // f holds the first 16 letters, lowercased, little-endian words
                 hi = ((unsigned long long)__byte_perm(f.x, 0, 0x0123) << 32) | __byte_perm(f.y, 0, 0x0123);
                 lo = ((unsigned long long)__byte_perm(f.z, 0, 0x0123) << 32) | __byte_perm(f.w, 0, 0x0123);
@@ -279,53 +254,50 @@ __device__ __forceinline__ void compact_long_body(const LSlot *ls, unsigned long
                 for (int j = 0; j < 8; j++) hi = (hi << 8) | (unsigned long long)(src[j] | 0x20u);
                 for (int j = 8; j < 16; j++) lo = (lo << 8) | (unsigned long long)(src[j] | 0x20u);
             }
-            emit_entry(ss, pos, hi, lo, c, full ? 0u : (uint32_t)(lidx + 1), hist, prep);
         }
+        emit(w, (uint32_t)rank, occ, hi, lo, c, full ? 0u : (uint32_t)(lidx + 1), (uint32_t)nocc, len);
     }
+}
+__device__ __forceinline__ void compact_long_body(const LSlot *ls, unsigned long long lcap, const SortScratch &ss,
+                                                  const DevTable &out, unsigned bid, unsigned nb, uint32_t *hist) {
+    const int lane = threadIdx.x & 31;
+    long_slots_body(ls, lcap, out, bid, nb, [&](unsigned long long, uint32_t rank, bool occ, unsigned long long hi,
+                                                unsigned long long lo, unsigned long long c, uint32_t lref, uint32_t nocc,
+                                                unsigned long long) {
+        unsigned long long tok = occ ? c : 0ull, pos = 0;
+        for (int d = 16; d; d >>= 1) tok += __shfl_xor_sync(kFull, tok, d);
+        if (lane == 0) {
+            pos = atomicAdd(&out.d_meta[0], (unsigned long long)nocc);
+            atomicAdd(&out.d_meta[3], tok);
+        }
+        pos = __shfl_sync(kFull, pos, 0) + rank;
+        if (occ) emit_entry(ss, pos, hi, lo, c, lref, hist);
+    });
 }
 
 // All three tables' occupied slots -> entries in one launch: blocks
 // [0, nb8) scan the 8-byte table, the next nb16 the 16-byte table and the
 // rest the long-word table.  The per-kind entry counts go to meta[5] (8-byte)
-// and meta[6] (16-byte).  In a single table's finish the entries' sort keys
-// are prepared here as well (`prep`; for the radix sort with the digit
-// histograms of its passes).
+// and meta[6] (16-byte).  The entries' radix keys and the digit histograms of
+// the passes are prepared here as well.
 __global__ void __launch_bounds__(256) k_compact_all(GTable g, unsigned long long cap8, unsigned long long cap16,
                                                      unsigned long long lcap, SortScratch ss, DevTable out,
-                                                     unsigned nb8, unsigned nb16, int prep) {
+                                                     unsigned nb8, unsigned nb16) {
     __shared__ uint32_t h[kPasses * 256];
     grid_dependency_wait();
     grid_dependency_trigger();
-    const bool hist = prep == kPrepRadix;
-    if (hist) {
-        for (int i = threadIdx.x; i < kPasses * 256; i += blockDim.x) h[i] = 0u;
-        __syncthreads();
-    }
-    uint32_t *hp = hist ? h : nullptr;
+    for (int i = threadIdx.x; i < kPasses * 256; i += blockDim.x) h[i] = 0u;
+    __syncthreads();
     const unsigned b = blockIdx.x;
-    if (b < nb8) compact8_body(g.slots8, cap8, ss, out.d_meta, b, nb8, hp, prep);
-    else if (b < nb8 + nb16) compact_short_body(g.slots, cap16, ss, out.d_meta, b - nb8, nb16, hp, prep);
-    else compact_long_body(g.lslots, lcap, ss, out, b - nb8 - nb16, gridDim.x - nb8 - nb16, hp, prep);
-    if (hist) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < kPasses * 256; i += blockDim.x)
-            if (h[i]) atomicAdd(&ss.hist_all[i], h[i]);
-    }
+    if (b < nb8) compact8_body(g.slots8, cap8, ss, out.d_meta, b, nb8, h);
+    else if (b < nb8 + nb16) compact_short_body(g.slots, cap16, ss, out.d_meta, b - nb8, nb16, h);
+    else compact_long_body(g.lslots, lcap, ss, out, b - nb8 - nb16, gridDim.x - nb8 - nb16, h);
+    __syncthreads();
+    for (int i = threadIdx.x; i < kPasses * 256; i += blockDim.x)
+        if (h[i]) atomicAdd(&ss.hist_all[i], h[i]);
 }
 
 // ---------------------------------------------------------------- radix sort
-// The sort kernels take one table's arguments as their parameter (OneJob) or
-// several tables' from a device array, table blockIdx.y (JobList): a batch's
-// class and global tables are sorted by one launch per pass.
-struct OneJob {
-    SortJob j;
-    __device__ __forceinline__ const SortJob &get() const { return j; }
-};
-struct JobList {
-    const SortJob *j;
-    __device__ __forceinline__ const SortJob &get() const { return j[blockIdx.y]; }
-};
-
 __device__ __forceinline__ uint32_t sort_digit(const SortScratch &s, uint32_t idx, int p) {
     if (p >= kPasses) return (s.doc[idx] >> (8 * (p - kPasses))) & 0xFFu;
     if (p < 8) return (uint32_t)(s.pk[idx] >> (8 * p)) & 0xFFu;
@@ -335,10 +307,9 @@ __device__ __forceinline__ uint32_t sort_digit(const SortScratch &s, uint32_t id
 
 // Packs the prefix keys, and takes the histograms of all digit positions
 // (for skipping constant digits) and the identity permutation.
-template <class J>
-__global__ void k_hist_all(J job, int passes) {
-    const SortScratch &s = job.get().s;
-    const unsigned long long *meta = job.get().meta;
+__global__ void k_hist_all(SortJob job, int passes) {
+    const SortScratch &s = job.s;
+    const unsigned long long *meta = job.meta;
     __shared__ uint32_t h[kPassesSeg * 256];
     for (int i = threadIdx.x; i < kPassesSeg * 256; i += blockDim.x) h[i] = 0;
     __syncthreads();
@@ -364,10 +335,9 @@ __device__ __forceinline__ bool pass_skipped(const SortScratch &s, int p, unsign
     return __syncthreads_or(mine) != 0;
 }
 
-template <class J>
-__global__ void __launch_bounds__(kSortThreads) k_pass_count(J job, int p, int e, int fused) {
-    const SortScratch &s = job.get().s;
-    const unsigned long long *meta = job.get().meta;
+__global__ void __launch_bounds__(kSortThreads) k_pass_count(SortJob job, int p, int e, int fused) {
+    const SortScratch &s = job.s;
+    const unsigned long long *meta = job.meta;
     __shared__ uint32_t h[256];
     const unsigned long long n = meta[0];
     const unsigned long long ntiles = (n + kSortTile - 1) / kSortTile;
@@ -403,10 +373,9 @@ __global__ void __launch_bounds__(kSortThreads) k_pass_count(J job, int p, int e
 // digit-major tile histogram: block d scans digit d's
 // row of tile counts, starting from the number of elements with a smaller
 // digit (from the all-pass histogram).  256 blocks of 256 threads.
-template <class J>
-__global__ void __launch_bounds__(256) k_pass_scan(J job, int p, int e, int last) {
-    const SortScratch &s = job.get().s;
-    const unsigned long long *meta = job.get().meta;
+__global__ void __launch_bounds__(256) k_pass_scan(SortJob job, int p, int e, int last) {
+    const SortScratch &s = job.s;
+    const unsigned long long *meta = job.meta;
     __shared__ uint32_t part[256];
     __shared__ uint32_t base_s;
     const unsigned long long n = meta[0];
@@ -454,10 +423,9 @@ __global__ void __launch_bounds__(256) k_pass_scan(J job, int p, int e, int last
 
 // Stable scatter: warp w ranks its 512 consecutive elements in order with
 // match_any; warps are combined in order, so equal digits keep their order.
-template <class J>
-__global__ void __launch_bounds__(kSortThreads) k_pass_scatter(J job, int p, int e, int fused, int last) {
-    const SortScratch &s = job.get().s;
-    const unsigned long long *meta = job.get().meta;
+__global__ void __launch_bounds__(kSortThreads) k_pass_scatter(SortJob job, int p, int e, int fused, int last) {
+    const SortScratch &s = job.s;
+    const unsigned long long *meta = job.meta;
     constexpr int WARPS = kSortThreads / 32;
     static_assert(kSortThreads == 256, "one thread per digit");
     __shared__ uint32_t wcount[WARPS][256];
@@ -581,12 +549,11 @@ __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t *p) {
     asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-template <class J>
-__global__ void __launch_bounds__(kSortThreads) k_pass_one(J job, int p, int e, int last) {
+__global__ void __launch_bounds__(kSortThreads) k_pass_one(SortJob job, int p, int e, int last) {
     grid_dependency_wait();
     grid_dependency_trigger();
-    const SortScratch &s = job.get().s;
-    const unsigned long long *meta = job.get().meta;
+    const SortScratch &s = job.s;
+    const unsigned long long *meta = job.meta;
     constexpr int WARPS = kSortThreads / 32;
     __shared__ uint32_t wcount[WARPS][256];
     __shared__ uint32_t wtot[WARPS];
@@ -710,300 +677,8 @@ __global__ void __launch_bounds__(kSortThreads) k_pass_one(J job, int p, int e, 
     }
 }
 
-// ---------------------------------------------------------------- merge sort
-// A single table's finish (counts below 2^32) sorts its entries by one
-// 128-bit key each (ms_key_prep: count descending, then the 16-letter
-// prefix); the entry index travels with the key.  Keys that tie belong to
-// long words sharing count and prefix, which the long-word fix-up orders
-// afterwards, so ties may come out in any order.  Blocks first sort runs of
-// kMsTile entries: each thread sorts kMsPer entries in registers (a bitonic
-// network), then the block merges pairs of sorted pieces in shared memory
-// until the run is whole.  Each round then merges pairs of runs into runs
-// twice as long, until one run holds every entry: ceil(log2(n / kMsTile))
-// rounds, each one launch in which no block waits for another.  A block of a
-// round writes kMsTile consecutive outputs of one merged pair: it finds how
-// many of them come from the first run at its first and last output (the
-// merge path split; each search step tests kMsThreads candidates at once, one
-// a thread, and keeps the interval between the last that goes first and the
-// first that does not), stages the two input pieces in shared memory, and
-// merges kMsPer outputs a thread.  Every merge takes the first run's entry on
-// a tie, and every search counts the same way.  Keys and indices alternate
-// between two buffers: the run sort writes buffer 1, round r reads buffer
-// r & 1.
-constexpr int kMsTile = 4096;
-constexpr int kMsThreads = 256;
-constexpr int kMsPer = kMsTile / kMsThreads;  // entries a thread sorts or merges
-static_assert(kMsPer == 16 && (kMsTile & (kMsTile - 1)) == 0, "16 entries a thread, power-of-two runs");
-// Shared memory: slot i at i + i / 16, so that the 16 consecutive entries of
-// each of a warp's threads fall in different banks.
-constexpr int kMsSlots = kMsTile + kMsTile / 16;
-constexpr size_t kMsSmem = (size_t)kMsSlots * (8 + 8 + 4);
-__host__ __device__ __forceinline__ int ms_rounds(unsigned long long n) {
-    int r = 0;
-    for (unsigned long long len = kMsTile; len < n; len <<= 1) r++;
-    return r;
-}
-struct MsKey {
-    unsigned long long h, l;
-    uint32_t x;  // entry index (not compared)
-};
-// A run sort's key: the index within the run in the 16 free low bits of l.
-struct MsKey2 {
-    unsigned long long h, l;
-};
-__device__ __forceinline__ bool ms_less(const MsKey &a, const MsKey &b) { return a.h != b.h ? a.h < b.h : a.l < b.l; }
-__device__ __forceinline__ bool ms_less(const MsKey2 &a, const MsKey2 &b) { return a.h != b.h ? a.h < b.h : a.l < b.l; }
-struct MsShared {
-    unsigned long long *h, *l;
-    uint32_t *x;
-    __device__ __forceinline__ explicit MsShared(unsigned long long *base)
-        : h(base), l(base + kMsSlots), x(reinterpret_cast<uint32_t *>(base + 2 * kMsSlots)) {}
-    __device__ __forceinline__ static uint32_t at(uint32_t i) { return i + (i >> 4); }
-    __device__ __forceinline__ void get(uint32_t i, MsKey &k) const {
-        const uint32_t j = at(i);
-        k = MsKey{h[j], l[j], x[j]};
-    }
-    __device__ __forceinline__ void get(uint32_t i, MsKey2 &k) const {
-        const uint32_t j = at(i);
-        k = MsKey2{h[j], l[j]};
-    }
-    __device__ __forceinline__ void put(uint32_t i, const MsKey &k) const {
-        const uint32_t j = at(i);
-        h[j] = k.h;
-        l[j] = k.l;
-        x[j] = k.x;
-    }
-    __device__ __forceinline__ void put(uint32_t i, const MsKey2 &k) const {
-        const uint32_t j = at(i);
-        h[j] = k.h;
-        l[j] = k.l;
-    }
-};
-// How many of sm[a0, a0 + na) lead the first d outputs of merging them with
-// sm[b0, b0 + nb) (the first piece first on ties), by bisection.
-template <class K>
-__device__ __forceinline__ uint32_t ms_split(const MsShared &sm, uint32_t a0, uint32_t na, uint32_t b0, uint32_t nb,
-                                             uint32_t d) {
-    uint32_t lo = d > nb ? d - nb : 0u, hi = d < na ? d : na;
-    while (lo < hi) {
-        const uint32_t m = (lo + hi) >> 1;
-        K ka, kb;
-        sm.get(a0 + m, ka);
-        sm.get(b0 + d - 1 - m, kb);
-        if (!ms_less(kb, ka)) lo = m + 1;
-        else hi = m;
-    }
-    return lo;
-}
-// cnt (<= kMsPer) outputs of merging sm[a0, a0 + na) with sm[b0, b0 + nb),
-// starting ia entries into the first and ib into the second, into v.
-template <class K>
-__device__ __forceinline__ void ms_merge_into(const MsShared &sm, uint32_t a0, uint32_t na, uint32_t b0, uint32_t nb,
-                                              uint32_t ia, uint32_t ib, uint32_t cnt, K (&v)[kMsPer]) {
-    K ka{}, kb{};
-    if (ia < na) sm.get(a0 + ia, ka);
-    if (ib < nb) sm.get(b0 + ib, kb);
-#pragma unroll
-    for (int k = 0; k < kMsPer; k++) {
-        if ((uint32_t)k < cnt) {  // ia + ib < na + nb: one of the pieces has an entry left
-            const bool fromA = ib >= nb || (ia < na && !ms_less(kb, ka));
-            v[k] = fromA ? ka : kb;
-            // one load path for either piece (lanes taking from different
-            // pieces do not diverge): the taken piece's next entry
-            ia += fromA ? 1u : 0u;
-            ib += fromA ? 0u : 1u;
-            const uint32_t nx = fromA ? ia : ib;
-            if (nx < (fromA ? na : nb)) {
-                K nk;
-                sm.get((fromA ? a0 : b0) + nx, nk);
-                if (fromA) ka = nk;
-                else kb = nk;
-            }
-        }
-    }
-}
-
-// Sorts entries [kMsTile * b, kMsTile * (b + 1)) of buffer 0 into buffer 1;
-// block 0 records which buffer the last round leaves the order in.
-__global__ void __launch_bounds__(kMsThreads) k_ms_runs(SortScratch s, const unsigned long long *meta) {
-    extern __shared__ __align__(16) unsigned long long ms_smem[];
-    const MsShared sm(ms_smem);
-    grid_dependency_wait();
-    grid_dependency_trigger();
-    const unsigned long long n = meta[0];
-    if (blockIdx.x == 0 && threadIdx.x == 0) s.cur[kCurFinal] = (ms_rounds(n) & 1) ? 0u : 1u;
-    const unsigned long long base = (unsigned long long)blockIdx.x * kMsTile;
-    if (base >= n) return;
-    const uint32_t m = (uint32_t)(n - base < (unsigned long long)kMsTile ? n - base : (unsigned long long)kMsTile);
-    const uint32_t t = threadIdx.x;
-    // coalesced loads into shared memory (padding past m sorts last), then
-    // each thread's kMsPer consecutive entries into registers
-    MsKey2 v[kMsPer];
-#pragma unroll
-    for (int k = 0; k < kMsPer; k++) {
-        const uint32_t i = t + (uint32_t)k * kMsThreads;
-        v[k] = i < m ? MsKey2{s.mk[0][base + i], s.mk[1][base + i] | i} : MsKey2{~0ull, ~0ull};
-    }
-#pragma unroll
-    for (int k = 0; k < kMsPer; k++) sm.put(t + (uint32_t)k * kMsThreads, v[k]);
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kMsPer; k++) sm.get(kMsPer * t + k, v[k]);
-    // bitonic network over the thread's entries (ascending)
-#pragma unroll
-    for (int k = 2; k <= kMsPer; k <<= 1)
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1)
-#pragma unroll
-            for (int i = 0; i < kMsPer; i++) {
-                const int p = i ^ j;
-                if (p > i && ms_less(v[p], v[i]) == ((i & k) == 0)) {
-                    const MsKey2 w = v[i];
-                    v[i] = v[p];
-                    v[p] = w;
-                }
-            }
-    // merge sorted pieces of sz entries in pairs until the run is whole;
-    // thread t produces outputs [kMsPer * t, kMsPer * (t + 1)) of its pair
-    for (uint32_t sz = kMsPer; sz < (uint32_t)kMsTile; sz <<= 1) {
-        __syncthreads();  // every thread has read the previous level
-#pragma unroll
-        for (int k = 0; k < kMsPer; k++) sm.put(kMsPer * t + k, v[k]);
-        __syncthreads();
-        const uint32_t g0 = (kMsPer * t) & ~(2 * sz - 1), d = kMsPer * t - g0;
-        const uint32_t ia = ms_split<MsKey2>(sm, g0, sz, g0 + sz, sz, d);
-        ms_merge_into(sm, g0, sz, g0 + sz, sz, ia, d - ia, kMsPer, v);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kMsPer; k++) sm.put(kMsPer * t + k, v[k]);
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kMsPer; k++) {
-        const uint32_t i = t + (uint32_t)k * kMsThreads;
-        if (i < m) {
-            MsKey2 w;
-            sm.get(i, w);
-            s.mk[2][base + i] = w.h;
-            s.mk[3][base + i] = w.l & ~0xFFFFull;
-            s.perm[1][base + i] = (uint32_t)(base + (w.l & 0xFFFFull));
-        }
-    }
-}
-
-// Round r: runs of kMsTile << (r - 1) entries merged in pairs.
-__global__ void __launch_bounds__(kMsThreads) k_ms_merge(SortScratch s, const unsigned long long *meta, int r) {
-    extern __shared__ __align__(16) unsigned long long ms_smem[];
-    const MsShared sm(ms_smem);
-    grid_dependency_wait();
-    grid_dependency_trigger();
-    const unsigned long long n = meta[0];
-    const unsigned long long R = (unsigned long long)kMsTile << (r - 1);
-    const unsigned long long out0 = (unsigned long long)blockIdx.x * kMsTile;
-    if (R >= n || out0 >= n) return;  // one run holds everything already / no tile
-    const uint32_t src = (uint32_t)r & 1u;
-    const unsigned long long *ih = s.mk[src ? 2 : 0], *il = s.mk[src ? 3 : 1];
-    const uint32_t *ix = s.perm_buf(src);
-    unsigned long long *oh = s.mk[src ? 0 : 2], *ol = s.mk[src ? 1 : 3];
-    uint32_t *ox = s.perm_buf(1u - src);
-    // this tile's pair: run A = [p0, ae), run B = [ae, be); outputs [out0, out1)
-    const unsigned long long out1 = out0 + kMsTile < n ? out0 + kMsTile : n;
-    const unsigned long long p0 = out0 / (2 * R) * (2 * R);
-    const unsigned long long ae = p0 + R < n ? p0 + R : n, be = p0 + 2 * R < n ? p0 + 2 * R : n;
-    const uint32_t la = (uint32_t)(ae - p0), lb = (uint32_t)(be - ae);
-    const uint32_t d0 = (uint32_t)(out0 - p0), d1 = (uint32_t)(out1 - p0);
-    // A[a] goes before B[d - 1 - a]: its key is not above (A first on ties)
-    auto first = [&](uint32_t d, uint32_t a) {
-        const unsigned long long bh = ih[ae + d - 1 - a], bl = il[ae + d - 1 - a];
-        const unsigned long long ah = ih[p0 + a], al = il[p0 + a];
-        return !(bh != ah ? bh < ah : bl < al);
-    };
-    // the splits of outputs d0 and d1, searched together: a in
-    // [max(0, d - lb), min(d, la)], every bound block-uniform.  An interval
-    // of w <= E candidates is tested whole (thread i tests lo + i); a wider
-    // one at the P = E - 1 points lo + (i + 1) w / E (no division: E = 256)
-    constexpr uint32_t E = kMsThreads, P = E - 1;
-    static_assert(kMsThreads == 256, "candidates placed by a shift of 8");
-    auto cand = [](uint32_t lo, uint32_t w, uint32_t i) -> uint32_t {
-        return w <= E ? lo + i : lo + (uint32_t)(((unsigned long long)(i + 1) * w) >> 8);
-    };
-    uint32_t lo0 = d0 > lb ? d0 - lb : 0u, hi0 = d0 < la ? d0 : la;
-    uint32_t lo1 = d1 > lb ? d1 - lb : 0u, hi1 = d1 < la ? d1 : la;
-    const uint32_t t = threadIdx.x;
-    while (lo0 < hi0 || lo1 < hi1) {  // each step leaves at most w / E + 1 of w > E candidates, 0 of fewer
-        const uint32_t w0 = hi0 - lo0, w1 = hi1 - lo1;
-        const bool b0 = t < (w0 <= E ? w0 : P) && first(d0, cand(lo0, w0, t));
-        const bool b1 = t < (w1 <= E ? w1 : P) && first(d1, cand(lo1, w1, t));
-        const uint32_t c0 = (uint32_t)__syncthreads_count(b0), c1 = (uint32_t)__syncthreads_count(b1);
-        if (w0 <= E) {
-            lo0 += c0;
-            hi0 = lo0;
-        } else {
-            const uint32_t nl = c0 ? cand(lo0, w0, c0 - 1) + 1 : lo0;
-            if (c0 < P) hi0 = cand(lo0, w0, c0);
-            lo0 = nl;
-        }
-        if (w1 <= E) {
-            lo1 += c1;
-            hi1 = lo1;
-        } else {
-            const uint32_t nl = c1 ? cand(lo1, w1, c1 - 1) + 1 : lo1;
-            if (c1 < P) hi1 = cand(lo1, w1, c1);
-            lo1 = nl;
-        }
-    }
-    // the tile's inputs, A[lo0, lo1) then B[d0 - lo0, d1 - lo1): na + nb = L
-    const uint32_t L = d1 - d0, na = lo1 - lo0, nb = L - na;
-    const unsigned long long ga = p0 + lo0, gb = ae + (d0 - lo0);
-    MsKey v[kMsPer];
-#pragma unroll
-    for (int k = 0; k < kMsPer; k++) {
-        const uint32_t i = t + (uint32_t)k * kMsThreads;
-        if (i < L) {
-            const unsigned long long g = i < na ? ga + i : gb + (i - na);
-            v[k] = MsKey{ih[g], il[g], ix[g]};
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < kMsPer; k++) {
-        const uint32_t i = t + (uint32_t)k * kMsThreads;
-        if (i < L) sm.put(i, v[k]);
-    }
-    __syncthreads();
-    // thread t: outputs [kMsPer * t, ...) of the tile, from its own split
-    const uint32_t dt = kMsPer * t < L ? kMsPer * t : L, cnt = L - dt < (uint32_t)kMsPer ? L - dt : (uint32_t)kMsPer;
-    const uint32_t ia = ms_split<MsKey>(sm, 0, na, na, nb, dt);
-    ms_merge_into(sm, 0, na, na, nb, ia, dt - ia, cnt, v);
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kMsPer; k++)
-        if ((uint32_t)k < cnt) sm.put(dt + k, v[k]);
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kMsPer; k++) {
-        const uint32_t i = t + (uint32_t)k * kMsThreads;
-        if (i < L) {
-            MsKey w;
-            sm.get(i, w);
-            oh[out0 + i] = w.h;
-            ol[out0 + i] = w.l;
-            ox[out0 + i] = w.x;
-        }
-    }
-}
-
-// Compares two entries whose 16-byte prefixes are equal by the bytes after
-// the prefix (a word that fits the prefix is a proper prefix of a longer one).
 __device__ __forceinline__ bool tail_less(const LongView &v, uint32_t a, uint32_t b) {
-    uint32_t ra = v.lref[a], rb = v.lref[b];
-    if (ra == 0) return rb != 0;   // the 16-letter (or shorter) word is a prefix
-    if (rb == 0) return false;
-    const uint8_t *pa = v.arena + v.loff[ra - 1], *pb = v.arena + v.loff[rb - 1];
-    unsigned long long la = v.llen[ra - 1], lb = v.llen[rb - 1];
-    unsigned long long m = la < lb ? la : lb;
-    for (unsigned long long i = 16; i < m; i++)
-        if (pa[i] != pb[i]) return pa[i] < pb[i];
-    return la < lb;
+    return lref_less(v, v.lref[a], v.lref[b]);
 }
 
 // After the last pass, entries are in (document, count desc, 16-letter prefix
@@ -1014,13 +689,12 @@ __device__ __forceinline__ bool tail_less(const LongView &v, uint32_t a, uint32_
 __device__ __forceinline__ bool same_run(const SortScratch &s, uint32_t a, uint32_t b, bool seg) {
     return s.khi[a] == s.khi[b] && s.klo[a] == s.klo[b] && s.cnt[a] == s.cnt[b] && (!seg || s.doc[a] == s.doc[b]);
 }
-template <class J>
-__global__ void k_fix_long(J job, int passes) {
+__global__ void k_fix_long(SortJob job, int passes) {
     grid_dependency_wait();
     grid_dependency_trigger();
-    const SortScratch &s = job.get().s;
-    const LongView &v = job.get().v;
-    const unsigned long long *meta = job.get().meta;
+    const SortScratch &s = job.s;
+    const LongView &v = job.v;
+    const unsigned long long *meta = job.meta;
     const unsigned long long n = meta[0];
     if (meta[1] == 0) return;
     const bool seg = passes > kPasses;
@@ -1056,12 +730,11 @@ __device__ __forceinline__ unsigned long long short_len(unsigned long long hi, u
     return 8 - (__ffsll((long long)hi) - 1) / 8;
 }
 
-template <class J>
-__global__ void k_gather_final(J job) {
+__global__ void k_gather_final(SortJob job) {
     grid_dependency_wait();
     grid_dependency_trigger();
-    const SortScratch &s = job.get().s;
-    const DevTable &out = job.get().out;
+    const SortScratch &s = job.s;
+    const DevTable &out = job.out;
     const unsigned long long n = out.d_meta[0];
     if (blockIdx.x == 0 && threadIdx.x == 0 && s.cur[kCurSortError]) atomicOr(out.d_status, ST_TIMEOUT);
     const uint32_t *perm = s.perm_buf(s.cur[kCurFinal]);
@@ -1114,26 +787,20 @@ static int grid_for(unsigned long long n, int threads, int max_blocks) {
     return (int)g;
 }
 
-// A single table's finish merge-sorts when the scratch has the key buffers
-// and every count is below 2^32 (the radix sort's count digits 4..7 skipped).
-static bool use_msort(const SortScratch &ss, uint32_t skip) {
-    return ss.mk[0] && ((skip >> (kSortKeyPasses + 4)) & 0xFu) == 0xFu;
+// ---------------------------------------------------------------- radix finish
+int sort_entries_launches(int passes, uint64_t cap, uint32_t skip) {
+    const bool fused = (cap + kSortTile - 1) / kSortTile <= kSortFusedMaxTiles;
+    const uint32_t mask = passes >= 32 ? ~0u : ((1u << passes) - 1u);
+    const int per = cap < (1ull << 30) ? 1 : (fused ? 2 : 3);
+    return 1 + 1 + per * (passes - __builtin_popcount(skip & mask));
 }
 
-// reset + fused compaction + (run sort + merge rounds + long-word fix-up, or
-// the sort without its key pass) + gather
-int finish_table_launches(const SortScratch &ss, uint32_t skip) {
-    if (use_msort(ss, skip)) return 2 + 1 + ms_rounds(ss.cap) + 1 + 1;
-    return 2 + sort_entries_launches(kPasses, ss.cap, skip) - 1 + 1;
-}
-
-// The passes of one sort, for one table (J = OneJob) or a list of them;
-// keyed: the compaction has prepared the sort keys and histograms already.
-template <class J>
-static void launch_sort(const J &job, uint64_t cap, int ntab, int passes, uint32_t skip, cudaStream_t st,
-                        bool keyed = false) {
+// The passes of one sort; keyed: the compaction has prepared the sort keys
+// and histograms already.
+static void launch_sort(const SortJob &job, int passes, uint32_t skip, cudaStream_t st, bool keyed = false) {
     const int sms = sm_count();
-    if (!keyed) k_hist_all<<<dim3(grid_for(cap, 256, sms * 2), ntab), 256, 0, st>>>(job, passes);
+    const uint64_t cap = job.s.cap;
+    if (!keyed) k_hist_all<<<grid_for(cap, 256, sms * 2), 256, 0, st>>>(job, passes);
     const int ntiles = (int)((cap + kSortTile - 1) / kSortTile);
     const int fused = (uint64_t)ntiles <= kSortFusedMaxTiles;
     int lastp = -1;
@@ -1147,42 +814,22 @@ static void launch_sort(const J &job, uint64_t cap, int ntab, int passes, uint32
         if ((skip >> p) & 1u) continue;
         const int last = p == lastp;
         if (onesweep) {  // overlaps its launch with the tail of the kernel before
-            launch_dependent(k_pass_one<J>, dim3(ntiles, ntab), dim3(kSortThreads), 0, st, job, p, e, last);
+            launch_dependent(k_pass_one, dim3(ntiles), dim3(kSortThreads), 0, st, job, p, e, last);
         } else {
-            k_pass_count<<<dim3(ntiles, ntab), kSortThreads, 0, st>>>(job, p, e, fused);
-            if (!fused) k_pass_scan<<<dim3(256, ntab), 256, 0, st>>>(job, p, e, last);
-            k_pass_scatter<<<dim3(ntiles, ntab), kSortThreads, 0, st>>>(job, p, e, fused, last);
+            k_pass_count<<<ntiles, kSortThreads, 0, st>>>(job, p, e, fused);
+            if (!fused) k_pass_scan<<<256, 256, 0, st>>>(job, p, e, last);
+            k_pass_scatter<<<ntiles, kSortThreads, 0, st>>>(job, p, e, fused, last);
         }
         e++;
     }
-    launch_dependent(k_fix_long<J>, dim3(grid_for(cap, 256, sms * 4), ntab), dim3(256), 0, st, job, passes);
-}
-
-// Merge sort of a single table's entries (keys from the compaction): the
-// runs, every round the capacity may need (rounds beyond the entries' own
-// return at once), then the long-word fix-up.
-static void launch_msort(const OneJob &job, uint64_t cap, cudaStream_t st) {
-    const int grid = (int)std::max<uint64_t>(1, (cap + kMsTile - 1) / kMsTile);
-    ensure_smem_limit((const void *)k_ms_runs, (int)kMsSmem);
-    ensure_smem_limit((const void *)k_ms_merge, (int)kMsSmem);
-    launch_dependent(k_ms_runs, dim3(grid), dim3(kMsThreads), kMsSmem, st, job.j.s, job.j.meta);
-    for (int r = 1; r <= ms_rounds(cap); r++)
-        launch_dependent(k_ms_merge, dim3(grid), dim3(kMsThreads), kMsSmem, st, job.j.s, job.j.meta, r);
-    launch_dependent(k_fix_long<OneJob>, dim3(grid_for(cap, 256, sm_count() * 4)), dim3(256), 0, st, job, kPasses);
+    launch_dependent(k_fix_long, dim3(grid_for(cap, 256, sms * 4)), dim3(256), 0, st, job, passes);
 }
 
 // LSD radix sort of the entries in ss (count n = meta[0]) into ss.perm_buf(ss.cur[passes]).
 cudaError_t sort_entries(SortScratch &ss, const unsigned long long *meta, const LongView &v, int passes,
                          cudaStream_t st, uint32_t skip) {
-    OneJob job{SortJob{ss, meta, v, DevTable{}}};
-    launch_sort(job, ss.cap, 1, passes, skip, st);
+    launch_sort(SortJob{ss, meta, v, DevTable{}}, passes, skip, st);
     return cudaGetLastError();
-}
-int sort_entries_launches(int passes, uint64_t cap, uint32_t skip) {
-    const bool fused = (cap + kSortTile - 1) / kSortTile <= kSortFusedMaxTiles;
-    const uint32_t mask = passes >= 32 ? ~0u : ((1u << passes) - 1u);
-    const int per = cap < (1ull << 30) ? 1 : (fused ? 2 : 3);
-    return 1 + 1 + per * (passes - __builtin_popcount(skip & mask));
 }
 
 uint32_t sort_skip_mask(uint64_t max_count, uint64_t ndocs) {
@@ -1219,52 +866,351 @@ void sort_state_reset(SortScratch &ss, cudaStream_t st) {
     k_sort_reset<<<grid_for(n, 256, sm_count() * 2), 256, 0, st>>>(ss, 256 * ntiles);
 }
 
-// Resets the sort state and compacts the three tables in one launch (with
-// `keyed`, also preparing the sort keys and histograms).
-static void launch_compaction(const GTable &g, uint64_t gcap8, uint64_t gcap, uint64_t glcap, SortScratch &ss,
-                              DevTable &out, cudaStream_t st, int prep) {
+// reset + compaction (with the sort keys) + passes + long-word fix-up + gather
+static void finish_by_radix(const GTable &g, uint64_t gcap8, uint64_t gcap, uint64_t glcap, SortScratch &ss,
+                            DevTable &out, cudaStream_t st, uint32_t skip) {
     const int sms = sm_count();
     sort_state_reset(ss, st);
     const int nb8 = grid_for(gcap8, 256 * kScanUnroll, sms * 8), nb16 = grid_for(gcap, 256 * kScanUnroll, sms * 8),
               nbl = grid_for(glcap, 256, sms * 8);
     launch_dependent(k_compact_all, dim3(nb8 + nb16 + nbl), dim3(256), 0, st, g, (unsigned long long)gcap8,
-                     (unsigned long long)gcap, (unsigned long long)glcap, ss, out, (unsigned)nb8, (unsigned)nb16, prep);
+                     (unsigned long long)gcap, (unsigned long long)glcap, ss, out, (unsigned)nb8, (unsigned)nb16);
+    const SortJob job{ss, out.d_meta, LongView{ss.lref, out.loff, out.llen, out.arena}, out};
+    launch_sort(job, kPasses, skip, st, true);
+    launch_dependent(k_gather_final, dim3(grid_for(ss.cap, 256 * kScanUnroll, sms * 8)), dim3(256), 0, st, job);
 }
 
-cudaError_t finish_table(const GTable &g, uint64_t gcap8, uint64_t gcap, uint64_t glcap, SortScratch &ss,
-                         DevTable &out, cudaStream_t st, uint32_t skip) {
-    const bool ms = use_msort(ss, skip);
-    launch_compaction(g, gcap8, gcap, glcap, ss, out, st, ms ? kPrepMerge : kPrepRadix);
-    OneJob job{SortJob{ss, out.d_meta, LongView{ss.lref, out.loff, out.llen, out.arena}, out}};
-    if (ms) launch_msort(job, ss.cap, st);
-    else launch_sort(job, ss.cap, 1, kPasses, skip, st, true);
-    launch_dependent(k_gather_final<OneJob>, dim3(grid_for(ss.cap, 256 * kScanUnroll, sm_count() * 8)), dim3(256), 0,
-                     st, job);
+// ---------------------------------------------------------------- bucket finish
+size_t bucket_scratch_bytes(uint64_t cap) {
+    BucketScratch s{};
+    bucket_scratch_carve(s, nullptr, cap);
+    return (size_t)reinterpret_cast<uintptr_t>(s.big_lref) + 4 * cap + 256;
+}
+
+void bucket_scratch_carve(BucketScratch &s, void *base, uint64_t cap) {
+    uintptr_t p = reinterpret_cast<uintptr_t>(base);
+    auto take = [&](size_t n) { void *r = reinterpret_cast<void *>(p); p += (n + 255) & ~(size_t)255; return r; };
+    s.groups = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(kBktGroups, (cap + kBktProbes - 1) / kBktProbes));
+    s.rank_blocks = s.groups;  // two keys a warp
+    s.tree = 2;
+    while (s.tree <= s.splits()) s.tree *= 2;
+    const size_t keep = (size_t)s.groups * kBktKeep, split = s.splits();
+    // twice the slots: tables are at most about half full, so a bucket may
+    // hold four times its share before entries spill
+    s.slots = kOneSlot ? cap / 16 : 2 * cap;  // (the one-slot test build spills)
+    s.kept = static_cast<ulonglong2 *>(take(keep * 16));
+    s.split = static_cast<ulonglong2 *>(take(split * 16));
+    s.kept_tie = static_cast<uint32_t *>(take(keep * 4));
+    s.split_tie = static_cast<uint32_t *>(take(split * 4));
+    s.found = static_cast<uint2 *>(take(s.groups * sizeof(uint2)));
+    s.count = static_cast<uint32_t *>(take((split + 1) * kBktStride * 4));
+    s.first = static_cast<uint32_t *>(take((split + 1) * 4));
+    s.state = static_cast<uint32_t *>(take(64));
+    s.key = static_cast<ulonglong2 *>(take(s.slots * 16));
+    s.lref = static_cast<uint32_t *>(take(s.slots * 4));
+    s.spill_key = static_cast<ulonglong2 *>(take(cap * 16));
+    s.spill_lref = static_cast<uint32_t *>(take(cap * 4));
+    s.spill_bucket = static_cast<uint32_t *>(take(cap * 4));
+    s.big_key = static_cast<ulonglong2 *>(take(cap * 16));
+    s.big_lref = static_cast<uint32_t *>(take(cap * 4));
+}
+
+// One table's finish; the kernels take it as their parameter (OneFinish) or
+// several tables' from a device array, table blockIdx.y (FinishList): a batch's
+// class and global tables are finished by one launch a step.
+struct FinishJob {
+    GTable g;
+    unsigned long long cap8, cap16, lcap;
+    BucketScratch s;
+    DevTable out;
+};
+struct OneFinish {
+    FinishJob j;
+    __device__ __forceinline__ const FinishJob &get() const { return j; }
+};
+struct FinishList {
+    const FinishJob *j;
+    __device__ __forceinline__ const FinishJob &get() const { return j[blockIdx.y]; }
+};
+
+// The slots of the three hash tables, one after another.
+struct TableSource {
+    const FinishJob &j;
+    __device__ __forceinline__ unsigned long long cap() const { return j.cap8 + j.cap16 + j.lcap; }
+    __device__ __forceinline__ bool get(unsigned long long i, Key128 &k, uint32_t &tie) const {
+        tie = 0u;
+        if (i < j.cap8) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(&j.g.slots8[i]);
+            if (!v.x) return false;
+            k = count_key(v.y, be_half((uint32_t)v.x, (uint32_t)(v.x >> 32)), 0ull);
+            return true;
+        }
+        i -= j.cap8;
+        if (i < j.cap16) {
+            const uint4 w = j.g.slots[i].key;
+            if (key_zero(w)) return false;
+            k = count_key(j.g.slots[i].cnt, be_half(w.x, w.y), be_half(w.z, w.w));
+            return true;
+        }
+        i -= j.cap16;
+        const LSlot &l = j.g.lslots[i];
+        if (l.h == 0ull && l.addr == 0ull) return false;
+        const uint4 f = (l.len & kLongReady) ? l.f : load_run16(reinterpret_cast<const uint8_t *>(l.addr), 16);
+        k = count_key(l.cnt, be_half(f.x, f.y), be_half(f.z, f.w));
+        tie = (uint32_t)i;
+        return true;
+    }
+};
+
+template <class J>
+__global__ void __launch_bounds__(kBktThreads) k_bucket_sample(J job) {
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    const FinishJob &j = job.get();
+    if (blockIdx.x >= j.s.groups) return;
+    bucket_sample(j.s, TableSource{j});
+}
+
+template <class J>
+__global__ void __launch_bounds__(kRankThreads) k_bucket_rank(J job) {
+    extern __shared__ __align__(16) uint8_t bsm[];
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    const FinishJob &j = job.get();
+    if (blockIdx.x < j.s.rank_blocks) bucket_rank(j.s, bsm, TableSource{j}.cap());
+}
+
+// Scans the three tables once: every entry goes to its bucket, long words'
+// bytes to the arena, the totals to the metadata.  Bound by L2 (the tables are
+// read once, 20 bytes an entry written) and by the splitter search (11 steps of
+// 16 bytes from shared memory an entry).
+constexpr int kScatterThreads = 512;
+constexpr int kScatterPerSm = 2;
+template <class J>
+__global__ void __launch_bounds__(kScatterThreads, kScatterPerSm) k_bucket_scatter(J job) {
+    extern __shared__ __align__(16) uint8_t bsm[];
+    __shared__ unsigned long long tot[6];  // entries (8-byte, 16-byte, long), tokens, word bytes
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    const FinishJob &j = job.get();
+    if (threadIdx.x < 6) tot[threadIdx.x] = 0ull;
+    SlotQueue q = slot_queue(bsm);
+    const Splitters sp = load_splitters(j.s, bsm + slot_queue_smem(kScatterThreads));
+    const unsigned long long step = (unsigned long long)gridDim.x * kScatterThreads * kScanUnroll;
+    const unsigned long long b0 = (unsigned long long)blockIdx.x * kScatterThreads * kScanUnroll;
+    unsigned long long n8 = 0, n16 = 0, nl = 0, tok = 0, bytes = 0;
+    auto make = [&](const uint4 &k, unsigned long long c) -> Key128 {
+        const unsigned long long khi = be_half(k.x, k.y), klo = be_half(k.z, k.w);
+        if (klo) n16++;
+        else n8++;
+        tok += c;
+        bytes += short_len(khi, klo);
+        return count_key(c, khi, klo);
+    };
+    for (unsigned long long b = b0; b < j.cap8; b += step) {  // block-uniform
+        ulonglong2 v[kScanUnroll];
+#pragma unroll
+        for (int u = 0; u < kScanUnroll; u++) {
+            const unsigned long long i = b + (unsigned long long)u * kScatterThreads + threadIdx.x;
+            v[u] = i < j.cap8 ? *reinterpret_cast<const ulonglong2 *>(&j.g.slots8[i]) : make_ulonglong2(0ull, 0ull);
+        }
+#pragma unroll
+        for (int u = 0; u < kScanUnroll; u++)
+            q.push(j.s, sp, v[u].x != 0ull, make_uint4((uint32_t)v[u].x, (uint32_t)(v[u].x >> 32), 0u, 0u), v[u].y, make);
+    }
+    for (unsigned long long b = b0; b < j.cap16; b += step) {
+        uint4 k[kScanUnroll];
+        unsigned long long c[kScanUnroll];
+#pragma unroll
+        for (int u = 0; u < kScanUnroll; u++) {
+            const unsigned long long i = b + (unsigned long long)u * kScatterThreads + threadIdx.x;
+            k[u] = make_uint4(0, 0, 0, 0);
+            c[u] = 0;
+            if (i < j.cap16) {
+                k[u] = j.g.slots[i].key;
+                c[u] = j.g.slots[i].cnt;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kScanUnroll; u++) q.push(j.s, sp, !key_zero(k[u]), k[u], c[u], make);
+    }
+    q.flush(j.s, sp, make);
+    long_slots_body(j.g.lslots, j.lcap, j.out, blockIdx.x, gridDim.x,
+                    [&](unsigned long long slot, uint32_t, bool occ, unsigned long long khi, unsigned long long klo,
+                        unsigned long long c, uint32_t lref, uint32_t, unsigned long long len) {
+                        if (!occ) return;
+                        nl++;
+                        tok += c;
+                        bytes += len;
+                        bucket_put(j.s, sp, count_key(c, khi, klo), (uint32_t)slot, lref);
+                    });
+    for (int d = 16; d; d >>= 1) {
+        n8 += __shfl_xor_sync(kFull, n8, d);
+        n16 += __shfl_xor_sync(kFull, n16, d);
+        nl += __shfl_xor_sync(kFull, nl, d);
+        tok += __shfl_xor_sync(kFull, tok, d);
+        bytes += __shfl_xor_sync(kFull, bytes, d);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (n8) atomicAdd(&tot[0], n8);
+        if (n16) atomicAdd(&tot[1], n16);
+        if (nl) atomicAdd(&tot[2], nl);
+        if (tok) atomicAdd(&tot[3], tok);
+        if (bytes) atomicAdd(&tot[4], bytes);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && tot[0] + tot[1] + tot[2]) {
+        unsigned long long *meta = j.out.d_meta;
+        atomicAdd(&meta[0], tot[0] + tot[1] + tot[2]);
+        atomicAdd(&meta[3], tot[3]);
+        atomicAdd(&meta[4], tot[4]);
+        if (tot[0]) atomicAdd(&meta[5], tot[0]);
+        if (tot[1]) atomicAdd(&meta[6], tot[1]);
+    }
+    bucket_close(j.s);
+}
+
+__device__ __forceinline__ void put_row(const DevTable &out, unsigned long long row, const Key128 &k, uint32_t lref) {
+    unsigned long long khi, klo;
+    key_prefix(k, khi, klo);
+    out.khi[row] = khi;
+    out.klo[row] = klo;
+    out.lref[row] = lref;
+    if (out.count_bits == 32) static_cast<uint32_t *>(out.cnt)[row] = (uint32_t)key_count(k);
+    else static_cast<unsigned long long *>(out.cnt)[row] = key_count(k);
+}
+
+template <class J>
+__global__ void __launch_bounds__(kBktSortThreads, kBktSortPerSm) k_bucket_sort(J job) {
+    extern __shared__ __align__(16) uint8_t bsm[];
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    const FinishJob &j = job.get();
+    if (blockIdx.x >= j.s.buckets()) return;
+    bucket_sort(
+        j.s, *reinterpret_cast<BucketShared *>(bsm),
+        [&](unsigned long long base, uint32_t m, auto &&row) {
+            for (uint32_t i = threadIdx.x; i < m; i += kBktSortThreads) {
+                Key128 k;
+                uint32_t r;
+                row(i, k, r);
+                put_row(j.out, base + i, k, r);
+            }
+        },
+        [&](unsigned long long row, const Key128 &k, uint32_t r) { put_row(j.out, row, k, r); });
+}
+
+// Runs of equal count and prefix (only words of 17+ letters, and one of 16,
+// share a prefix) ordered by their remaining bytes: the rows of a run differ
+// in lref alone.  The first long row of a run sorts it by insertion; returns
+// at once when the bucket sort saw no two equal keys.
+template <class J>
+__global__ void k_fix_rows(J job) {
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    const FinishJob &j = job.get();
+    if (!j.s.state[kBktTied]) return;
+    const DevTable &t = j.out;
+    const unsigned long long n = t.d_meta[0];
+    const LongView v{t.lref, t.loff, t.llen, t.arena};
+    auto same = [&](unsigned long long a, unsigned long long b) {
+        if (t.khi[a] != t.khi[b] || t.klo[a] != t.klo[b]) return false;
+        return t.count_bits == 32 ? static_cast<const uint32_t *>(t.cnt)[a] == static_cast<const uint32_t *>(t.cnt)[b]
+                                  : static_cast<const unsigned long long *>(t.cnt)[a] ==
+                                        static_cast<const unsigned long long *>(t.cnt)[b];
+    };
+    for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (unsigned long long)gridDim.x * blockDim.x) {
+        // the last row of a run sorts it (a run holds at most one row without a long reference)
+        if (i == 0 || (i + 1 < n && same(i, i + 1)) || !same(i - 1, i)) continue;
+        unsigned long long lo = i - 1;
+        while (lo > 0 && same(lo - 1, i)) lo--;
+        for (unsigned long long a = lo + 1; a <= i; a++) {
+            const uint32_t x = t.lref[a];
+            unsigned long long b = a;
+            while (b > lo && lref_less(v, x, t.lref[b - 1])) { t.lref[b] = t.lref[b - 1]; b--; }
+            t.lref[b] = x;
+        }
+    }
+}
+
+// sample, rank, scatter, sort, fix-up
+constexpr int kBucketLaunches = 5;
+
+// most: the largest table's scratch.
+template <class J>
+static cudaError_t launch_buckets(const J &job, const BucketScratch &most, uint64_t cap, int ntab, cudaStream_t st) {
+    const int sms = sm_count();
+    const size_t smem = splitters_smem(most);
+    const uint32_t groups = most.groups;
+    cudaError_t e = ensure_smem_limit((const void *)k_bucket_rank<J>, (int)kept_smem(kBktGroups));
+    if (e == cudaSuccess) e = ensure_smem_limit((const void *)k_bucket_scatter<J>, (int)(kSplittersMax + slot_queue_smem(kScatterThreads)));
+    if (e == cudaSuccess) e = ensure_smem_limit((const void *)k_bucket_sort<J>, (int)sizeof(BucketShared));
+    if (e != cudaSuccess) return e;
+    launch_dependent(k_bucket_sample<J>, dim3(groups, ntab), dim3(kBktThreads), 0, st, job);
+    launch_dependent(k_bucket_rank<J>, dim3(groups, ntab), dim3(kRankThreads), kept_smem(groups), st, job);
+    launch_dependent(k_bucket_scatter<J>, dim3(grid_for(cap, kScatterThreads * kScanUnroll, sms * kScatterPerSm), ntab),
+                     dim3(kScatterThreads), smem + slot_queue_smem(kScatterThreads), st, job);
+    launch_dependent(k_bucket_sort<J>, dim3(most.buckets(), ntab), dim3(kBktSortThreads), sizeof(BucketShared), st, job);
+    launch_dependent(k_fix_rows<J>, dim3(grid_for(cap, 256, sms), ntab), dim3(256), 0, st, job);
     return cudaGetLastError();
 }
 
-size_t finish_tables_job_bytes(int n) { return sizeof(SortJob) * (size_t)(n > 0 ? n : 1); }
-int finish_tables_launches(int n, uint64_t cap, uint32_t skip) {
-    return 2 * n + sort_entries_launches(kPasses, cap, skip) + 1;
+bool finish_by_buckets(const BucketScratch &bs, uint32_t skip) {
+    return bs.key && ((skip >> (kSortKeyPasses + 6)) & 3u) == 3u;
+}
+
+int finish_table_launches(const SortScratch &ss, const BucketScratch &bs, uint32_t skip) {
+    if (finish_by_buckets(bs, skip)) return kBucketLaunches;
+    return 2 + sort_entries_launches(kPasses, ss.cap, skip) - 1 + 1;
+}
+
+cudaError_t finish_table(const GTable &g, uint64_t gcap8, uint64_t gcap, uint64_t glcap, SortScratch &ss,
+                         const BucketScratch &bs, DevTable &out, cudaStream_t st, uint32_t skip) {
+    if (finish_by_buckets(bs, skip))
+        return launch_buckets(OneFinish{FinishJob{g, gcap8, gcap, glcap, bs, out}}, bs, gcap8 + gcap + glcap, 1, st);
+    finish_by_radix(g, gcap8, gcap, glcap, ss, out, st, skip);
+    return cudaGetLastError();
+}
+
+size_t finish_tables_job_bytes(int n) { return sizeof(FinishJob) * (size_t)(n > 0 ? n : 1); }
+
+static bool all_by_buckets(const FinishSpec *spec, int n, uint32_t skip) {
+    for (int t = 0; t < n; t++)
+        if (!finish_by_buckets(*spec[t].bs, skip)) return false;
+    return true;
+}
+
+int finish_tables_launches(const FinishSpec *spec, int n, uint32_t skip) {
+    if (all_by_buckets(spec, n, skip)) return kBucketLaunches;
+    int k = 0;
+    for (int t = 0; t < n; t++) k += finish_table_launches(*spec[t].ss, *spec[t].bs, skip);
+    return k;
 }
 
 cudaError_t finish_tables(const FinishSpec *spec, int n, void *d_jobs, cudaStream_t st, uint32_t skip) {
     if (n <= 0) return cudaSuccess;
-    std::vector<SortJob> jobs((size_t)n);
+    if (!all_by_buckets(spec, n, skip)) {
+        for (int t = 0; t < n; t++) {
+            const FinishSpec &f = spec[t];
+            const cudaError_t e = finish_table(f.g, f.gcap8, f.gcap, f.glcap, *f.ss, *f.bs, *f.out, st, skip);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
+    std::vector<FinishJob> jobs((size_t)n);
     uint64_t cap = 0;
+    const BucketScratch *most = spec[0].bs;
     for (int t = 0; t < n; t++) {
         const FinishSpec &f = spec[t];
-        launch_compaction(f.g, f.gcap8, f.gcap, f.glcap, *f.ss, *f.out, st, kPrepNone);
-        jobs[t] = SortJob{*f.ss, f.out->d_meta, LongView{f.ss->lref, f.out->loff, f.out->llen, f.out->arena}, *f.out};
-        cap = std::max<uint64_t>(cap, f.ss->cap);
+        jobs[t] = FinishJob{f.g, f.gcap8, f.gcap, f.glcap, *f.bs, *f.out};
+        cap = std::max<uint64_t>(cap, f.gcap8 + f.gcap + f.glcap);
+        if (f.bs->groups > most->groups) most = f.bs;
     }
-    cudaError_t e = cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(SortJob) * jobs.size(), cudaMemcpyHostToDevice, st);
+    const cudaError_t e =
+        cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(FinishJob) * jobs.size(), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return e;
-    JobList list{static_cast<const SortJob *>(d_jobs)};
-    launch_sort(list, cap, n, kPasses, skip, st);
-    launch_dependent(k_gather_final<JobList>, dim3(grid_for(cap, 256 * kScanUnroll, sm_count() * 8), n), dim3(256), 0,
-                     st, list);
-    return cudaGetLastError();
+    return launch_buckets(FinishList{static_cast<const FinishJob *>(d_jobs)}, *most, cap, n, st);
 }
 
 // ---------------------------------------------------------------- merge
