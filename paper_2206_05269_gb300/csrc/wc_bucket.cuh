@@ -107,11 +107,16 @@ __device__ __forceinline__ void bucket_sample(const BucketScratch &s, const Sour
     if (keep > v) keep = v;
     __shared__ ulonglong2 key[kBktKeep];
     __shared__ uint32_t tie[kBktKeep];
+    // evenly spaced among those found (the first ones would all lie at the table's
+    // start, which is no random place when the slots are rows in count order)
 #pragma unroll
     for (int r = 0; r < kPer; r++)
-        if (at[r] < keep) {
-            key[at[r]] = make_ulonglong2(k[r].hi, k[r].lo);
-            tie[at[r]] = e[r];
+        if (at[r] < v) {
+            const uint32_t m = at[r] * keep / v;
+            if (at[r] == 0u || (at[r] - 1u) * keep / v != m) {
+                key[m] = make_ulonglong2(k[r].hi, k[r].lo);
+                tie[m] = e[r];
+            }
         }
     if (t == 0) s.found[g] = make_uint2(v, keep);
     __syncthreads();
