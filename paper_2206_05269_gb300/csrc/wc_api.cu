@@ -432,6 +432,8 @@ wc_status table_sync(const wc_table *ct) {
     t->nlong = meta[1];
     t->tokens = meta[3];
     t->word_bytes = meta[4];
+    t->n8 = meta[5];
+    t->n16 = meta[6];
     t->status_bits = status;
     t->sync_status = status_from_bits(status);
     if (t->sync_status != WC_OK) {
@@ -754,7 +756,7 @@ wc_status wc_merge(wc_ctx *ctx, const wc_table *const *in, uint32_t n, cudaStrea
     if (!ctx || !out || (n && !in)) return WC_ERR_INVALID_ARG;
     *out = nullptr;
     cudaSetDevice(ctx->device);
-    uint64_t sum_cap = 0, sum_lcap = 0, sum_arena = 0, chunks = 0, max_tokens = 0;
+    uint64_t sum8 = 0, sum16 = 0, sum_lcap = 0, sum_arena = 0, chunks = 0, max_tokens = 0;
     std::vector<MergeSrc> src(n);
     std::vector<uint64_t> cstart(n + 1, 0);
     for (uint32_t i = 0; i < n; i++) {
@@ -764,19 +766,21 @@ wc_status wc_merge(wc_ctx *ctx, const wc_table *const *in, uint32_t n, cudaStrea
                           d.arena_cap};
         // a table already waited for gives its sizes, any other its capacities
         const bool known = in[i]->synced && in[i]->sync_status == WC_OK;
-        sum_cap += known ? in[i]->n : d.cap;
+        const bool kinds = known && in[i]->n8 + in[i]->n16 + in[i]->nlong == in[i]->n;  // told apart by key size
+        sum8 += kinds ? in[i]->n8 : (known ? in[i]->n : d.cap);
+        sum16 += kinds ? in[i]->n16 : (known ? in[i]->n : d.cap);
         sum_lcap += known ? in[i]->nlong : d.lcap;
         sum_arena += known ? in[i]->word_bytes + in[i]->nlong : d.arena_cap;
         const uint64_t tok = known ? in[i]->tokens : in[i]->max_tokens;
         max_tokens = tok > UINT64_MAX - max_tokens ? UINT64_MAX : max_tokens + tok;
         cstart[i] = chunks;
-        chunks += (d.cap + kMergeChunk - 1) / kMergeChunk;
+        chunks += ((known ? in[i]->n : d.cap) + kMergeChunk - 1) / kMergeChunk;
         cudaStreamWaitEvent(stream, in[i]->done, 0);
     }
     cstart[n] = chunks;
     CapPlan plan;
-    plan.cap8 = pow2_at_least(std::max<uint64_t>(1024, 2 * sum_cap));
-    plan.cap16 = plan.cap8;
+    plan.cap8 = pow2_at_least(std::max<uint64_t>(1024, 2 * sum8));
+    plan.cap16 = pow2_at_least(std::max<uint64_t>(1024, 2 * sum16));
     plan.caplong = pow2_at_least(std::max<uint64_t>(256, 2 * sum_lcap));
     plan.arena = std::max<uint64_t>(4096, sum_arena);
     CountScratch cs;

@@ -66,6 +66,7 @@ struct wc_table {
     bool synced = false;
     wc_status sync_status = WC_OK;
     uint64_t n = 0, nlong = 0, tokens = 0, word_bytes = 0;
+    uint64_t n8 = 0, n16 = 0;  // words of at most 8 and of 9..16 letters (0 when the table does not tell)
     uint32_t status_bits = 0;
     uint64_t max_tokens = UINT64_MAX;  // no count of this table, nor their sum, exceeds it
     uint64_t src_bytes = 0;  // input size of a single-document count (capacity hints)

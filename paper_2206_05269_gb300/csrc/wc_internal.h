@@ -299,7 +299,7 @@ struct MergeSrc {
 };
 cudaError_t launch_merge_insert(const MergeSrc *d_src, const uint64_t *h_chunk_start, uint32_t nsrc,
                                 uint64_t total_chunks, const GTable &g, cudaStream_t s);
-constexpr int kMergeChunk = 1024;
+constexpr int kMergeChunk = 256;  // rows a merge block inserts, one a thread
 
 cudaError_t launch_topk_copy(const DevTable &in, uint64_t k, DevTable &out, cudaStream_t s);
 
