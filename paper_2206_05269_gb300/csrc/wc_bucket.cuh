@@ -107,15 +107,19 @@ __device__ __forceinline__ void bucket_sample(const BucketScratch &s, const Sour
     if (keep > v) keep = v;
     __shared__ ulonglong2 key[kBktKeep];
     __shared__ uint32_t tie[kBktKeep];
-    // evenly spaced among those found (the first ones would all lie at the table's
-    // start, which is no random place when the slots are rows in count order)
+    // evenly spaced among those found, each block's starting at its own phase:
+    // where the slots are rows in order (a vocabulary's source), the blocks' kept
+    // places together are spread evenly too (golden-ratio steps: neighbouring
+    // blocks read neighbouring slots)
+    const uint32_t phase = ((g * 0x9E3779B9u >> 16) * v) >> 16;
 #pragma unroll
     for (int r = 0; r < kPer; r++)
         if (at[r] < v) {
-            const uint32_t m = at[r] * keep / v;
-            if (at[r] == 0u || (at[r] - 1u) * keep / v != m) {
-                key[m] = make_ulonglong2(k[r].hi, k[r].lo);
-                tie[m] = e[r];
+            const uint32_t x = at[r] * keep + phase, m = x / v;
+            if (x < keep || (x - keep) / v != m) {
+                const uint32_t i = m - (phase < keep ? 0u : 1u);
+                key[i] = make_ulonglong2(k[r].hi, k[r].lo);
+                tie[i] = e[r];
             }
         }
     if (t == 0) s.found[g] = make_uint2(v, keep);
