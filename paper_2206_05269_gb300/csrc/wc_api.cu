@@ -51,6 +51,7 @@ wc_status wc_ctx::alloc(void **p, size_t bytes, cudaStream_t s) {
     bytes = (bytes + 255) & ~(size_t)255;
     // reserve the bytes against the budget first (compare-and-swap: two
     // callers can never both pass a budget that holds only one of them)
+    collect(budget && used.load() + bytes > budget);
     uint64_t cur = used.load();
     do {
         if (budget && cur + bytes > budget) return fail(WC_ERR_BUDGET, "allocation over the context budget");
@@ -67,23 +68,12 @@ wc_status wc_ctx::alloc(void **p, size_t bytes, cudaStream_t s) {
     }
     return WC_OK;
 }
-namespace {
-struct ReleaseArg {
-    wc_ctx *ctx;
-    size_t bytes;
-};
-void CUDART_CB release_done(void *a) {  // runs once the stream has passed the free
-    ReleaseArg *r = static_cast<ReleaseArg *>(a);
-    r->ctx->used -= r->bytes;
-    delete r;
-}
-}  // namespace
-
 // Stream-ordered free: the bytes stay charged to the budget until the stream
-// has passed the free (a host callback after it), because work enqueued
-// before it may still use them.  While the stream is being captured into a
-// graph the charge is dropped at once (the graph's own allocation and free
-// nodes balance on every replay).
+// has passed the free (an event behind it), because work enqueued before it may
+// still use them.  (A host callback took them off the charge before: the
+// stream's next work waited for it, tens of microseconds a small count.)
+// While the stream is being captured into a graph the charge is dropped at once
+// (the graph's own allocation and free nodes balance on every replay).
 void wc_ctx::release(void *p, size_t bytes, cudaStream_t s) {
     if (!p) return;
     if (bytes == 0) bytes = 256;
@@ -95,12 +85,42 @@ void wc_ctx::release(void *p, size_t bytes, cudaStream_t s) {
         cap = cudaStreamCaptureStatusActive;  // unknown: do not defer
     }
     if (cap == cudaStreamCaptureStatusNone) {
-        ReleaseArg *r = new ReleaseArg{this, bytes};
-        if (cudaLaunchHostFunc(s, release_done, r) == cudaSuccess) return;
+        cudaEvent_t ev = nullptr;
+        if (!spare_events.empty()) {
+            ev = spare_events.back();
+            spare_events.pop_back();
+        } else if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
+            ev = nullptr;
+        }
+        if (ev && cudaEventRecord(ev, s) == cudaSuccess) {
+            freed.push_back(Freed{ev, bytes});
+            if (freed.size() > 1024) collect(true);
+            return;
+        }
         cudaGetLastError();
-        delete r;
+        if (ev) cudaEventDestroy(ev);
     }
     used -= bytes;
+}
+
+void wc_ctx::collect(bool all) {
+    auto passed = [&](const Freed &f) {
+        const cudaError_t e = cudaEventQuery(f.ev);
+        if (e == cudaErrorNotReady) {
+            cudaGetLastError();
+            return false;
+        }
+        if (e != cudaSuccess) cudaGetLastError();  // the stream or device failed: nothing will use the bytes
+        used -= f.bytes;
+        spare_events.push_back(f.ev);
+        return true;
+    };
+    while (!freed.empty() && passed(freed.front())) freed.pop_front();
+    if (!all) return;
+    for (size_t i = 0; i < freed.size();) {
+        if (passed(freed[i])) freed.erase(freed.begin() + (long)i);
+        else i++;
+    }
 }
 
 void wc_ctx::prof_mark(std::vector<cudaEvent_t> &v, cudaStream_t s) {
@@ -246,6 +266,9 @@ void wc_destroy(wc_ctx *ctx) {
     cudaSetDevice(ctx->device);
     cudaDeviceSynchronize();
     prof_clear(ctx);
+    ctx->collect(true);
+    for (auto &f : ctx->freed) cudaEventDestroy(f.ev);
+    for (auto e : ctx->spare_events) cudaEventDestroy(e);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     if (ctx->meta_host) cudaFreeHost(ctx->meta_host);
     cudaMemPoolDestroy(ctx->pool);
@@ -300,6 +323,8 @@ wc_status wc_buffer_free(wc_ctx *ctx, void *p, uint64_t bytes, cudaStream_t stre
 
 wc_status wc_mem_usage(wc_ctx *ctx, uint64_t *used, uint64_t *peak, int reset) {
     if (!ctx) return WC_ERR_INVALID_ARG;
+    cudaSetDevice(ctx->device);
+    ctx->collect(true);
     const uint64_t u = ctx->used.load();
     if (used) *used = u;
     if (peak) *peak = ctx->peak.load();
@@ -334,7 +359,7 @@ wc_status wc_selftest_wait(wc_ctx *ctx, uint32_t polls, int arrive, cudaStream_t
 // ---------------------------------------------------------------- tables
 static size_t table_bytes(uint64_t cap, uint64_t lcap, uint64_t arena, int bits) {
     auto r = [](size_t n) { return (n + 255) & ~(size_t)255; };
-    return r(8 * 8) + r(4) + r(cap * 8) * 2 + r(cap * (bits / 8)) + r(cap * 4) + r(lcap * 8) * 2 + r(arena);
+    return r(8 * 8 + 4) + r(cap * 8) * 2 + r(cap * (bits / 8)) + r(cap * 4) + r(lcap * 8) * 2 + r(arena);
 }
 
 wc_status table_create(wc_ctx *ctx, uint64_t cap, uint64_t lcap, uint64_t arena, int bits, cudaStream_t s,
@@ -351,8 +376,8 @@ wc_status table_create(wc_ctx *ctx, uint64_t cap, uint64_t lcap, uint64_t arena,
     d.lcap = lcap;
     d.arena_cap = arena;
     d.count_bits = bits;
-    d.d_meta = reinterpret_cast<unsigned long long *>(take(8 * 8));
-    d.d_status = reinterpret_cast<uint32_t *>(take(4));
+    d.d_meta = reinterpret_cast<unsigned long long *>(take(8 * 8 + 4));  // metadata, then the status word
+    d.d_status = reinterpret_cast<uint32_t *>(d.d_meta + 8);
     d.khi = reinterpret_cast<unsigned long long *>(take(cap * 8));
     d.klo = reinterpret_cast<unsigned long long *>(take(cap * 8));
     d.cnt = take(cap * (bits / 8));
@@ -360,7 +385,7 @@ wc_status table_create(wc_ctx *ctx, uint64_t cap, uint64_t lcap, uint64_t arena,
     d.loff = reinterpret_cast<unsigned long long *>(take(lcap * 8));
     d.llen = reinterpret_cast<unsigned long long *>(take(lcap * 8));
     d.arena = take(arena);
-    cudaMemsetAsync(t->mem, 0, 512, s);  // meta + status
+    cudaMemsetAsync(t->mem, 0, 68, s);  // meta + status
     t->stream = s;
     cudaEventCreateWithFlags(&t->done, cudaEventDisableTiming);
     *out = t;
@@ -398,8 +423,9 @@ void table_mark_done(wc_table *t, cudaStream_t s) {
     if (t->meta_slot < 0) t->meta_slot = t->ctx->meta_take();
     if (t->meta_slot >= 0) {
         uint8_t *h = t->ctx->meta_host + (size_t)t->meta_slot * wc_ctx::kMetaSlotBytes;
-        cudaMemcpyAsync(h, t->dt.d_meta, 64, cudaMemcpyDeviceToHost, s);
-        cudaMemcpyAsync(h + 64, t->dt.d_status, 4, cudaMemcpyDeviceToHost, s);
+        const bool together = t->dt.d_status == reinterpret_cast<uint32_t *>(t->dt.d_meta + 8);
+        cudaMemcpyAsync(h, t->dt.d_meta, together ? 68 : 64, cudaMemcpyDeviceToHost, s);
+        if (!together) cudaMemcpyAsync(h + 64, t->dt.d_status, 4, cudaMemcpyDeviceToHost, s);
     }
     cudaEventRecord(t->done, s);
 }
@@ -481,7 +507,8 @@ wc_status wc_table_export(const wc_table *t, uint8_t *h_words, uint64_t *h_word_
     // the counts go to the host on the context's copy stream while the word
     // bytes and offsets are built on `stream` (overlapped when h_counts is pinned)
     cudaEvent_t ev[2] = {nullptr, nullptr};
-    const bool side = h_counts && n && (h_words || h_word_offsets) &&
+    // (not for small tables: the events cost more than the overlap gives)
+    const bool side = h_counts && n * (d.count_bits / 8) >= (1u << 20) && (h_words || h_word_offsets) &&
                       (ctx->copy_stream || cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) ==
                                                cudaSuccess) &&
                       cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming) == cudaSuccess &&
@@ -507,27 +534,18 @@ wc_status wc_table_export(const wc_table *t, uint8_t *h_words, uint64_t *h_word_
         return st;
     };
     if (h_words || h_word_offsets) {
-        size_t sb = export_scratch_bytes(d.cap);
-        size_t wb = t->word_bytes ? t->word_bytes : 1;
-        void *scratch = nullptr, *dwords = nullptr, *doffs = nullptr;
-        if ((s = ctx->alloc(&scratch, sb, stream)) != WC_OK) return abandon(s);
-        if ((s = ctx->alloc(&dwords, wb, stream)) != WC_OK) {
-            ctx->release(scratch, sb, stream);
-            return abandon(s);
-        }
-        if ((s = ctx->alloc(&doffs, (d.cap + 1) * 8, stream)) != WC_OK) {
-            ctx->release(scratch, sb, stream);
-            ctx->release(dwords, wb, stream);
-            return abandon(s);
-        }
-        e = launch_export(d, scratch, static_cast<uint8_t *>(dwords), static_cast<unsigned long long *>(doffs), stream);
+        auto r = [](size_t x) { return (x + 255) & ~(size_t)255; };
+        const size_t sb = r(export_scratch_bytes(n)), wb = r(t->word_bytes ? t->word_bytes : 1), ob = r((n + 1) * 8);
+        void *mem = nullptr;  // scan scratch, word bytes, offsets
+        if ((s = ctx->alloc(&mem, sb + wb + ob, stream)) != WC_OK) return abandon(s);
+        uint8_t *dwords = static_cast<uint8_t *>(mem) + sb;
+        unsigned long long *doffs = reinterpret_cast<unsigned long long *>(dwords + wb);
+        e = launch_export(d, n, mem, dwords, doffs, stream);
         if (e == cudaSuccess && h_words && t->word_bytes)
             e = cudaMemcpyAsync(h_words, dwords, t->word_bytes, cudaMemcpyDeviceToHost, stream);
         if (e == cudaSuccess && h_word_offsets)
             e = cudaMemcpyAsync(h_word_offsets, doffs, (n + 1) * 8, cudaMemcpyDeviceToHost, stream);
-        ctx->release(scratch, sb, stream);
-        ctx->release(dwords, wb, stream);
-        ctx->release(doffs, (d.cap + 1) * 8, stream);
+        ctx->release(mem, sb + wb + ob, stream);
     }
     if (side) cudaStreamWaitEvent(stream, ev[1], 0);
     const cudaError_t es = cudaStreamSynchronize(stream);

@@ -96,10 +96,9 @@ static wc_status batch_sync(const wc_batch *cb) {
     if (b->synced) return b->sync_status;
     cudaError_t e = cudaEventSynchronize(b->done);
     if (e != cudaSuccess) return b->ctx->cuda_fail(e, "batch sync");
-    unsigned long long meta[4];
-    uint32_t st = 0;
-    e = cudaMemcpy(meta, b->args.meta, sizeof(meta), cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) e = cudaMemcpy(&st, b->args.status, 4, cudaMemcpyDeviceToHost);
+    unsigned long long meta[9];  // the status word follows the metadata
+    e = cudaMemcpy(meta, b->args.meta, 68, cudaMemcpyDeviceToHost);
+    const uint32_t st = (uint32_t)meta[8];
     if (e != cudaSuccess) return b->ctx->cuda_fail(e, "batch metadata");
     b->entries = meta[0];
     b->sync_status = WC_OK;
@@ -259,15 +258,15 @@ static wc_status batch_alloc(wc_batch *b, cudaStream_t stream) {
     auto r = [](size_t n) { return (n + 255) & ~(size_t)255; };
     const size_t nd = std::max<uint32_t>(b->ndocs, 1);
     const uint64_t out_cap = b->args.out_cap, lcap = b->args.lcap, arena_cap = b->args.arena_cap;
-    b->bytes = r(64) + r(16) + r(out_cap * 8) * 2 + r(out_cap * 4) * 2 + r(nd * 8) + r(nd * 4) * 2 + r(lcap * 8) * 2 +
+    b->bytes = r(64 + 16) + r(out_cap * 8) * 2 + r(out_cap * 4) * 2 + r(nd * 8) + r(nd * 4) * 2 + r(lcap * 8) * 2 +
                r(arena_cap) + r(nd * 4);
     wc_status st = ctx->alloc(&b->mem, b->bytes, stream);
     if (st != WC_OK) return st;
     uint8_t *p = static_cast<uint8_t *>(b->mem);
     auto take = [&](size_t n) { uint8_t *q = p; p += r(n); return q; };
     BatchArgs &a = b->args;
-    a.meta = reinterpret_cast<unsigned long long *>(take(64));
-    a.status = reinterpret_cast<uint32_t *>(take(16));
+    a.meta = reinterpret_cast<unsigned long long *>(take(64 + 16));  // metadata, then the status word
+    a.status = reinterpret_cast<uint32_t *>(a.meta + 8);
     a.out_khi = reinterpret_cast<unsigned long long *>(take(out_cap * 8));
     a.out_klo = reinterpret_cast<unsigned long long *>(take(out_cap * 8));
     a.out_cnt = reinterpret_cast<uint32_t *>(take(out_cap * 4));
@@ -315,7 +314,7 @@ static cudaError_t batch_enqueue(wc_batch *b, const uint8_t *d_text, const uint6
     const size_t nd = std::max<uint32_t>(b->ndocs, 1);
     a.text = d_text;
     a.doc_off = reinterpret_cast<const unsigned long long *>(d_offsets);
-    cudaMemsetAsync(a.meta, 0, 64 + 256, stream);
+    cudaMemsetAsync(a.meta, 0, 64 + 16, stream);
     cudaMemsetAsync(a.doc_start, 0, nd * 8, stream);
     cudaMemsetAsync(a.doc_n, 0, nd * 4, stream);
     cudaMemsetAsync(a.doc_flags, 0, nd * 4, stream);

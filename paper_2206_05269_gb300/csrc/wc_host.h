@@ -2,6 +2,7 @@
 #pragma once
 #include <atomic>
 #include <cstdint>
+#include <deque>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -15,7 +16,7 @@ struct wc_ctx {
     int device = 0;
     int sms = 1;
     uint64_t budget = 0;
-    std::atomic<uint64_t> used{0};   // device bytes the context holds (pool allocations not yet released)
+    std::atomic<uint64_t> used{0};   // device bytes the context holds (pool allocations whose free has not been seen done)
     std::atomic<uint64_t> peak{0};   // the largest `used` since creation or the last wc_mem_usage reset
     int count_bits = 64;
     int autotune = 0;
@@ -52,6 +53,16 @@ struct wc_ctx {
     wc_status cuda_fail(cudaError_t e, const char *what);
     wc_status alloc(void **p, size_t bytes, cudaStream_t s);
     void release(void *p, size_t bytes, cudaStream_t s);
+    // Stream-ordered frees still charged to `used`: each with an event recorded
+    // behind it.  collect(all) takes those whose event has passed off the charge,
+    // from the oldest to the first that has not (all: every one).
+    struct Freed {
+        cudaEvent_t ev;
+        size_t bytes;
+    };
+    std::deque<Freed> freed;
+    std::vector<cudaEvent_t> spare_events;
+    void collect(bool all);
 };
 
 struct wc_table {

@@ -1397,13 +1397,63 @@ __global__ void k_export_write(DevTable t, unsigned long long *offs, const unsig
     }
 }
 
-cudaError_t launch_export(const DevTable &t, void *scratch, uint8_t *d_words, unsigned long long *d_offs,
+// A table of at most kExportSmall rows in one block: lengths, their scan and the
+// bytes (three launches for a top-100 answer were most of its device time).
+constexpr int kExportSmall = 4096, kExportSmallThreads = 1024;
+__global__ void __launch_bounds__(kExportSmallThreads) k_export_small(DevTable t, uint32_t n, unsigned long long *offs,
+                                                                      uint8_t *words) {
+    constexpr int kPer = kExportSmall / kExportSmallThreads;
+    __shared__ unsigned long long wsum[kExportSmallThreads / 32];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, i0 = threadIdx.x * kPer;
+    unsigned long long hi[kPer], lo[kPer], len[kPer], own = 0;
+    uint32_t r[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; q++) {
+        const uint32_t i = i0 + q;
+        r[q] = i < n ? t.lref[i] : 0u;
+        hi[q] = i < n ? t.khi[i] : 0ull;
+        lo[q] = i < n ? t.klo[i] : 0ull;
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; q++) {
+        len[q] = i0 + q >= n ? 0ull : (r[q] ? t.llen[r[q] - 1] : short_len(hi[q], lo[q]));
+        own += len[q];
+    }
+    unsigned long long incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long x = __shfl_up_sync(kFull, incl, o);
+        if (lane >= (uint32_t)o) incl += x;
+    }
+    if (lane == 31u) wsum[warp] = incl;
+    __syncthreads();
+    unsigned long long run = incl - own;
+    for (uint32_t w = 0; w < warp; w++) run += wsum[w];
+#pragma unroll
+    for (int q = 0; q < kPer; q++) {
+        const uint32_t i = i0 + q;
+        if (i < n) {
+            offs[i] = run;
+            const uint8_t *p = r[q] ? t.arena + t.loff[r[q] - 1] : nullptr;
+            for (unsigned long long j = 0; j < len[q]; j++)
+                words[run + j] = p ? p[j] : (uint8_t)((j < 8 ? hi[q] >> (56 - 8 * j) : lo[q] >> (56 - 8 * (j - 8))) & 0xFF);
+        }
+        run += len[q];
+    }
+    if (threadIdx.x == kExportSmallThreads - 1) offs[n] = run;
+}
+
+cudaError_t launch_export(const DevTable &t, uint64_t n, void *scratch, uint8_t *d_words, unsigned long long *d_offs,
                           cudaStream_t s) {
+    if (n <= (uint64_t)kExportSmall) {
+        k_export_small<<<1, kExportSmallThreads, 0, s>>>(t, (uint32_t)n, d_offs, d_words);
+        return cudaGetLastError();
+    }
     unsigned long long *blocksum = static_cast<unsigned long long *>(scratch);
-    const int nb = (int)((t.cap + kScanBlock - 1) / kScanBlock);
-    k_export_lens<<<nb > 0 ? nb : 1, 256, 0, s>>>(t, d_offs, blocksum);
+    const int nb = (int)((n + kScanBlock - 1) / kScanBlock);
+    k_export_lens<<<nb, 256, 0, s>>>(t, d_offs, blocksum);
     k_export_blocksums<<<1, kBlockSumThreads, 0, s>>>(t, blocksum, d_offs);
-    k_export_write<<<grid_for(t.cap, 256, sm_count() * 8), 256, 0, s>>>(t, d_offs, blocksum, d_words);
+    k_export_write<<<grid_for(n, 256, sm_count() * 8), 256, 0, s>>>(t, d_offs, blocksum, d_words);
     return cudaGetLastError();
 }
 

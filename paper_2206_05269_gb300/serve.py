@@ -166,19 +166,21 @@ def serve_batched(counter: wc.Counter, requests: list[Request], topk: int = 100,
                 if e.status != wc.WC_ERR_BUDGET or not make_room():
                     raise
 
+    room_at = [None]  # bytes held when room was last looked for with nothing running
+
     def make_room():
         """Frees budget for a refused allocation: finishes the oldest running
         unit; with nothing running, waits for the device, since memory freed
         in stream order is charged until its stream has passed the free.
-        False when neither frees anything."""
+        False when that frees nothing more than the last time."""
         if running:
+            room_at[0] = None
             finish(running.popleft())
             return True
-        used = counter.mem_usage()[0]
-        if used:
-            torch.cuda.synchronize(dev)
-            return counter.mem_usage()[0] < used
-        return False
+        torch.cuda.synchronize(dev)
+        used, before = counter.mem_usage()[0], room_at[0]
+        room_at[0] = used
+        return before is None or used < before
 
     def finish(wk: _Work):
         wk.event.synchronize()
@@ -271,6 +273,7 @@ def serve_batched(counter: wc.Counter, requests: list[Request], topk: int = 100,
         if (small or big) and free_streams:
             stream = free_streams.popleft()
             if launch(stream):
+                room_at[0] = None
                 stats["max_running"] = max(stats["max_running"], len(running))
                 continue
             stats["budget_waits"] += 1
