@@ -132,6 +132,15 @@ __device__ __forceinline__ uint4 cas128_shared(uint4 *p, uint4 val) {  // compar
         : "memory");
     return make_uint4((uint32_t)r0, (uint32_t)(r0 >> 32), (uint32_t)r1, (uint32_t)(r1 >> 32));
 }
+// Slot hash of a word's key in a document's table (its top bits pick the slot):
+// the four 32-bit words times odd constants, summed, folded and multiplied once
+// more.  Seven instructions where a 64-bit finalizer took about thirty.
+__device__ __forceinline__ uint32_t doc_hash(uint4 k) {
+    if (kOneSlot) return 0u;
+    uint32_t h = k.x * 0x9E3779B1u + k.y * 0x85EBCA77u + k.z * 0xC2B2AE3Du + k.w * 0x27D4EB2Fu;
+    h ^= h >> 15;
+    return h * 0x2C1B3C6Du;
+}
 // Adds 1 to marked key km from home slot s; false when the word must spill
 // (the probe limit, or an empty slot found with the table filled to its limit).
 __device__ __forceinline__ bool doc_table_add(uint4 *skey, uint32_t *scnt, uint32_t *nfill, uint32_t mask,
@@ -169,10 +178,19 @@ struct DocCfg {
     static constexpr int TOKCAP = 32 + 256;
     static constexpr int LCAP = 64;            // distinct long words per document in shared memory
     static constexpr uint32_t FILL = C1 * 3 / 4;
-    static constexpr size_t SMEM = (size_t)WINB + (size_t)W * TOKCAP * 4 +  // window + queues (sort buffer)
-                                   (size_t)C1 * 16 + (size_t)C1 * 4 +  // keys, counts
+    // entries of a document: the table's fill limit, which every thread may
+    // pass by one claim, and the long words
+    static constexpr uint32_t NMAX = FILL + BLOCK + LCAP;
+    static constexpr uint32_t PARTS = C1 > 1024 ? 256 : 128;  // parts of the sort
+    // window + queues; the sort reuses them: three 16-bit lists, the coarse
+    // splitters and their ranges, the part counters
+    static constexpr size_t SORT_LISTS = (size_t)NMAX * 6;
+    static constexpr size_t SORT = SORT_LISTS + (kBktCoarse + 1) * 16 + kBktCoarse * sizeof(KeyRange) + PARTS * 4;
+    static constexpr size_t QUEUES = (size_t)WINB + (size_t)W * TOKCAP * 4;
+    static constexpr size_t AREA = ((SORT > QUEUES ? SORT : QUEUES) + 15) & ~(size_t)15;
+    static constexpr size_t SMEM = AREA + (size_t)C1 * 16 + (size_t)C1 * 4 +  // ..., keys, counts
                                    (size_t)LCAP * (8 + 8 + 4 + 4 + 16) + 16 + 64;
-    static_assert((size_t)WINB + (size_t)W * TOKCAP * 4 >= (size_t)C1 * 2, "sort buffer must fit");
+    static_assert(NMAX % 8 == 0 && BLOCK >= kBktCoarse, "16-byte aligned lists, a thread a coarse splitter");
     // blocks per SM that the shared memory allows: the register budget follows
     static constexpr int MINB = (int)((227u * 1024u) / SMEM) < 1 ? 1 : ((int)((227u * 1024u) / SMEM) > 8 ? 8 : (int)((227u * 1024u) / SMEM));
     static_assert(C1 <= 32768, "16-bit sort indices");
@@ -185,7 +203,7 @@ struct DocShared {  // per-block scalars
     uint32_t spilled;
     uint32_t nent;
     uint32_t nlong;
-    unsigned long long base, lbase, abase;
+    unsigned long long base, lbase, abase, abytes;
     uint32_t ok;
 };
 
@@ -195,8 +213,13 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
     extern __shared__ __align__(16) uint8_t smem[];
     uint8_t *win = smem;
     uint32_t *tokall = reinterpret_cast<uint32_t *>(smem + C::WINB);
-    uint16_t *sidx = reinterpret_cast<uint16_t *>(smem);  // sort buffer, reuses window + queues
-    uint4 *skey = reinterpret_cast<uint4 *>(smem + C::WINB + (size_t)C::W * C::TOKCAP * 4);
+    // the sort's lists, reusing window + queues: entries as found, their parts and
+    // then rows, entries by part and then in order
+    uint16_t *found = reinterpret_cast<uint16_t *>(smem), *prow = found + C::NMAX, *sidx = prow + C::NMAX;
+    ulonglong2 *coarse = reinterpret_cast<ulonglong2 *>(smem + C::SORT_LISTS);
+    KeyRange *range = reinterpret_cast<KeyRange *>(coarse + kBktCoarse + 1);
+    uint32_t *pcount = reinterpret_cast<uint32_t *>(range + kBktCoarse);
+    uint4 *skey = reinterpret_cast<uint4 *>(smem + C::AREA);
     uint32_t *scnt = reinterpret_cast<uint32_t *>(skey + C::C1);
     unsigned long long *laddr = reinterpret_cast<unsigned long long *>(scnt + C::C1);
     unsigned long long *llen = laddr + C::LCAP;
@@ -235,6 +258,7 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
             while (ceff < (uint32_t)C::C1 && ceff < want) ceff <<= 1;
         }
         const uint32_t fill_limit = ceff / 4u * 3u;
+        const int cshift = __clz((int)ceff) + 1;  // 32 - log2(ceff)
         for (int i = threadIdx.x; i < (int)ceff; i += BLOCK) {
             skey[i] = make_uint4(0u, 0u, 0u, 0u);
             scnt[i] = 0u;
@@ -252,7 +276,7 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
                 const uint32_t p = e >> 5, len = e & 31u;
                 uint4 k = load_key16(win, p, len);
                 if (!doc_table_add(skey, scnt, &sh.nfill, ceff - 1u, fill_limit, mark_key(k),
-                                   (uint32_t)(hash_key(k) >> 40) & (ceff - 1u), (int)ceff)) {
+                                   doc_hash(k) >> cshift, (int)ceff)) {
                     doc_insert_key(a.g, d, k, 1ull);
                     sh.spilled = 1u;
                 }
@@ -414,80 +438,145 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
                 }
             }
         }
-        // Every live entry becomes a 128-bit composite in place (its count,
-        // its 16-letter prefix packed 5 bits a letter, a long-word flag and
-        // index): integer order on composites is the output order (count
-        // desc, word asc) except among long words sharing a prefix, which a
-        // fix-up orders below.  The sort then moves 16-bit indices and
+        // The live entries' list (its order is fixed by the sort below; one shared
+        // atomic per warp and step), then each becomes a 128-bit composite in
+        // place (its count, its 16-letter prefix packed 5 bits a letter, a
+        // long-word flag and index): integer order on composites is the output
+        // order (count desc, word asc) except among long words sharing a prefix,
+        // which a fix-up orders below.  The sort then moves 16-bit indices and
         // compares composites.
         if (threadIdx.x == 0) {
             sh.nent = 0;
             sh.nlong = 0;
         }
         __syncthreads();
-        // composites in place, and the index list of live entries (its order
-        // is fixed by the sort below): one shared atomic per warp and step
         static_assert(C::C1 % BLOCK == 0, "whole steps over the shared table");
         for (int i0 = 0; i0 < (int)ceff; i0 += BLOCK) {
             const int i = i0 + threadIdx.x;
-            const uint4 km = skey[i];
-            const bool live = !key_zero(km);
-            if (live) {
-                const uint4 k = unmark_key(km);
-                reinterpret_cast<ulonglong2 *>(skey)[i] =
-                    doc_composite(be64b(k.x, k.y), be64b(k.z, k.w), scnt[i], false, 0u);
-            }
+            const bool live = scnt[i] != 0u;
             const uint32_t m = __ballot_sync(kFull, live);
             uint32_t base = 0;
             if (lane == 0 && m) base = atomicAdd(&sh.nent, (uint32_t)__popc(m));
             base = __shfl_sync(kFull, base, 0);
-            if (live) sidx[base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)i;
+            if (live) found[base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)i;
+        }
+        __syncthreads();
+        const uint32_t nshort = sh.nent;
+        for (uint32_t e = threadIdx.x; e < nshort; e += BLOCK) {
+            const uint32_t i = found[e];
+            const uint4 k = unmark_key(skey[i]);
+            reinterpret_cast<ulonglong2 *>(skey)[i] =
+                doc_composite(be64b(k.x, k.y), be64b(k.z, k.w), scnt[i], false, 0u);
         }
         for (uint32_t j = threadIdx.x; j < nl; j += BLOCK) {
             const uint8_t *p = reinterpret_cast<const uint8_t *>(laddr[j]);
             lkey[j] = doc_composite(be_bytes16(p, 0), be_bytes16(p, 8), lcnt[j], true, j);
         }
-        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < C::PARTS; i += BLOCK) pcount[i] = 0u;
+        // the long entries, and the output reserved: entries, long words, arena
+        // bytes (the atomics' round trips pass while the block sorts)
+        unsigned long long got_base = 0, got_lbase = 0, got_abase = 0;
         if (threadIdx.x == 0) {
-            uint32_t r = 0;
+            uint32_t r = 0, m = nshort;
+            unsigned long long ab = 0;
             for (uint32_t j = 0; j < nl; j++) {
-                if (lcnt[j]) { lrank[j] = r++; sidx[sh.nent++] = (uint16_t)(C::C1 + j); }
+                if (!lcnt[j]) continue;
+                lrank[j] = r++;
+                found[m++] = (uint16_t)(C::C1 + j);
+                ab += llen[j] + 1;
             }
+            sh.nent = m;
             sh.nlong = r;
+            sh.abytes = ab;
+            got_base = atomicAdd(&a.meta[0], (unsigned long long)m);
+            if (r) got_lbase = atomicAdd(&a.meta[1], (unsigned long long)r);
+            if (ab) got_abase = atomicAdd(&a.meta[2], ab);
         }
         __syncthreads();
         const uint32_t n = sh.nent;
-        uint32_t N = 1;
-        while (N < n) N <<= 1;
-        __syncthreads();
         auto key_of = [&](uint32_t s) -> ulonglong2 {
             return s < (uint32_t)C::C1 ? reinterpret_cast<const ulonglong2 *>(skey)[s] : lkey[s - C::C1];
         };
-        // Bitonic network over N = 2^m >= n positions, every merge ascending:
-        // its first stage compares each position of a block's lower half with
-        // its mirror in the upper half, the later stages with the position j
-        // above.  Positions from n on stand for entries above every real
-        // one, so a pair that reaches one never swaps and is skipped: the
-        // padding is never touched.  The pairs of thread t lie in the 64
-        // positions from 64 * (t / 32) while a stage works within blocks of
-        // at most 64, so a warp owns the same positions through consecutive
-        // such stages and only a change to or from a wider stage needs a
-        // block-wide barrier.
-        for (uint32_t k = 2; k <= N; k <<= 1) {
-            for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-                const bool mirror = j == (k >> 1);
-                for (uint32_t t = threadIdx.x; t < N / 2; t += BLOCK) {
-                    const uint32_t i = 2 * t - (t & (j - 1)), q = mirror ? (i ^ (k - 1)) : i + j;
-                    if (q >= n) continue;
-                    const uint32_t x = sidx[i], y = sidx[q];
-                    const ulonglong2 kx = key_of(x), ky = key_of(y);
-                    if (ky.x != kx.x ? ky.x < kx.x : ky.y < kx.y) { sidx[i] = (uint16_t)y; sidx[q] = (uint16_t)x; }
-                }
-                const uint32_t span = 2 * j, span_next = j > 1 ? j : 2 * k;  // block sizes of this and the next stage
-                if (span <= 64 && span_next <= 64) __syncwarp();
-                else __syncthreads();
+        // Sort: parts of a few entries (32 coarse ones between evenly spaced
+        // entries of the document, each split evenly by interpolation), then each
+        // entry's row is its part's first row plus the part's entries before it.
+        // About 200 instructions an entry; a bitonic network over the list took
+        // 500 (200 entries) to 1,800 (6,000) and a block barrier a stage.
+        uint32_t fine = 1;
+        while (fine < C::PARTS / kBktCoarse && fine * kBktCoarse * 3u < n) fine <<= 1;
+        {
+            ulonglong2 *cand = reinterpret_cast<ulonglong2 *>(sidx);
+            constexpr uint32_t kLanes = BLOCK / kBktCoarse;  // threads that rank one candidate
+            if (threadIdx.x + 1 < (uint32_t)kBktCoarse && n) cand[threadIdx.x] = key_of(found[(threadIdx.x + 1) * n / kBktCoarse]);
+            __syncthreads();
+            const uint32_t i = threadIdx.x / kLanes;
+            uint32_t r = 0;
+            if (i + 1 < (uint32_t)kBktCoarse) {
+                const ulonglong2 k = cand[i];
+                for (uint32_t j = threadIdx.x % kLanes; j + 1 < (uint32_t)kBktCoarse; j += kLanes)
+                    r += row_less(cand[j], j, k, i) ? 1u : 0u;
+            }
+#pragma unroll
+            for (uint32_t o = kLanes / 2; o; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
+            if (threadIdx.x % kLanes == 0u) {
+                if (i + 1 < (uint32_t)kBktCoarse) coarse[r + 1] = cand[i];
+                else coarse[0] = make_ulonglong2(0ull, 0ull);
+            }
+            if (threadIdx.x == 0) coarse[kBktCoarse] = make_ulonglong2(~0ull, ~0ull);
+        }
+        __syncthreads();
+        if (threadIdx.x < (uint32_t)kBktCoarse) range[threadIdx.x].set(coarse[threadIdx.x], coarse[threadIdx.x + 1], fine);
+        __syncthreads();
+        for (uint32_t e = threadIdx.x; e < n; e += BLOCK) {
+            const ulonglong2 k = key_of(found[e]);
+            uint32_t c = 0;
+#pragma unroll
+            for (uint32_t step = kBktCoarse / 2; step; step >>= 1) {
+                const ulonglong2 v = coarse[c + step];
+                if (v.x != k.x ? v.x < k.x : v.y <= k.y) c += step;
+            }
+            const uint32_t q = c * fine + range[c](k);
+            prow[e] = (uint16_t)q;
+            atomicAdd(&pcount[q], 1u);
+        }
+        __syncthreads();
+        if (warp == 0) {  // counts -> first rows
+            constexpr int kPer = C::PARTS / 32;
+            uint32_t c[kPer], own = 0;
+#pragma unroll
+            for (int q = 0; q < kPer; q++) {
+                c[q] = pcount[lane * kPer + q];
+                own += c[q];
+            }
+            uint32_t incl = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t x = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += x;
+            }
+            uint32_t run = incl - own;
+#pragma unroll
+            for (int q = 0; q < kPer; q++) {
+                pcount[lane * kPer + q] = run;
+                run += c[q];
             }
         }
+        __syncthreads();
+        for (uint32_t e = threadIdx.x; e < n; e += BLOCK) sidx[atomicAdd(&pcount[prow[e]], 1u)] = found[e];
+        __syncthreads();
+        // pcount[q] is now the first row after part q
+        for (uint32_t e = threadIdx.x; e < n; e += BLOCK) {
+            const uint32_t q = prow[e], lo = q ? pcount[q - 1] : 0u, hi = pcount[q];
+            const ulonglong2 k = key_of(found[e]);
+            uint32_t rank = lo;
+            for (uint32_t i = lo; i < hi; i++) {
+                const ulonglong2 o = key_of(sidx[i]);
+                rank += (o.x != k.x ? o.x < k.x : o.y < k.y) ? 1u : 0u;
+            }
+            prow[e] = (uint16_t)rank;
+        }
+        __syncthreads();
+        for (uint32_t e = threadIdx.x; e < n; e += BLOCK) sidx[prow[e]] = found[e];
         __syncthreads();
         // long words with equal count and prefix: order by their remaining
         // bytes (insertion over each such run; runs are rare and short)
@@ -527,15 +616,11 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
             }
             __syncthreads();
         }
-        // reserve output: entries, long words, arena bytes
         if (threadIdx.x == 0) {
-            unsigned long long ab = 0;
-            for (uint32_t j = 0; j < nl; j++)
-                if (lcnt[j]) ab += llen[j] + 1;
-            sh.base = atomicAdd(&a.meta[0], (unsigned long long)n);
-            sh.lbase = sh.nlong ? atomicAdd(&a.meta[1], (unsigned long long)sh.nlong) : 0ull;
-            sh.abase = ab ? atomicAdd(&a.meta[2], ab) : 0ull;
-            sh.ok = (sh.base + n <= a.out_cap && sh.lbase + sh.nlong <= a.lcap && sh.abase + ab <= a.arena_cap);
+            sh.base = got_base;
+            sh.lbase = got_lbase;
+            sh.abase = got_abase;
+            sh.ok = (sh.base + n <= a.out_cap && sh.lbase + sh.nlong <= a.lcap && sh.abase + sh.abytes <= a.arena_cap);
             if (!sh.ok) atomicOr(a.status, ST_OUT_FULL);
             a.doc_start[d] = sh.base;
             a.doc_n[d] = sh.ok ? n : 0u;

@@ -113,22 +113,7 @@ __device__ __forceinline__ bool key_eq(uint4 a, uint4 b) {
 }
 __device__ __forceinline__ bool key_zero(uint4 a) { return (a.x | a.y | a.z | a.w) == 0u; }
 
-// 64-bit slot hash of a 16-byte key: MurmurHash3's fmix64 finalizer
-// (Appleby, public domain) over the two halves folded together.  It only picks
-// slots; equality is always decided on the full key.
-__device__ __forceinline__ uint64_t hash_key(uint4 k) {
-    if (kOneSlot) return 0ull;
-    uint64_t lo = ((uint64_t)k.y << 32) | k.x;
-    uint64_t hi = ((uint64_t)k.w << 32) | k.z;
-    uint64_t x = lo ^ (hi * 0x9E3779B97F4A7C15ull);
-    x ^= x >> 33;
-    x *= 0xFF51AFD7ED558CCDull;
-    x ^= x >> 33;
-    x *= 0xC4CEB9FE1A85EC53ull;
-    x ^= x >> 33;
-    return x;
-}
-
+// MurmurHash3's fmix64 finalizer (Appleby, public domain).
 __device__ __forceinline__ unsigned long long fmix64(unsigned long long x) {
     x ^= x >> 33;
     x *= 0xFF51AFD7ED558CCDull;
