@@ -17,7 +17,8 @@ namespace {
 
 constexpr uint64_t kSmallMax = 8 << 10;     // whole documents up to 8 KB: small shape
 constexpr uint64_t kMediumMax = 32 << 10;   // whole documents up to 32 KB: medium shape; larger: large shape
-constexpr uint64_t kSplitMin = 64 << 10;    // documents above 64 KB are split into ranges
+constexpr uint64_t kSplitMin = 64 << 10;    // documents above 64 KB may be split into ranges
+constexpr uint64_t kSplitAll = 128000;      // documents above this always are (a composite holds counts below 2^16)
 constexpr uint64_t kRange = 32 << 10;       // byte range per item of a split document
 constexpr uint32_t kMaxDocs = 1u << 24;     // (document, word) keys carry 24 document bits
 
@@ -62,7 +63,7 @@ struct wc_batch {
     // planning
     std::vector<DocItem> items;
     uint32_t nsmall = 0, nmedium = 0;  // items: small, then medium, then large
-    int shape_small = 1, shape_medium = 3, shape_large = 4;
+    int shape_small = 1, shape_medium = 3, shape_large = 5;
     uint64_t cap8 = 0, cap16 = 0, caplong = 0;
     BatchScratch scr;
     // after sync
@@ -208,6 +209,12 @@ static wc_status batch_plan(wc_ctx *ctx, const uint64_t *h_offsets, uint32_t ndo
     b->ctx = ctx;
     b->ndocs = ndocs;
     b->nclasses = nclasses;
+    // A document between the two is split when it would keep one block busy for
+    // longer than a sixteenth of an even share of the batch: its words then pass
+    // through the global (document, word) tables and the sort after them, which
+    // costs more in all than one block's shared table does.
+    const uint64_t bytes = ndocs ? h_offsets[ndocs] - h_offsets[0] : 0;
+    const uint64_t split = std::min(kSplitAll, std::max(kSplitMin, bytes / (16 * (uint64_t)ctx->sms)));
     std::vector<DocItem> small, medium, large;
     uint64_t out_est = 0, glob_est = 0, long_est = 0, total = 0;
     for (uint32_t d = 0; d < ndocs; d++) {
@@ -220,7 +227,7 @@ static wc_status batch_plan(wc_ctx *ctx, const uint64_t *h_offsets, uint32_t ndo
         b->max_doc_bytes = std::max(b->max_doc_bytes, s);
         if (s <= kSmallMax) small.push_back({lo, hi, d, 0});
         else if (s <= kMediumMax) medium.push_back({lo, hi, d, 0});
-        else if (s <= kSplitMin) large.push_back({lo, hi, d, 0});
+        else if (s <= split) large.push_back({lo, hi, d, 0});
         else {
             glob_est += e;
             for (uint64_t r = lo; r < hi; r += kRange) large.push_back({r, std::min(hi, r + kRange), d, 1});

@@ -181,10 +181,12 @@ constexpr int kBktApart = 3;     // sampled keys between two splitters at least
 constexpr int kBktMean = 384;    // entries a bucket is meant to hold
 constexpr int kBktStride = 8;    // words between two buckets' counters
 constexpr int kBktSplits = 0, kBktRoom = 1, kBktSpilled = 2, kBktTied = 3, kBktBig = 4, kBktTicket = 5;  // BucketScratch::state
-// Tables of more slots are radix sorted: there are at most 2,730 splitters (54 KB
-// of shared memory in the scatter kernels), and 8M entries would put 3,000 in a
-// bucket; from 2,560 on a block sorts in global memory.
-constexpr uint64_t kBktMaxCap = 1ull << 24;
+// Tables of more slots are radix sorted.  There are at most 2,730 splitters (54 KB
+// of shared memory in the scatter kernels); buckets of more than 2,560 entries
+// are sorted in global memory, which at 10,000 entries a bucket still takes a
+// quarter of the radix passes' time; past that the radix sort's cost an entry is
+// the smaller one.
+constexpr uint64_t kBktMaxCap = 1ull << 26;
 struct BucketScratch {
     uint32_t groups;              // sample blocks
     unsigned long long slots;     // entries `key` and `lref` hold, shared out evenly to the buckets
