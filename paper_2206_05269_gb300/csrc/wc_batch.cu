@@ -213,9 +213,9 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
     extern __shared__ __align__(16) uint8_t smem[];
     uint8_t *win = smem;
     uint32_t *tokall = reinterpret_cast<uint32_t *>(smem + C::WINB);
-    // the sort's lists, reusing window + queues: entries as found, their parts and
-    // then rows, entries by part and then in order
-    uint16_t *found = reinterpret_cast<uint16_t *>(smem), *prow = found + C::NMAX, *sidx = prow + C::NMAX;
+    // the sort's lists, reusing window + queues: entries as found (then in order),
+    // their parts, entries by part
+    uint16_t *found = reinterpret_cast<uint16_t *>(smem), *prow = found + C::NMAX, *byparts = prow + C::NMAX;
     ulonglong2 *coarse = reinterpret_cast<ulonglong2 *>(smem + C::SORT_LISTS);
     KeyRange *range = reinterpret_cast<KeyRange *>(coarse + kBktCoarse + 1);
     uint32_t *pcount = reinterpret_cast<uint32_t *>(range + kBktCoarse);
@@ -502,6 +502,7 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
         // entry's row is its part's first row plus the part's entries before it.
         // About 200 instructions an entry; a bitonic network over the list took
         // 500 (200 entries) to 1,800 (6,000) and a block barrier a stage.
+        uint16_t *sidx = byparts;
         uint32_t fine = 1;
         while (fine < C::PARTS / kBktCoarse && fine * kBktCoarse * 3u < n) fine <<= 1;
         {
@@ -522,7 +523,7 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
                 if (i + 1 < (uint32_t)kBktCoarse) coarse[r + 1] = cand[i];
                 else coarse[0] = make_ulonglong2(0ull, 0ull);
             }
-            if (threadIdx.x == 0) coarse[kBktCoarse] = make_ulonglong2(~0ull, ~0ull);
+            if (threadIdx.x == 0) coarse[kBktCoarse] = make_ulonglong2((0xFFFFull << 48) - 1ull, ~0ull);  // counts are at least 1
         }
         __syncthreads();
         if (threadIdx.x < (uint32_t)kBktCoarse) range[threadIdx.x].set(coarse[threadIdx.x], coarse[threadIdx.x + 1], fine);
@@ -564,20 +565,26 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
         __syncthreads();
         for (uint32_t e = threadIdx.x; e < n; e += BLOCK) sidx[atomicAdd(&pcount[prow[e]], 1u)] = found[e];
         __syncthreads();
-        // pcount[q] is now the first row after part q
-        for (uint32_t e = threadIdx.x; e < n; e += BLOCK) {
-            const uint32_t q = prow[e], lo = q ? pcount[q - 1] : 0u, hi = pcount[q];
-            const ulonglong2 k = key_of(found[e]);
+        // pcount[q] is now the first row after part q.  Thread and place agree (not
+        // thread and entry), so that a warp's lanes rank within the same few parts
+        // and a long part holds up only the warps that own it.
+        uint16_t *order = found;
+        for (uint32_t j = threadIdx.x; j < n; j += BLOCK) {
+            uint32_t q = 0;
+#pragma unroll
+            for (uint32_t step = C::PARTS / 2; step; step >>= 1)
+                if (pcount[q + step - 1] <= j) q += step;
+            const uint32_t lo = q ? pcount[q - 1] : 0u, hi = pcount[q], mine = sidx[j];
+            const ulonglong2 k = key_of(mine);
             uint32_t rank = lo;
             for (uint32_t i = lo; i < hi; i++) {
                 const ulonglong2 o = key_of(sidx[i]);
                 rank += (o.x != k.x ? o.x < k.x : o.y < k.y) ? 1u : 0u;
             }
-            prow[e] = (uint16_t)rank;
+            order[rank] = (uint16_t)mine;  // (the entries as found are not read any more)
         }
         __syncthreads();
-        for (uint32_t e = threadIdx.x; e < n; e += BLOCK) sidx[prow[e]] = found[e];
-        __syncthreads();
+        sidx = order;
         // long words with equal count and prefix: order by their remaining
         // bytes (insertion over each such run; runs are rare and short)
         if (sh.nlong) {

@@ -392,7 +392,8 @@ struct KeyRange {
         const unsigned long long span = window(to) - w0;
         up = (uint8_t)(span ? __clzll((long long)span) : 0);
         const unsigned long long top = (span << up) >> 32;
-        scale = span ? (uint32_t)(((unsigned long long)parts << 32) / (top + 1ull)) : 0u;
+        // at most parts * 2^32 / (top + 1): the last number is below parts (parts < 2^16)
+        scale = span ? (parts << 16) / ((uint32_t)(top >> 16) + 1u) : 0u;
     }
     __device__ __forceinline__ uint32_t operator()(const ulonglong2 &k) const {
         return __umulhi((uint32_t)(((window(k) - w0) << up) >> 32), scale);
