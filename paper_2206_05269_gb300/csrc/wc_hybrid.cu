@@ -1,10 +1,13 @@
 // The reduce of the paper's hybrid pipeline (Sec. 3.3 "Reduce on GPU",
 // measured in Sec. 4.1): the host has mapped every document to a dictionary
 // and laid the per-document counts of each word out as one row of a
-// zero-padded matrix; the GPU sums each row.  Here one warp sums one row
-// with coalesced loads and a shuffle reduction and writes one 64-bit total;
-// warps take rows in a grid-stride loop.  It reads the matrix once: bound by
-// HBM (rows x cols x 4 bytes read, rows x 8 written).
+// zero-padded matrix; the GPU sums each row.  It reads the matrix once: bound by
+// HBM (rows x cols x 4 bytes read, rows x 8 written).  One warp sums one row with
+// 16-byte loads (the row's first and last words that are not part of an aligned
+// 16 bytes by single loads), eight a lane issued before the first sum, so a row of
+// 1,000 counts is in flight at once, and a shuffle reduction; one block for every
+// eight rows, which evens out the rows better than a grid of resident blocks.
+// 30,000 x 1,000: 26.3 us with four 4-byte loads a lane in flight.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -13,17 +16,40 @@
 
 namespace wc {
 
-__global__ void k_row_sums(const uint32_t *m, unsigned long long rows, unsigned long long cols,
-                           unsigned long long *out) {
-    const int lane = threadIdx.x & 31;
+__device__ __forceinline__ uint4 ld_once16(const uint4 *p) {
+    uint4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p));
+    return v;
+}
+
+constexpr int kRowLoads = 8;  // 16-byte loads a lane has in flight
+__global__ void __launch_bounds__(256) k_row_sums(const uint32_t *m, unsigned long long rows, unsigned long long cols,
+                                                  unsigned long long *out) {
+    const uint32_t lane = threadIdx.x & 31u;
     const unsigned long long nw = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
     for (unsigned long long r = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < rows; r += nw) {
         const uint32_t *row = m + r * cols;
+        // row[0, head) up to the first 16-byte boundary, nv aligned groups of four, the rest
+        unsigned long long head = (4u - (uint32_t)(reinterpret_cast<uintptr_t>(row) >> 2)) & 3u;
+        if (head > cols) head = cols;
+        const unsigned long long nv = (cols - head) >> 2, tail = head + 4 * nv;
+        const uint4 *v = reinterpret_cast<const uint4 *>(row + head);
         unsigned long long s = 0;
-        unsigned long long c = lane;
-        for (; c + 96 < cols; c += 128)  // four independent loads in flight per lane
-            s += (unsigned long long)__ldg(row + c) + __ldg(row + c + 32) + __ldg(row + c + 64) + __ldg(row + c + 96);
-        for (; c < cols; c += 32) s += __ldg(row + c);
+        for (unsigned long long b = 0; b < nv; b += 32 * kRowLoads) {
+            uint4 x[kRowLoads];
+#pragma unroll
+            for (int q = 0; q < kRowLoads; q++) {
+                const unsigned long long i = b + 32u * q + lane;
+                x[q] = i < nv ? ld_once16(v + i) : make_uint4(0u, 0u, 0u, 0u);
+            }
+#pragma unroll
+            for (int q = 0; q < kRowLoads; q++)
+                s += ((unsigned long long)x[q].x + x[q].y) + ((unsigned long long)x[q].z + x[q].w);
+        }
+        if (lane < head) s += __ldg(row + lane);
+        if (tail + lane < cols) s += __ldg(row + tail + lane);
         for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
         if (lane == 0) out[r] = s;
     }
@@ -32,11 +58,7 @@ __global__ void k_row_sums(const uint32_t *m, unsigned long long rows, unsigned 
 cudaError_t launch_row_sums(const uint32_t *m, unsigned long long rows, unsigned long long cols,
                             unsigned long long *out, cudaStream_t s) {
     if (!rows) return cudaSuccess;
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const unsigned long long want = (rows + 7) / 8;  // 8 warps (rows) a block
-    const unsigned long long cap = (unsigned long long)(sms > 0 ? sms : 1) * 16;
+    const unsigned long long want = (rows + 7) / 8, cap = 1ull << 20;  // 8 warps (rows) a block
     k_row_sums<<<(unsigned)(want < cap ? want : cap), 256, 0, s>>>(m, rows, cols, out);
     return cudaGetLastError();
 }
