@@ -686,6 +686,8 @@ wc_status wc_count(wc_ctx *ctx, const uint8_t *d_text, uint64_t nbytes, cudaStre
 }
 
 // ---------------------------------------------------------------- counting from host memory
+constexpr uint64_t kTaperMin = 8ull << 20;  // the smallest automatic piece
+
 static bool host_letter(uint8_t b) { return (uint8_t)((b | 0x20) - 0x61) < 26 && b < 0x80; }
 
 wc_status wc_count_host(wc_ctx *ctx, const uint8_t *h_text, uint64_t nbytes, uint8_t *d_buf, uint64_t piece_bytes,
@@ -703,10 +705,18 @@ wc_status wc_count_host(wc_ctx *ctx, const uint8_t *h_text, uint64_t nbytes, uin
         return ctx->fail(WC_ERR_CUDA, "cudaStreamCreate (copy stream)");
     }
     // pieces cut where a letter is not followed by a letter: no word spans two
+    // automatic pieces: the last ones halve down to 8 MB, since what remains after
+    // the last copy (its count, the finish) is not overlapped by any
+    // (texts of 32 MB and less gain nothing: each piece has its own launches, and the
+    // first must be long enough to pick a head)
+    const bool taper = !piece_bytes && nbytes > 4 * kTaperMin;
     if (!piece_bytes) piece_bytes = std::max<uint64_t>(64ull << 20, (nbytes + 31) / 32);
     std::vector<uint64_t> cut{0};
     while (cut.back() < nbytes) {
-        uint64_t e = std::min(nbytes, cut.back() + piece_bytes);
+        const uint64_t left = nbytes - cut.back();
+        uint64_t piece = piece_bytes;
+        if (taper && left > kTaperMin && left <= 2 * piece) piece = std::max<uint64_t>(kTaperMin, (left + 1) / 2);
+        uint64_t e = std::min(nbytes, cut.back() + piece);
         while (e < nbytes && host_letter(h_text[e - 1]) && host_letter(h_text[e])) e++;
         cut.push_back(e);
     }
@@ -797,8 +807,10 @@ wc_status wc_merge(wc_ctx *ctx, const wc_table *const *in, uint32_t n, cudaStrea
     }
     cstart[n] = chunks;
     CapPlan plan;
-    plan.cap8 = pow2_at_least(std::max<uint64_t>(1024, 2 * sum8));
-    plan.cap16 = pow2_at_least(std::max<uint64_t>(1024, 2 * sum16));
+    // at most four fifths full even if no word is shared (usually far less: at
+    // twice the words the tables of a large merge no longer fit the L2)
+    plan.cap8 = pow2_at_least(std::max<uint64_t>(1024, sum8 + sum8 / 4));
+    plan.cap16 = pow2_at_least(std::max<uint64_t>(1024, sum16 + sum16 / 4));
     plan.caplong = pow2_at_least(std::max<uint64_t>(256, 2 * sum_lcap));
     plan.arena = std::max<uint64_t>(4096, sum_arena);
     CountScratch cs;

@@ -69,7 +69,7 @@ struct wc_batch {
     // after sync
     bool synced = false;
     wc_status sync_status = WC_OK;
-    uint64_t entries = 0, word_bytes = 0;
+    uint64_t entries = 0, word_bytes = 0, nlong = 0;
     // lazily built
     bool tables_built = false;
     bool exact = false;  // capacities at the exact bounds
@@ -102,6 +102,7 @@ static wc_status batch_sync(const wc_batch *cb) {
     const uint32_t st = (uint32_t)meta[8];
     if (e != cudaSuccess) return b->ctx->cuda_fail(e, "batch metadata");
     b->entries = meta[0];
+    b->nlong = meta[1];
     b->sync_status = WC_OK;
     if (st & (ST_TABLE_FULL | ST_LONG_FULL | ST_ARENA_FULL | ST_OUT_FULL)) b->sync_status = WC_ERR_CAPACITY;
     else if (st & ST_TIMEOUT) b->sync_status = WC_ERR_TIMEOUT;
@@ -645,7 +646,8 @@ static wc_status build_tables_at(wc_batch *b, const std::vector<uint64_t> &est, 
         CapPlan plan;
         plan.cap8 = pow2_ge(std::max<uint64_t>(1024, 2 * d));
         plan.cap16 = pow2_ge(std::max<uint64_t>(1024, d + d / 4));
-        plan.caplong = pow2_ge(std::max<uint64_t>(256, 2 * std::min<uint64_t>(d, b->args.lcap)));
+        // no table holds more words of 17+ letters than the documents' rows do
+        plan.caplong = pow2_ge(std::max<uint64_t>(256, 2 * std::min<uint64_t>(d, b->nlong)));
         plan.arena = std::max<uint64_t>(4096, b->args.arena_cap);
         CountScratch &cs = c < b->nclasses ? scr[c] : b->gscratch;
         if ((st = scratch_create(ctx, plan, false, s, cs)) != WC_OK) break;
@@ -915,23 +917,27 @@ struct RatioArgs {
     unsigned long long *out_n;
 };
 
+// Entry i's count in the class and outside it.
+__device__ __forceinline__ void ratio_counts(const RatioArgs &r, unsigned long long i, unsigned long long &cin,
+                                             unsigned long long &cout) {
+    const unsigned long long c = static_cast<const uint32_t *>(r.cls.cnt)[i];
+    const uint32_t lr = r.cls.lref[i];
+    const unsigned long long hi8 = r.cls.khi[i], lo8 = r.cls.klo[i];
+    uint4 k;
+    k.x = __byte_perm((uint32_t)(hi8 >> 32), 0, 0x0123);
+    k.y = __byte_perm((uint32_t)hi8, 0, 0x0123);
+    k.z = __byte_perm((uint32_t)(lo8 >> 32), 0, 0x0123);
+    k.w = __byte_perm((uint32_t)lo8, 0, 0x0123);
+    const uint8_t *lw = lr ? r.cls.arena + r.cls.loff[lr - 1] : nullptr;
+    const unsigned long long g = lookup_count(r.g, k, lw, lr ? r.cls.llen[lr - 1] : 0);
+    cin = c;
+    cout = g >= c ? g - c : 0;  // g < c cannot happen for consistent tables
+}
 __global__ void k_ratio_prepare(RatioArgs r) {
     const unsigned long long n = r.cls.d_meta[0];
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (unsigned long long)gridDim.x * blockDim.x) {
-        const unsigned long long c = static_cast<const uint32_t *>(r.cls.cnt)[i];
-        const uint32_t lr = r.cls.lref[i];
-        const unsigned long long hi8 = r.cls.khi[i], lo8 = r.cls.klo[i];
-        uint4 k;
-        k.x = __byte_perm((uint32_t)(hi8 >> 32), 0, 0x0123);
-        k.y = __byte_perm((uint32_t)hi8, 0, 0x0123);
-        k.z = __byte_perm((uint32_t)(lo8 >> 32), 0, 0x0123);
-        k.w = __byte_perm((uint32_t)lo8, 0, 0x0123);
-        const uint8_t *lw = lr ? r.cls.arena + r.cls.loff[lr - 1] : nullptr;
-        const unsigned long long g = lookup_count(r.g, k, lw, lr ? r.cls.llen[lr - 1] : 0);
-        r.cin[i] = c;
-        r.cout[i] = g >= c ? g - c : 0;  // g < c cannot happen for consistent tables
-    }
+         i += (unsigned long long)gridDim.x * blockDim.x)
+        ratio_counts(r, i, r.cin[i], r.cout[i]);
 }
 
 // true when entry a ranks above entry b: cin/cout descending (cout = 0 is
@@ -1078,6 +1084,72 @@ __global__ void __launch_bounds__(kRatioSort / 2) k_ratio_round(RatioArgs r, con
     for (uint32_t j = threadIdx.x; j < keep; j += blockDim.x) dst[(unsigned long long)blockIdx.x * keep + j] = si[j];
 }
 
+// k up to kRatioCountMax: block b ranks the 256 list entries src[b * 256, ...) by
+// counting, for each, the entries before it (256 comparisons a thread and no
+// barrier, where the bitonic network has 55 stages of 1,024; 25 us a round), and
+// keeps its first `keep`; the list shrinks at least 4 x a round.  An entry's
+// 128-bit key is its quotient cin / cout in double (positive: its bits order as it
+// does, and integer comparisons do not run at the fp64 pipe's rate), then cin,
+// then the entry's index reversed.  Division rounds monotonically, and quotients
+// of counts below 2^25 are equal only if exactly equal (two unequal ones differ
+// by 2^-50 of their value at least); a block that holds a larger count compares
+// exactly.  The first round (src null) looks the entries' counts up and stores
+// them for the others; the last (one block) writes the rows.
+constexpr int kRatioSlice2 = 256;
+constexpr uint32_t kRatioCountMax = kRatioSlice2 / 4;
+__global__ void __launch_bounds__(kRatioSlice2) k_ratio_count(RatioArgs r, const unsigned long long *src,
+                                                              unsigned long long len, unsigned long long *dst,
+                                                              uint32_t keep, unsigned long long *rows) {
+    __shared__ ulonglong2 sk[kRatioSlice2];
+    __shared__ unsigned long long si[kRatioSlice2], sc[kRatioSlice2], so[kRatioSlice2];
+    grid_dependency_wait();
+    grid_dependency_trigger();
+    const uint32_t t = threadIdx.x;
+    const unsigned long long p = (unsigned long long)blockIdx.x * kRatioSlice2 + t;
+    unsigned long long i = kNoEntry, c = 0, o = 0;
+    if (p < len) i = src ? src[p] : p;
+    if (i != kNoEntry) {
+        if (src) {
+            c = r.cin[i];
+            o = r.cout[i];
+        } else {
+            ratio_counts(r, i, c, o);
+            r.cin[i] = c;
+            r.cout[i] = o;
+        }
+    }
+    // no entry: after every entry (a quotient is above 0), in place order
+    const unsigned long long q = i == kNoEntry ? 0ull
+                                 : o           ? (unsigned long long)__double_as_longlong((double)c / (double)o)
+                                               : ~0ull;
+    const ulonglong2 mine = make_ulonglong2(q, (c << 32) | (0xFFFFFFFFull - (i == kNoEntry ? t : i)));
+    sk[t] = mine;
+    si[t] = i;
+    sc[t] = c;
+    so[t] = o;
+    uint32_t rank = 0;
+    if (!__syncthreads_or(c >= (1ull << 25) || o >= (1ull << 25))) {
+#pragma unroll 8
+        for (int j = 0; j < kRatioSlice2; j++) {
+            const ulonglong2 x = sk[j];
+            rank += (x.x != q ? x.x > q : x.y > mine.y) ? 1u : 0u;
+        }
+    } else {
+        for (int j = 0; j < kRatioSlice2; j++)
+            if (j != (int)t && (i == kNoEntry ? si[j] != kNoEntry || j < (int)t
+                                              : si[j] != kNoEntry && ratio_better(si[j], sc[j], so[j], i, c, o)))
+                rank++;
+    }
+    if (rank < keep) {
+        dst[(unsigned long long)blockIdx.x * keep + rank] = i;
+        if (rows && i != kNoEntry) {
+            rows[3 * rank] = i;
+            rows[3 * rank + 1] = c;
+            rows[3 * rank + 2] = o;
+        }
+    }
+}
+
 // Rows j < m of the ranking: (entry index, cin, cout).
 __global__ void k_ratio_rows(RatioArgs r, const unsigned long long *list, unsigned long long m, unsigned long long *rows) {
     for (unsigned long long j = threadIdx.x; j < m; j += blockDim.x) {
@@ -1103,13 +1175,13 @@ wc_status wc_class_ratio_topk(wc_ctx *ctx, const wc_batch *cb, uint32_t cls, uin
     const uint64_t n = ct->n;
     const uint64_t m = std::min<uint64_t>(k, n);  // rows of the answer
     if (m == 0) return WC_OK;
-    const bool rounds = k <= kRatioKeepMax;
+    const bool counted = m <= kRatioCountMax, rounds = k <= kRatioKeepMax;
     const uint64_t nblk = (n + kRatioSlice - 1) / kRatioSlice;  // first-round blocks (kRatioSort == kRatioSlice)
-    // cin, cout, the answer rows; then two round lists (bitonic rounds) or
-    // the top k + its length, the slices' winners + lengths and taken flags
-    const size_t list_bytes = nblk * (size_t)m * 8;
+    // cin, cout, the answer rows; then two round lists (counting or bitonic rounds)
+    // or the top k + its length, the slices' winners + lengths and taken flags
+    const size_t list = (counted ? (n + kRatioSlice2 - 1) / kRatioSlice2 : nblk) * (size_t)m;
     const size_t bytes = n * 16 + m * 24 +
-                         (rounds ? 2 * list_bytes : ((size_t)k + 1) * 8 + nblk * ((size_t)k + 1) * 8 + n + nblk * k) + 256;
+                         (counted || rounds ? 16 * list : ((size_t)k + 1) * 8 + nblk * ((size_t)k + 1) * 8 + n + nblk * k) + 256;
     void *mem = nullptr;
     if ((st = ctx->alloc(&mem, bytes, stream)) != WC_OK) return st;
     uint8_t *p = static_cast<uint8_t *>(mem);
@@ -1122,37 +1194,49 @@ wc_status wc_class_ratio_topk(wc_ctx *ctx, const wc_batch *cb, uint32_t cls, uin
     r.k = k;
     r.out_idx = r.out_n = nullptr;
     const int sms = ctx->sms;
-    uint64_t launches = 2;  // prepare, rows
-    k_ratio_prepare<<<std::max<int>(1, std::min<int>(sms * 4, (int)((n + 255) / 256))), 256, 0, stream>>>(r);
-    const unsigned long long *top = nullptr;
-    if (rounds) {
-        unsigned long long *list[2] = {rows + 3 * m, rows + 3 * m + nblk * m};
+    unsigned long long *lists[2] = {rows + 3 * m, rows + 3 * m + list};
+    if (counted) {
         const unsigned long long *src = nullptr;
         uint64_t len = n;
-        int w = 0;
-        for (;;) {
-            const uint64_t nb = (len + kRatioSort - 1) / kRatioSort;
-            k_ratio_round<<<(unsigned int)nb, kRatioSort / 2, 0, stream>>>(r, src, len, list[w], (uint32_t)m);
-            launches++;
+        for (int w = 0;; w ^= 1) {
+            const uint64_t nb = (len + kRatioSlice2 - 1) / kRatioSlice2;
+            launch_dependent(k_ratio_count, dim3((unsigned int)nb), dim3(kRatioSlice2), 0, stream, r, src,
+                             (unsigned long long)len, lists[w], (uint32_t)m, nb == 1 ? rows : nullptr);
+            ctx->launches++;
             if (nb == 1) break;
-            src = list[w];
+            src = lists[w];
             len = nb * m;
-            w ^= 1;
         }
-        top = list[w];
     } else {
-        r.out_idx = rows + 3 * m;
-        r.out_n = r.out_idx + k;
-        unsigned long long *cand = r.out_n + 1, *cand_n = cand + nblk * k;
-        unsigned char *taken = reinterpret_cast<unsigned char *>(cand_n + nblk);
-        cudaMemsetAsync(taken, 0, n + nblk * k, stream);
-        k_ratio_select_slices<<<(unsigned int)nblk, 256, 0, stream>>>(r, taken, cand, cand_n);
-        k_ratio_select<<<1, 1024, 0, stream>>>(r, taken + n, cand, cand_n, (unsigned int)nblk);
-        top = r.out_idx;
-        launches += 2;
+        const unsigned long long *top = nullptr;
+        uint64_t launches = 2;  // prepare, rows
+        k_ratio_prepare<<<std::max<int>(1, std::min<int>(sms * 4, (int)((n + 255) / 256))), 256, 0, stream>>>(r);
+        if (rounds) {
+            const unsigned long long *src = nullptr;
+            uint64_t len = n;
+            for (int w = 0;; w ^= 1) {
+                const uint64_t nb = (len + kRatioSort - 1) / kRatioSort;
+                k_ratio_round<<<(unsigned int)nb, kRatioSort / 2, 0, stream>>>(r, src, len, lists[w], (uint32_t)m);
+                launches++;
+                src = lists[w];
+                len = nb * m;
+                if (nb == 1) break;
+            }
+            top = src;
+        } else {
+            r.out_idx = rows + 3 * m;
+            r.out_n = r.out_idx + k;
+            unsigned long long *cand = r.out_n + 1, *cand_n = cand + nblk * k;
+            unsigned char *taken = reinterpret_cast<unsigned char *>(cand_n + nblk);
+            cudaMemsetAsync(taken, 0, n + nblk * k, stream);
+            k_ratio_select_slices<<<(unsigned int)nblk, 256, 0, stream>>>(r, taken, cand, cand_n);
+            k_ratio_select<<<1, 1024, 0, stream>>>(r, taken + n, cand, cand_n, (unsigned int)nblk);
+            top = r.out_idx;
+            launches += 2;
+        }
+        ctx->launches += launches;
+        k_ratio_rows<<<1, 256, 0, stream>>>(r, top, m, rows);
     }
-    ctx->launches += launches;
-    k_ratio_rows<<<1, 256, 0, stream>>>(r, top, m, rows);
     std::vector<unsigned long long> h(3 * m);
     cudaError_t e = cudaMemcpyAsync(h.data(), rows, m * 24, cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
