@@ -363,7 +363,7 @@ static size_t table_bytes(uint64_t cap, uint64_t lcap, uint64_t arena, int bits)
 }
 
 wc_status table_create(wc_ctx *ctx, uint64_t cap, uint64_t lcap, uint64_t arena, int bits, cudaStream_t s,
-                       wc_table **out) {
+                       wc_table **out, bool clear) {
     wc_table *t = new wc_table();
     t->ctx = ctx;
     t->bytes = table_bytes(cap, lcap, arena, bits);
@@ -385,7 +385,7 @@ wc_status table_create(wc_ctx *ctx, uint64_t cap, uint64_t lcap, uint64_t arena,
     d.loff = reinterpret_cast<unsigned long long *>(take(lcap * 8));
     d.llen = reinterpret_cast<unsigned long long *>(take(lcap * 8));
     d.arena = take(arena);
-    cudaMemsetAsync(t->mem, 0, 68, s);  // meta + status
+    if (clear) cudaMemsetAsync(t->mem, 0, 68, s);  // meta + status
     t->stream = s;
     cudaEventCreateWithFlags(&t->done, cudaEventDisableTiming);
     *out = t;
@@ -646,6 +646,29 @@ wc_status wc_count_ex(wc_ctx *ctx, const uint8_t *d_text, uint64_t nbytes, const
     if (ctx->count_bits == 32 && nbytes >= (1ull << 33))
         return ctx->fail(WC_ERR_UNSUPPORTED, "32-bit counts need inputs under 2^33 bytes");
     cudaSetDevice(ctx->device);
+    // short texts without capacity hints: one block does it all (at the limit, count +
+    // size 48-180 us against 127-11,500 by the general path's chain of launches)
+    const bool hints = opts && (opts->table_slots || opts->long_slots || opts->arena_bytes || opts->no_level1);
+    if (nbytes && nbytes <= kSmallCountMax && !hints) {
+        uint64_t cap = 0, lcap = 0, arena = 0;
+        small_count_caps(nbytes, &cap, &lcap, &arena);
+        wc_table *t = nullptr;
+        const wc_status st = table_create(ctx, cap, lcap, arena, ctx->count_bits, stream, &t, false);
+        if (st != WC_OK) return st;
+        t->src_bytes = nbytes;
+        t->max_tokens = nbytes / 2 + 1;
+        ctx->prof_mark(ctx->ev_count, stream);
+        const cudaError_t e = launch_count_small(d_text, nbytes, t->dt, stream);
+        ctx->prof_mark(ctx->ev_count, stream);
+        ctx->launches++;
+        table_mark_done(t, stream);
+        if (e != cudaSuccess) {
+            wc_table_free(t);
+            return ctx->cuda_fail(e, "count launch");
+        }
+        *out = t;
+        return WC_OK;
+    }
     const CapPlan plan = plan_capacity(ctx, nbytes, opts);
     CountScratch cs;
     // head scratch only for texts long enough to sample a head from

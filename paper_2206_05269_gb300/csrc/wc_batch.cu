@@ -213,8 +213,7 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
     extern __shared__ __align__(16) uint8_t smem[];
     uint8_t *win = smem;
     uint32_t *tokall = reinterpret_cast<uint32_t *>(smem + C::WINB);
-    // the sort's lists, reusing window + queues: entries as found (then in order),
-    // their parts, entries by part
+    // order_by_parts' lists and tables, reusing window + queues
     uint16_t *found = reinterpret_cast<uint16_t *>(smem), *prow = found + C::NMAX, *byparts = prow + C::NMAX;
     ulonglong2 *coarse = reinterpret_cast<ulonglong2 *>(smem + C::SORT_LISTS);
     KeyRange *range = reinterpret_cast<KeyRange *>(coarse + kBktCoarse + 1);
@@ -497,94 +496,8 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
         auto key_of = [&](uint32_t s) -> ulonglong2 {
             return s < (uint32_t)C::C1 ? reinterpret_cast<const ulonglong2 *>(skey)[s] : lkey[s - C::C1];
         };
-        // Sort: parts of a few entries (32 coarse ones between evenly spaced
-        // entries of the document, each split evenly by interpolation), then each
-        // entry's row is its part's first row plus the part's entries before it.
-        // About 200 instructions an entry; a bitonic network over the list took
-        // 500 (200 entries) to 1,800 (6,000) and a block barrier a stage.
-        uint16_t *sidx = byparts;
-        uint32_t fine = 1;
-        while (fine < C::PARTS / kBktCoarse && fine * kBktCoarse * 3u < n) fine <<= 1;
-        {
-            ulonglong2 *cand = reinterpret_cast<ulonglong2 *>(sidx);
-            constexpr uint32_t kLanes = BLOCK / kBktCoarse;  // threads that rank one candidate
-            if (threadIdx.x + 1 < (uint32_t)kBktCoarse && n) cand[threadIdx.x] = key_of(found[(threadIdx.x + 1) * n / kBktCoarse]);
-            __syncthreads();
-            const uint32_t i = threadIdx.x / kLanes;
-            uint32_t r = 0;
-            if (i + 1 < (uint32_t)kBktCoarse) {
-                const ulonglong2 k = cand[i];
-                for (uint32_t j = threadIdx.x % kLanes; j + 1 < (uint32_t)kBktCoarse; j += kLanes)
-                    r += row_less(cand[j], j, k, i) ? 1u : 0u;
-            }
-#pragma unroll
-            for (uint32_t o = kLanes / 2; o; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
-            if (threadIdx.x % kLanes == 0u) {
-                if (i + 1 < (uint32_t)kBktCoarse) coarse[r + 1] = cand[i];
-                else coarse[0] = make_ulonglong2(0ull, 0ull);
-            }
-            if (threadIdx.x == 0) coarse[kBktCoarse] = make_ulonglong2((0xFFFFull << 48) - 1ull, ~0ull);  // counts are at least 1
-        }
-        __syncthreads();
-        if (threadIdx.x < (uint32_t)kBktCoarse) range[threadIdx.x].set(coarse[threadIdx.x], coarse[threadIdx.x + 1], fine);
-        __syncthreads();
-        for (uint32_t e = threadIdx.x; e < n; e += BLOCK) {
-            const ulonglong2 k = key_of(found[e]);
-            uint32_t c = 0;
-#pragma unroll
-            for (uint32_t step = kBktCoarse / 2; step; step >>= 1) {
-                const ulonglong2 v = coarse[c + step];
-                if (v.x != k.x ? v.x < k.x : v.y <= k.y) c += step;
-            }
-            const uint32_t q = c * fine + range[c](k);
-            prow[e] = (uint16_t)q;
-            atomicAdd(&pcount[q], 1u);
-        }
-        __syncthreads();
-        if (warp == 0) {  // counts -> first rows
-            constexpr int kPer = C::PARTS / 32;
-            uint32_t c[kPer], own = 0;
-#pragma unroll
-            for (int q = 0; q < kPer; q++) {
-                c[q] = pcount[lane * kPer + q];
-                own += c[q];
-            }
-            uint32_t incl = own;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t x = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o) incl += x;
-            }
-            uint32_t run = incl - own;
-#pragma unroll
-            for (int q = 0; q < kPer; q++) {
-                pcount[lane * kPer + q] = run;
-                run += c[q];
-            }
-        }
-        __syncthreads();
-        for (uint32_t e = threadIdx.x; e < n; e += BLOCK) sidx[atomicAdd(&pcount[prow[e]], 1u)] = found[e];
-        __syncthreads();
-        // pcount[q] is now the first row after part q.  Thread and place agree (not
-        // thread and entry), so that a warp's lanes rank within the same few parts
-        // and a long part holds up only the warps that own it.
-        uint16_t *order = found;
-        for (uint32_t j = threadIdx.x; j < n; j += BLOCK) {
-            uint32_t q = 0;
-#pragma unroll
-            for (uint32_t step = C::PARTS / 2; step; step >>= 1)
-                if (pcount[q + step - 1] <= j) q += step;
-            const uint32_t lo = q ? pcount[q - 1] : 0u, hi = pcount[q], mine = sidx[j];
-            const ulonglong2 k = key_of(mine);
-            uint32_t rank = lo;
-            for (uint32_t i = lo; i < hi; i++) {
-                const ulonglong2 o = key_of(sidx[i]);
-                rank += (o.x != k.x ? o.x < k.x : o.y < k.y) ? 1u : 0u;
-            }
-            order[rank] = (uint16_t)mine;  // (the entries as found are not read any more)
-        }
-        __syncthreads();
-        sidx = order;
+        uint16_t *sidx = order_by_parts<BLOCK, C::PARTS>(n, found, prow, byparts, coarse, range, pcount, key_of,
+                                                         [](uint32_t, uint32_t) { return false; });
         // long words with equal count and prefix: order by their remaining
         // bytes (insertion over each such run; runs are rare and short)
         if (sh.nlong) {

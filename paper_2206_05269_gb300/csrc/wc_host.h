@@ -106,8 +106,9 @@ struct CapPlan {
     uint64_t cap8, cap16, caplong, arena;
 };
 
+// clear: zero the metadata and status (for kernels that add to them).
 wc_status table_create(wc_ctx *ctx, uint64_t cap, uint64_t lcap, uint64_t arena, int bits, cudaStream_t s,
-                       wc_table **out);
+                       wc_table **out, bool clear = true);
 void table_mark_done(wc_table *t, cudaStream_t s);
 wc_status table_sync(const wc_table *t);
 CapPlan plan_capacity(const wc_ctx *ctx, uint64_t nbytes, const wc_count_opts *o);

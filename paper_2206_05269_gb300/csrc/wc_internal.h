@@ -40,6 +40,11 @@ cudaError_t launch_wait_selftest(uint32_t *d_status, uint32_t polls, int arrive,
 int count_global_launches(uint64_t nbytes, bool head, bool scratch);
 size_t head_scratch_bytes();
 
+// Texts of at most kSmallCountMax bytes: the whole table by one block, no scratch
+// (wc_small.cu).  small_count_caps: sizes of `out` that always suffice.
+constexpr uint64_t kSmallCountMax = 16384;
+void small_count_caps(uint64_t nbytes, uint64_t *cap, uint64_t *lcap, uint64_t *arena);
+
 // ---------------------------------------------------------------- dependent launches
 // A kernel launched with launch_dependent may have its blocks scheduled
 // before the previous kernel in the stream has finished; it must call
@@ -94,6 +99,10 @@ struct DevTable {
     unsigned long long *loff, *llen;
     uint8_t *arena;
 };
+
+// Counts d_text[0, nbytes) into `out` (metadata and status written too); nbytes
+// in 1 .. kSmallCountMax.
+cudaError_t launch_count_small(const uint8_t *d_text, uint64_t nbytes, DevTable &out, cudaStream_t s);
 
 // Scratch for compaction + sort of up to `cap` entries.
 // Radix passes of the entry sort: 10 byte digits of the packed 16-letter
