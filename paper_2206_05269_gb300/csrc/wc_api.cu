@@ -671,8 +671,7 @@ wc_status wc_count_ex(wc_ctx *ctx, const uint8_t *d_text, uint64_t nbytes, const
     }
     const CapPlan plan = plan_capacity(ctx, nbytes, opts);
     CountScratch cs;
-    // head scratch only for texts long enough to sample a head from
-    wc_status st = scratch_create(ctx, plan, nbytes >= count_global_head_min(), stream, cs);
+    wc_status st = scratch_create(ctx, plan, nbytes >= count_global_scratch_min(), stream, cs);
     if (st != WC_OK) return st;
     wc_table *t = nullptr;
     st = table_create(ctx, cs.entries(), plan.caplong, plan.arena, ctx->count_bits, stream, &t);
@@ -688,7 +687,7 @@ wc_status wc_count_ex(wc_ctx *ctx, const uint8_t *d_text, uint64_t nbytes, const
     cl.main_ev[1] = ctx->prof_event(ctx->ev_count);
     cudaError_t e = launch_count_global(cl, stream);
     ctx->prof_mark(ctx->ev_count, stream);
-    ctx->launches += count_global_launches(nbytes, !cl.no_level1, cs.head != nullptr);
+    ctx->launches += count_global_launches(nbytes, nbytes >= count_global_head_min() && !cl.no_level1, cs.head != nullptr);
     ctx->prof_mark(ctx->ev_finish, stream);
     const uint32_t skip = sort_skip_mask(nbytes / 2 + 1, 0);  // no count exceeds the token bound
     if (e == cudaSuccess) e = finish_table(g, cs.gcap8, cs.gcap, cs.glcap, cs.ss, cs.bs, t->dt, stream, skip);
@@ -778,10 +777,10 @@ wc_status wc_count_host(wc_ctx *ctx, const uint8_t *h_text, uint64_t nbytes, uin
         e = cudaMemcpyAsync(dt + cut[i], h_text + cut[i], cut[i + 1] - cut[i], cudaMemcpyHostToDevice, ctx->copy_stream);
         if (e == cudaSuccess) e = cudaEventRecord(ev[i], ctx->copy_stream);
     }
-    const bool head = np && cut[1] - cut[0] >= count_global_head_min();  // the first piece picks the head
+    const bool head = np && cut[1] - cut[0] >= count_global_scratch_min();  // the first piece picks the head
     for (size_t i = 0; i < np && e == cudaSuccess; i++) {
         e = cudaStreamWaitEvent(stream, ev[i], 0);
-        CountLaunch cl{dt, cut[i], cut[i + 1], g, 0, cs.head, {nullptr, nullptr}, i == 0 ? 0 : (head ? 1 : 2)};
+        CountLaunch cl{dt, cut[i], cut[i + 1], g, 0, cs.head, {nullptr, nullptr}, head ? (i == 0 ? 3 : 1) : 2};
         cl.no_level1 = opts && opts->no_level1 ? 1 : 0;
         if (e == cudaSuccess) e = launch_count_global(cl, stream);
         ctx->launches += count_global_launches(cut[i + 1] - cut[i], i == 0 && head && !cl.no_level1, cs.head != nullptr);

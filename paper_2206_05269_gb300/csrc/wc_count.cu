@@ -5,16 +5,16 @@
 // conclusion (Sec. 5.2) asks for a GPU dictionary so the whole map and reduce
 // run on the device.  This file is that design for one document.
 //
-// Work split.  The document is cut into 512-byte strips (16-byte aligned in
-// absolute address space).  Every warp of the grid owns every
-// (grid x warps)-th strip and stages its strips through a private ring of
-// four buffers: a strip's window (16 bytes before it, the strip, 32 bytes
-// after it) arrives by one TMA bulk copy that completes an mbarrier of that
+// Work split.  The document is cut into strips of 512 bytes (1 KB in texts of
+// 16 MB or more; 16-byte aligned in absolute address space).  Every warp of the
+// grid owns every (grid x warps)-th strip and stages its strips through a
+// private ring of four (two) buffers: a strip's window (16 bytes before it, the
+// strip, 32 bytes after it) arrives by one TMA bulk copy that completes an mbarrier of that
 // warp; windows touching the document's edges are loaded by the warp with
 // plain loads and the outside masked to spaces (a document edge separates
 // words).  No warp ever waits for another.
 //
-// Per strip a lane classifies 16 bytes (SWAR letter mask); word starts are
+// Per strip a lane classifies 16 or 32 bytes (SWAR letter mask); word starts are
 // letters whose previous byte is not one (carried across lanes, and from the
 // window's lead byte across strips); a word belongs to the strip holding its
 // first byte and is read through the window's lookahead.  Starts of words of
@@ -22,10 +22,11 @@
 // are processed 32 at a time, one per lane (with a HEAD table, two batches of
 // 32 at once, their lookups interleaved):
 //   * level 1 (shared memory): a word of at most 8 letters is looked up in
-//     the block's table of 8,192 keys and, if there, its shared count is
+//     the block's table of 4,096 keys and, if there, its shared count is
 //     incremented.  Two table kinds:
-//       HEAD  (texts of 16 MB or more): a read-only image of the words a
-//             sampling pass found most frequent, placed by hash-and-displace
+//       HEAD  (texts of 80 MB or more; pieces of 16 MB or more that arrive from
+//             the host): a read-only image of the words a sampling pass found
+//             most frequent, placed by hash-and-displace
 //             (one displacement byte per bucket of keys), so a lookup is one
 //             displacement load and one key compare;
 //       LOCAL (smaller texts, and the sampling pass itself): an empty table
@@ -34,7 +35,7 @@
 //   * level 2 (global memory): every other word goes to a per-warp tail
 //     queue of 16-byte keys, flushed 32 at a time into the global 8-byte-key
 //     or 16-byte-key open-addressing table (slot loads issued one flush
-//     ahead, fire-and-forget reductions, CAS only for a word's first claim).
+//     ahead, fire-and-forget reductions and claims).
 // Words of 17+ letters are queued by address and, with head scratch (texts
 // of 16 MB or more), appended to a global queue that k_long_deferred drains
 // after this kernel; otherwise (or when that queue is full) they are inserted
@@ -51,31 +52,63 @@
 
 namespace wc {
 
-constexpr int kWarps = 20;                // warps of the counting kernel, each with its own ring
-constexpr int kBlock = kWarps * 32;
-constexpr int kStrip = 512;               // bytes a warp classifies per step (16 per lane)
 constexpr int kLead = 16;                 // window bytes before the strip (the previous byte, aligned)
-constexpr int kWinB = kLead + kStrip + 32;  // + 32 lookahead: 560 bytes, a multiple of 16
-constexpr int kStages = 4;                // ring buffers per warp
-constexpr int kTokCap = 32 + 256;         // queued words: < 32 left over + at most 256 starts a strip
-constexpr int kTailCap = 64;
+constexpr int kTailCap = 64;              // < 32 left over + at most 32 misses a batch
 constexpr int kLongCap = 48;              // < 16 left over + at most 32 starts a step
-constexpr int kHeadSlots = 8192;          // level-1 table keys
 constexpr int kHeadBuckets = 2048;        // hash-and-displace buckets of the HEAD image
 constexpr int kLocalProbes = 4;
 constexpr int kSamplePieces = 32;
 constexpr int kSamplePieceBytes = 65536;
-constexpr uint64_t kHeadMinBytes = 16ull << 20;
+constexpr uint64_t kWideMinBytes = 16ull << 20;  // texts from here on: wide strips, long words deferred
+constexpr uint64_t kHeadMinBytes = 80ull << 20;  // texts from here on: HEAD (see launch_count_global)
 constexpr unsigned long long kSampleSlots = 1ull << 19;
-constexpr int kHeadRegions = 16;          // the image is placed region by region, one warp each
+// Level-1 table keys.  With 8,192 (96 KB with their counts) the counting
+// kernel's block took 193 KB of shared memory, which leaves 60 KB of L1 for the
+// tail's loads in flight, and their latency was the largest stall; at 4,096 the
+// block fits the 164 KB carveout (92 KB of L1), has room for 24 warps instead of
+// 20, and a quarter more of the words go to the tail: 64 MB 148 -> 134 us, 1 GB
+// 1,478 -> 1,503 us, and the image is placed in half the time (88 -> 46 us).
+constexpr int kHeadSlots = 4096;
+constexpr int kHeadRegions = 32;          // the image is placed region by region, one warp each
 constexpr int kRegionSlots = kHeadSlots / kHeadRegions;
-constexpr uint32_t kHeadMax = kHeadSlots * 80 / 100;  // head candidates (load factor of the image)
+constexpr uint32_t kHeadMax = kHeadSlots * 85 / 100;  // head candidates (load of the image)
 constexpr uint32_t kHotMax = 512;                     // candidates placed first (the sample's most frequent)
 constexpr unsigned long long kLongQCap = 1ull << 21;  // deferred long words per launch
-static_assert(kWinB % 16 == 0, "TMA bulk copies move multiples of 16 bytes");
-static_assert(kStages == 4, "2-bit stage tag in queued words");
 
-enum : int { MODE_HEAD = 0, MODE_LOCAL = 1, MODE_SAMPLE = 2 };
+enum : int { MODE_HEAD = 0, MODE_LOCAL = 1, MODE_SAMPLE = 2, MODE_WIDE = 3 };  // WIDE: LOCAL in wide strips
+
+// The strips of a mode, and the shared memory that follows the level-1 table.
+// Wide strips (32 bytes a lane): what a strip costs apart from its words (the
+// window's wait and refill, the prefix sum, the carries between lanes, the
+// slowest lane's share of the extraction) is paid half as often: 1 GB 1,747 ->
+// 1,561 us, 40 MB by LOCAL 328 -> 320.  With two buffers the next window is
+// asked for as soon as the previous strip's last words are looked up.  Texts
+// under 16 MB keep 512-byte strips: a warp has only a few of them, and half as
+// many twice as long ones end later (100 KB 162 -> 177 us).
+template <int MODE>
+struct Geo {
+    static constexpr bool kWide = MODE == MODE_HEAD || MODE == MODE_WIDE;
+    static constexpr int kWarps = MODE == MODE_HEAD ? 24 : 20;  // each with its own ring
+    static constexpr int kBlock = kWarps * 32;
+    static constexpr int kLane = kWide ? 32 : 16;  // bytes a lane classifies per step
+    static constexpr int kStrip = 32 * kLane;
+    static constexpr int kWinB = kLead + kStrip + 32;  // + 32 lookahead
+    static constexpr int kStages = kWide ? 2 : 4;      // ring buffers per warp
+    static constexpr int kTokCap = 32 + kStrip / 2;    // queued words: < 32 left over + at most one start per two bytes
+    static constexpr size_t kRing = (size_t)kWarps * kStages * kWinB, kTok = (size_t)kWarps * kTokCap * 2;
+    static constexpr size_t kTail = (size_t)kWarps * kTailCap * 16, kLong = (size_t)kWarps * kLongCap * 8;
+    static constexpr size_t kBars = (size_t)kWarps * kStages * 8;
+    static constexpr size_t kKeys = (size_t)kHeadSlots * 8, kCnts = (size_t)kHeadSlots * 4, kDisp = (size_t)kHeadBuckets;
+    static constexpr size_t kSmem = kKeys + kCnts + kDisp + kRing + kTok + kTail + kLong + kBars;
+    static_assert(kWinB % 16 == 0, "TMA bulk copies move multiples of 16 bytes");
+    static_assert((kStages & (kStages - 1)) == 0 && kStages * kWinB <= 4096, "12-bit ring positions in queued words");
+    static_assert((kKeys + kCnts + kDisp) % 16 == 0 && kRing % 16 == 0 && kTok % 16 == 0, "16-byte aligned queues");
+    // The dynamic shared memory plus the static 256 bytes and the 1 KB the SM
+    // reserves per block stay within the 164 KB carveout.  The tail's loads never
+    // hit L1, but each holds a line of it while in flight (1 GB, the same kernel:
+    // 28 KB of L1 2,222 us, 60 KB 1,507).
+    static_assert(kSmem + 256 + 1024 <= 164 * 1024, "keep the 164 KB shared-memory carveout");
+};
 
 struct Count2Args {
     const uint8_t *text;
@@ -90,7 +123,7 @@ struct Count2Args {
     const uint8_t *head_disp;         // HEAD image: kHeadBuckets displacements
     unsigned long long *lq;           // deferred long words (kLongQCap entries), or null: inserted in place
     unsigned long long *lqn;          // entries appended to lq (may pass kLongQCap: the rest were inserted in place)
-    int l1_off;                       // LOCAL: no level-1 table (every word to the global tables)
+    int l1_off;                       // LOCAL, WIDE: no level-1 table (every word to the global tables)
 };
 
 // ---------------------------------------------------------------- TMA + mbarrier
@@ -152,26 +185,29 @@ __device__ __forceinline__ uint4 spaces16() { return make_uint4(0x20202020u, 0x2
 // 2^40 bytes and grids have at least 128 blocks), so it sees fewer than 2^32
 // words.
 //
-// Level-1 hash of an 8-byte key: the high letters folded onto the low bits,
-// times an odd constant, so that every bit of the product depends on every
-// letter.
-__device__ __forceinline__ unsigned long long l1_mix(unsigned long long key) {
-    if (kOneSlot) return 0ull;  // test build: one home slot, one bucket
-    return (key ^ (key >> 29)) * 0xBF58476D1CE4E5B9ull;
+// Level-1 hashes of an 8-byte key: its halves times odd constants, summed; the
+// high bits depend on every letter.  (32-bit products: four instructions a key
+// instead of eight for a 64-bit one, 1 GB 1,773 -> 1,747 us.)
+__device__ __forceinline__ uint2 l1_mix(unsigned long long key) {
+    if (kOneSlot) return make_uint2(0u, 0u);  // test build: one home slot, one bucket
+    const uint32_t lo = (uint32_t)key, hi = (uint32_t)(key >> 32);
+    return make_uint2(lo * 0x9E3779B1u + hi * 0x85EBCA77u, lo * 0xC2B2AE3Du + hi * 0x27D4EB2Fu);
 }
 // HEAD image (hash and displace): a key's bucket is the top 11 bits of its
-// hash and its region the bucket's low 4 bits; every key of a bucket is
-// placed in its region at base + d * step (mod 512) for the bucket's one
-// displacement d, with base and odd step taken from other bits of the hash,
-// so the slots of one key for d = 0, 1, ... are all distinct.
-static_assert(kHeadSlots == 8192 && kHeadBuckets == 2048 && kRegionSlots == 512, "hash bit fields below");
-__device__ __forceinline__ uint32_t head_bucket(unsigned long long h) { return (uint32_t)(h >> 53); }
-__device__ __forceinline__ uint32_t head_slot(unsigned long long h, uint32_t d) {
-    const uint32_t base = (uint32_t)(h >> 32), step = ((uint32_t)h >> 12) | 1u;
-    return ((head_bucket(h) & (uint32_t)(kHeadRegions - 1)) << 9) | ((base + d * step) & (uint32_t)(kRegionSlots - 1));
+// first hash and its region the bucket's low 5 bits; every key of a bucket is
+// placed in its region at base + d * step (mod 128) for the bucket's one
+// displacement d, with base and odd step taken from its second hash, so the
+// slots of one key for d = 0, 1, ... 127 are all distinct.
+static_assert(kHeadSlots == 4096 && kHeadBuckets == 2048 && kRegionSlots == 128, "hash bit fields below");
+__device__ __forceinline__ uint32_t head_bucket(uint2 h) { return h.x >> 21; }
+__device__ __forceinline__ uint32_t head_in_region(uint2 h, uint32_t d) {
+    return ((h.y >> 25) + d * ((h.y >> 18) | 1u)) & (uint32_t)(kRegionSlots - 1);
 }
-// LOCAL table: home slot = the top 13 bits of the hash.
-__device__ __forceinline__ uint32_t local_home(unsigned long long h) { return (uint32_t)(h >> 51); }
+__device__ __forceinline__ uint32_t head_slot(uint2 h, uint32_t d) {
+    return ((head_bucket(h) & (uint32_t)(kHeadRegions - 1)) << 7) | head_in_region(h, d);
+}
+// LOCAL table: home slot = the top 12 bits of the first hash.
+__device__ __forceinline__ uint32_t local_home(uint2 h) { return h.x >> 20; }
 
 // The LOCAL slot holding `key`, claiming the first empty slot on its probe
 // path by 64-bit CAS; -1 after kLocalProbes occupied slots of other keys.
@@ -191,17 +227,16 @@ __device__ __forceinline__ int local_slot(unsigned long long *skey, unsigned lon
 
 // ---------------------------------------------------------------- keys
 __device__ __forceinline__ unsigned long long key_lo(uint4 k) { return ((unsigned long long)k.y << 32) | k.x; }
-// 16 lowercased bytes of the word win[p, p + len) (len <= 16), zero padded:
+// 16 lowercased bytes of the word win[p, p + len) (1 <= len <= 16), zero padded:
 // a word of at most 8 letters has a zero upper half, and its lower half is
-// its 8-byte key.  mask[len] keeps the low len bytes; lowercasing and masking
+// its 8-byte key.  m keeps the low len bytes; lowercasing and masking
 // take one three-input logic operation per word.  Reads win[p & ~3, +20).
-__device__ __forceinline__ uint4 window_key16(const uint8_t *win, uint32_t p, uint32_t len, const uint4 *mask) {
+__device__ __forceinline__ uint4 window_key16(const uint8_t *win, uint32_t p, uint2 m, uint2 mh) {
     const uint32_t *w = reinterpret_cast<const uint32_t *>(win + (p & ~3u));
     const uint32_t sh = (p & 3u) * 8u;
     const uint32_t a0 = w[0], a1 = w[1], a2 = w[2], a3 = w[3], a4 = w[4];
-    const uint4 m = mask[len];
     return make_uint4((__funnelshift_r(a0, a1, sh) | 0x20202020u) & m.x, (__funnelshift_r(a1, a2, sh) | 0x20202020u) & m.y,
-                      (__funnelshift_r(a2, a3, sh) | 0x20202020u) & m.z, (__funnelshift_r(a3, a4, sh) | 0x20202020u) & m.w);
+                      (__funnelshift_r(a2, a3, sh) | 0x20202020u) & mh.x, (__funnelshift_r(a3, a4, sh) | 0x20202020u) & mh.y);
 }
 
 // ---------------------------------------------------------------- level 2
@@ -213,9 +248,9 @@ __device__ __forceinline__ uint4 window_key16(const uint8_t *win, uint32_t p, ui
 // land) it advances one step:
 //   * the key is in one of the two slots: a fire-and-forget add, done;
 //   * else the first of them not holding another key for good is empty (or,
-//     for 16-byte keys, half written): a CAS claims it, and its result is
-//     checked at the following flush (the word is done if the CAS won or
-//     found the same key, else probing resumes after that slot);
+//     for 16-byte keys, half written): a CAS whose result is not waited for
+//     claims it, and the slot is loaded again (a load after the CAS sees it
+//     taken, by this word or another);
 //   * both slots hold other keys: loads of the next two slots are started.
 // Keys are written once and never move, so a key seen in a slot is final.
 // Both key sizes take the same path: the table (8-byte slots of 16 bytes,
@@ -229,12 +264,12 @@ static_assert(sizeof(GSlot) == 32 && offsetof(GSlot, cnt) == 16, "16-byte slot l
 template <int MODE>
 struct Tail {
     const GTable &g;
-    uint32_t st = 0;  // 0 free, 1 loads in flight, 2 CAS in flight
+    bool busy = false;
     bool p16 = false;
     uint32_t probes = 0;
     unsigned long long k0 = 0, k1 = 0;  // key halves (k1 = 0 for 8-byte keys)
     unsigned long long pslot = 0;
-    uint4 v0, v1;  // slots pslot and pslot + 1 (first 16 bytes), or the CAS result in v0
+    uint4 v0, v1;  // slots pslot and pslot + 1 (first 16 bytes), loads in flight between rounds
 
     __device__ __forceinline__ explicit Tail(const GTable &gt) : g(gt) {}
 
@@ -244,119 +279,92 @@ struct Tail {
     __device__ __forceinline__ unsigned long long msk() const { return p16 ? g.mask : g.mask8; }
     __device__ __forceinline__ uint32_t shf() const { return p16 ? 5u : 4u; }
 
-    __device__ __forceinline__ void load() {
-        uint8_t *t = tab();
-        v0 = ld_relaxed_v2(t + (pslot << shf()));
-        v1 = ld_relaxed_v2(t + (((pslot + 1) & msk()) << shf()));
-        st = 1;
-    }
-    __device__ __forceinline__ void take(uint4 k) {
-        k0 = key_lo(k);
-        k1 = ((unsigned long long)k.w << 32) | k.z;
-        p16 = MODE != MODE_SAMPLE && k1 != 0ull;
-        pslot = hash_slot(k0, k1) >> __clzll((long long)msk());
-        probes = 0;
-        load();
-    }
-    __device__ __forceinline__ void add_at(unsigned long long s) {
-        red_add_u64(reinterpret_cast<unsigned long long *>(tab() + (s << shf()) + (p16 ? 16u : 8u)), 1ull);
-        st = 0;
-    }
-    __device__ __forceinline__ void claim(unsigned long long s) {
-        pslot = s;
-        if (!p16) {
-            const unsigned long long old = atomicCAS(&g.slots8[s].key, 0ull, k0);
-            v0 = make_uint4((uint32_t)old, (uint32_t)(old >> 32), 0u, 0u);
-        } else {
-            const uint4 want = make_uint4((uint32_t)k0, (uint32_t)(k0 >> 32), (uint32_t)k1, (uint32_t)(k1 >> 32));
-            v0 = cas128_global(&g.slots[s].key, make_uint4(0u, 0u, 0u, 0u), want);
-        }
-        st = 2;
-    }
-    __device__ __forceinline__ void next(unsigned long long from) {
-        probes += 2;
-        if (probes >= (uint32_t)kGlobalProbeLimit) {  // the table is full: reported, the word dropped
-            atomicOr(g.status, ST_TABLE_FULL);
-            st = 0;
-            return;
-        }
-        pslot = from & msk();
-        load();
-    }
-    // One step of a busy lane with what its last step fetched.
-    __device__ __forceinline__ void step() {
+    // One step of a busy lane with the two slots its last round loaded; true
+    // when it needs the slots at (the new) pslot.
+    __device__ __forceinline__ bool step() {
         const unsigned long long m = msk();
         const unsigned long long a0 = key_lo(v0), a1 = ((unsigned long long)v0.w << 32) | v0.z;
-        if (st == 2) {  // the CAS result (an 8-byte claim left a1 = 0 = k1)
-            const bool mine = (a0 == 0ull && a1 == 0ull) || (a0 == k0 && a1 == k1);
-            if (mine) add_at(pslot);
-            else next(pslot + 1);
-            return;
-        }
         const unsigned long long b0 = key_lo(v1), b1 = ((unsigned long long)v1.w << 32) | v1.z;
         // an 8-byte slot's second word is its count: only 16-byte keys compare it
         const bool m0 = a0 == k0 && (!p16 || a1 == k1), m1 = b0 == k0 && (!p16 || b1 == k1);
-        if (m0 || m1) { add_at(m0 ? pslot : ((pslot + 1) & m)); return; }
+        if (m0 || m1) {
+            const unsigned long long s = m0 ? pslot : ((pslot + 1) & m);
+            red_add_u64(reinterpret_cast<unsigned long long *>(tab() + (s << shf()) + (p16 ? 16u : 8u)), 1ull);
+            busy = false;
+            return false;
+        }
         // a 16-byte slot with both halves non-zero holds another key for good
         const bool e0 = a0 == 0ull || (p16 && a1 == 0ull), e1 = b0 == 0ull || (p16 && b1 == 0ull);
-        if (e0 || e1) { claim(e0 ? pslot : ((pslot + 1) & m)); return; }
-        next(pslot + 2);
+        pslot = e0 ? pslot : ((pslot + (e1 ? 1 : 2)) & m);
+        if (e0 || e1) {  // claim it; the load that follows shows whose it became
+            uint8_t *slot = tab() + (pslot << shf());
+            if (p16) cas128_drop(slot, k0, k1);
+            else cas64_drop(slot, k0);
+        }
+        probes += 2;
+        if (probes >= (uint32_t)kGlobalProbeLimit) {  // the table is full: reported, the word dropped
+            atomicOr(g.status, ST_TABLE_FULL);
+            busy = false;
+        }
+        return busy;
     }
     // One flush round: busy lanes step, free lanes take words from the end of
     // the queue (tailn, warp-uniform, is updated).
     __device__ __forceinline__ void round(const uint4 *tailq, uint32_t &tailn, int lane) {
-        if (st) step();
-        const uint32_t freem = __ballot_sync(kFull, st == 0u);
+        bool need = false;
+        if (busy) need = step();
+        const uint32_t freem = __ballot_sync(kFull, !busy);
         const uint32_t nf = __popc(freem);
         const uint32_t tk = nf < tailn ? nf : tailn;
         const uint32_t r = __popc(freem & ((1u << lane) - 1u));
-        if (st == 0u && r < tk) take(tailq[tailn - tk + r]);
+        if (!busy && r < tk) {
+            const uint4 k = tailq[tailn - tk + r];
+            k0 = key_lo(k);
+            k1 = ((unsigned long long)k.w << 32) | k.z;
+            p16 = MODE != MODE_SAMPLE && k1 != 0ull;
+            pslot = hash_slot(k0, k1) >> __clzll((long long)msk());
+            probes = 0;
+            busy = need = true;
+        }
+        // the round's only loads (at one place, so that no copy of their
+        // registers makes the warp wait for them here)
+        if (need) {
+            uint8_t *t = tab();
+            v0 = ld_relaxed_v2(t + (pslot << shf()));
+            v1 = ld_relaxed_v2(t + (((pslot + 1) & msk()) << shf()));
+        }
         tailn -= tk;
         __syncwarp();
     }
 };
 
 // ---------------------------------------------------------------- kernel
-constexpr size_t kSmemKeys = (size_t)kHeadSlots * 8;
-constexpr size_t kSmemCnts = (size_t)kHeadSlots * 4;
-constexpr size_t kSmemDisp = (size_t)kHeadBuckets;
-constexpr size_t kSmemRing = (size_t)kWarps * kStages * kWinB;
-constexpr size_t kSmemTok = (size_t)kWarps * kTokCap * 4;
-constexpr size_t kSmemTail = (size_t)kWarps * kTailCap * 16;
-constexpr size_t kSmemLong = (size_t)kWarps * kLongCap * 8;
-constexpr size_t kSmemBars = (size_t)kWarps * kStages * 8;
-constexpr size_t kCountSmem = kSmemKeys + kSmemCnts + kSmemDisp + kSmemRing + kSmemTok + kSmemTail + kSmemLong + kSmemBars;
-static_assert((kSmemKeys + kSmemCnts + kSmemDisp) % 16 == 0 && kSmemRing % 16 == 0 && kSmemTok % 16 == 0,
-              "16-byte aligned ring buffers and queues");
-static_assert(kCountSmem <= 227 * 1024, "counting kernel shared memory");
-// Measured: the dynamic shared memory plus the static 384 bytes and the 1 KB
-// the SM reserves per block must stay within the 196 KB shared-memory
-// carveout.  The next carveout (228 KB) leaves 28 KB of L1 instead of 60 KB,
-// and the tail's global loads then miss L1 (a 10 KB larger tail queue made
-// the kernel 29 % slower).
-static_assert(kCountSmem + 384 + 1024 <= 196 * 1024, "keep the 196 KB shared-memory carveout");
-
 template <int MODE>
-__global__ void __launch_bounds__(kBlock, 1) k_count3(Count2Args a) {
+__global__ void __launch_bounds__(Geo<MODE>::kBlock, 1) k_count3(Count2Args a) {
     extern __shared__ __align__(128) uint8_t smem[];
     // an ordinary launch (measured: as a dependent of the head kernels, with
     // its blocks scheduled early, the kernel ran about 1 % slower); no early
     // trigger, so the deferred long-word kernel launches as its blocks exit
     grid_dependency_wait();
+    using G = Geo<MODE>;
+    constexpr int kWarps = G::kWarps, kBlock = G::kBlock, kLane = G::kLane, kStrip = G::kStrip;
+    constexpr int kWinB = G::kWinB, kStages = G::kStages, kTokCap = G::kTokCap;
     unsigned long long *skey = reinterpret_cast<unsigned long long *>(smem);
-    uint32_t *scnt = reinterpret_cast<uint32_t *>(smem + kSmemKeys);
-    uint8_t *sdisp = smem + kSmemKeys + kSmemCnts;
-    uint8_t *ring_all = sdisp + kSmemDisp;
-    uint32_t *tok_all = reinterpret_cast<uint32_t *>(ring_all + kSmemRing);
-    uint4 *tail_all = reinterpret_cast<uint4 *>(reinterpret_cast<uint8_t *>(tok_all) + kSmemTok);
-    unsigned long long *long_all = reinterpret_cast<unsigned long long *>(reinterpret_cast<uint8_t *>(tail_all) + kSmemTail);
-    uint64_t *bar_all = reinterpret_cast<uint64_t *>(reinterpret_cast<uint8_t *>(long_all) + kSmemLong);
+    uint32_t *scnt = reinterpret_cast<uint32_t *>(smem + G::kKeys);
+    uint8_t *sdisp = smem + G::kKeys + G::kCnts;
+    uint8_t *ring_all = sdisp + G::kDisp;
+    uint16_t *tok_all = reinterpret_cast<uint16_t *>(ring_all + G::kRing);
+    uint4 *tail_all = reinterpret_cast<uint4 *>(reinterpret_cast<uint8_t *>(tok_all) + G::kTok);
+    unsigned long long *long_all = reinterpret_cast<unsigned long long *>(reinterpret_cast<uint8_t *>(tail_all) + G::kTail);
+    uint64_t *bar_all = reinterpret_cast<uint64_t *>(reinterpret_cast<uint8_t *>(long_all) + G::kLong);
 
-    __shared__ uint4 kmask[17];  // kmask[n]: the low n bytes of 16 kept
+    // [n]: the low n + 1 bytes of 16 kept, as two halves: each array covers the
+    // 32 banks once, so lanes with different lengths never conflict
+    __shared__ uint2 kmask[2][16];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint8_t *ring = ring_all + (size_t)warp * kStages * kWinB;
     uint64_t *full = bar_all + warp * kStages;
-    uint32_t *tok = tok_all + warp * kTokCap;
+    uint16_t *tok = tok_all + warp * kTokCap;  // ring position << 4 | length - 1
     uint4 *tailq = tail_all + warp * kTailCap;
     unsigned long long *longq = long_all + warp * kLongCap;
 
@@ -366,9 +374,10 @@ __global__ void __launch_bounds__(kBlock, 1) k_count3(Count2Args a) {
     }
     if (MODE == MODE_HEAD)
         for (int i = threadIdx.x; i < kHeadBuckets; i += kBlock) sdisp[i] = a.head_disp[i];
-    if (threadIdx.x <= 16) {
-        const int n = threadIdx.x;
-        kmask[n] = make_uint4(byte_keep_mask(n), byte_keep_mask(n - 4), byte_keep_mask(n - 8), byte_keep_mask(n - 12));
+    if (threadIdx.x < 16) {
+        const int n = threadIdx.x + 1;
+        kmask[0][n - 1] = make_uint2(byte_keep_mask(n), byte_keep_mask(n - 4));
+        kmask[1][n - 1] = make_uint2(byte_keep_mask(n - 8), byte_keep_mask(n - 12));
     }
     if (lane == 0) {
         for (int b = 0; b < kStages; b++) mbar_init(&full[b], 1);
@@ -379,26 +388,27 @@ __global__ void __launch_bounds__(kBlock, 1) k_count3(Count2Args a) {
     const uintptr_t vb = reinterpret_cast<uintptr_t>(a.text) + a.lo, ve = reinterpret_cast<uintptr_t>(a.text) + a.hi;
     const uint8_t *end = reinterpret_cast<const uint8_t *>(ve);
     const unsigned long long policy = policy_evict_first();
-    // this warp's strips: s0, s0 + stride, ...
+    // this warp's strips: s0, s0 + stride, ... (a block reads under 2^33 bytes: 32-bit counts)
     const unsigned long long stride = (unsigned long long)gridDim.x * kWarps;
     const unsigned long long s0 = (unsigned long long)blockIdx.x * kWarps + (unsigned long long)warp;
-    const unsigned long long nk = s0 < a.nstrips ? (a.nstrips - s0 + stride - 1) / stride : 0ull;
+    const uint32_t nk = s0 < a.nstrips ? (uint32_t)((a.nstrips - s0 + stride - 1) / stride) : 0u;
 
-    auto win_start = [&](unsigned long long k) -> uintptr_t {
+    auto win_start = [&](uint32_t k) -> uintptr_t {
         const unsigned long long s = s0 + k * stride;
-        if (a.piece_strips == 0u) return a.base_al + (uintptr_t)(s * kStrip) - kLead;
+        if (MODE != MODE_SAMPLE) return a.base_al + (uintptr_t)(s * kStrip) - kLead;
         const unsigned long long q = s / a.piece_strips, r = s % a.piece_strips;
         return a.base_al + (uintptr_t)(q * a.piece_stride + r * kStrip) - kLead;
     };
-    // Stages this warp's k-th strip into ring buffer k % kStages (strips are
-    // produced in order; `issued` is one past the last one).
-    unsigned long long issued = 0;
-    auto produce = [&](unsigned long long k) {
-        if (k >= nk) return;
-        issued = k + 1;
-        const int b = (int)(k % kStages);
+    // Stages this warp's next strip into ring buffer `issued` % kStages (strips
+    // are produced in order).
+    uint32_t issued = 0;
+    uintptr_t w0 = win_start(0);
+    const uintptr_t wstep = (uintptr_t)(stride * kStrip);
+    auto produce = [&]() {
+        if (issued >= nk) return;
+        const uint32_t b = issued % kStages;
         uint8_t *win = ring + b * kWinB;
-        const uintptr_t w0 = win_start(k);
+        if (MODE == MODE_SAMPLE) w0 = win_start(issued);
         if (w0 >= vb && w0 + kWinB <= ve) {
             if (lane == 0) {
                 fence_proxy_async();
@@ -417,26 +427,33 @@ __global__ void __launch_bounds__(kBlock, 1) k_count3(Count2Args a) {
             __syncwarp();
             if (lane == 0) mbar_arrive(&full[b]);
         }
+        issued++;
+        w0 += wstep;
         __syncwarp();
     };
 
     Tail<MODE> tl(a.g);
     uint32_t tailn = 0;
+    auto push_tail = [&](bool tail, uint4 tk) {
+        const uint32_t tb = __ballot_sync(kFull, tail);
+        if (tail) tailq[tailn + __popc(tb & ((1u << lane) - 1u))] = tk;
+        tailn += __popc(tb);
+        __syncwarp();
+        while (tailn >= 32) tl.round(tailq, tailn, lane);
+    };
     // One queued word per lane (have: this lane holds one).
     auto process = [&](uint32_t e, bool have) {
         bool tail = false;
         uint4 tk = make_uint4(0u, 0u, 0u, 0u);
         if (have) {
-            const uint32_t len = e & 31u, p = (e >> 5) & 0x3FFu;
-            const uint8_t *w = ring + (e >> 27) * kWinB;
             // one key load for every length (no divergent paths)
-            tk = window_key16(w, p, len, kmask);
+            tk = window_key16(ring, e >> 4, kmask[0][e & 15u], kmask[1][e & 15u]);
             tail = true;
-            if (len <= 8u && (MODE != MODE_LOCAL || !a.l1_off)) {
+            if (!(e & 8u) && ((MODE != MODE_LOCAL && MODE != MODE_WIDE) || !a.l1_off)) {
                 const unsigned long long key = key_lo(tk);
                 int s;
                 if (MODE == MODE_HEAD) {
-                    const unsigned long long h = l1_mix(key);
+                    const uint2 h = l1_mix(key);
                     const uint32_t hs = head_slot(h, sdisp[head_bucket(h)]);
                     s = skey[hs] == key ? (int)hs : -1;
                 } else {
@@ -450,34 +467,20 @@ __global__ void __launch_bounds__(kBlock, 1) k_count3(Count2Args a) {
                 tail = false;  // the sampling pass looks for frequent words of <= 8 letters only
             }
         }
-        const uint32_t tb = __ballot_sync(kFull, tail);
-        if (tail) tailq[tailn + __popc(tb & ((1u << lane) - 1u))] = tk;
-        tailn += __popc(tb);
-        __syncwarp();
-        // flush: the lanes' previous words advance (their loads have had time
-        // to land), free lanes take new ones; the queue ends below 32 words
-        while (tailn >= 32) tl.round(tailq, tailn, lane);
+        push_tail(tail, tk);
     };
     // HEAD mode, two full batches of queued words: the two words' head
     // lookups are independent, so they run interleaved (every load issued
     // before the compares; a word of more than 8 letters never hits), then
-    // each batch's misses are queued and flushed as process does.
-    auto push_tail = [&](bool tail, uint4 tk) {
-        const uint32_t tb = __ballot_sync(kFull, tail);
-        if (tail) tailq[tailn + __popc(tb & ((1u << lane) - 1u))] = tk;
-        tailn += __popc(tb);
-        __syncwarp();
-        while (tailn >= 32) tl.round(tailq, tailn, lane);
-    };
+    // each batch's misses are queued.
     auto process2 = [&](uint32_t e0, uint32_t e1) {
-        const uint32_t n0 = e0 & 31u, n1 = e1 & 31u;
-        const uint4 k0 = window_key16(ring + (e0 >> 27) * kWinB, (e0 >> 5) & 0x3FFu, n0, kmask);
-        const uint4 k1 = window_key16(ring + (e1 >> 27) * kWinB, (e1 >> 5) & 0x3FFu, n1, kmask);
+        const uint4 k0 = window_key16(ring, e0 >> 4, kmask[0][e0 & 15u], kmask[1][e0 & 15u]);
+        const uint4 k1 = window_key16(ring, e1 >> 4, kmask[0][e1 & 15u], kmask[1][e1 & 15u]);
         const unsigned long long y0 = key_lo(k0), y1 = key_lo(k1);
-        const unsigned long long h0 = l1_mix(y0), h1 = l1_mix(y1);
+        const uint2 h0 = l1_mix(y0), h1 = l1_mix(y1);
         const uint32_t s0 = head_slot(h0, sdisp[head_bucket(h0)]), s1 = head_slot(h1, sdisp[head_bucket(h1)]);
         const unsigned long long v0 = skey[s0], v1 = skey[s1];
-        const bool hit0 = n0 <= 8u && v0 == y0, hit1 = n1 <= 8u && v1 == y1;
+        const bool hit0 = !(e0 & 8u) && v0 == y0, hit1 = !(e1 & 8u) && v1 == y1;
         if (hit0) atomicAdd(&scnt[s0], 1u);
         if (hit1) atomicAdd(&scnt[s1], 1u);
         push_tail(!hit0, k0);
@@ -514,30 +517,54 @@ __global__ void __launch_bounds__(kBlock, 1) k_count3(Count2Args a) {
         __syncwarp();
     };
 
-    for (unsigned long long k = 0; k < kStages; k++) produce(k);
+    for (int i = 0; i < kStages; i++) produce();
 
     uint32_t tcount = 0;  // queued words (warp-uniform)
     uint32_t tprev = 0;   // how many of them belong to the previous strip
-    unsigned long long k = 0;
+    uint32_t k = 0;
     bool timed_out = false;
     for (; k < nk; k++) {
-        const int b = (int)(k % kStages);
-        if (!mbar_wait(&full[b], (uint32_t)(k / kStages) & 1u)) { timed_out = true; break; }
+        const uint32_t b = k % kStages;
+        if (!mbar_wait(&full[b], (k / kStages) & 1u)) { timed_out = true; break; }
         const uint8_t *win = ring + b * kWinB;
-        // ---- classify this lane's 16 bytes
-        const uint32_t L = letter_mask16(*reinterpret_cast<const uint4 *>(win + kLead + 16 * lane));
+        // ---- classify this lane's bytes: L its letters, N those of the next kLane bytes
+        uint32_t L = letter_mask16(*reinterpret_cast<const uint4 *>(win + kLead + kLane * lane));
+        if (kLane == 32) L |= letter_mask16(*reinterpret_cast<const uint4 *>(win + kLead + kLane * lane + 16)) << 16;
         // the 32 lookahead bytes after the strip, one per lane, as one mask
         const uint32_t A = __ballot_sync(kFull, is_letter(win[kLead + kStrip + lane]));
         const uint32_t prevL = is_letter(win[kLead - 1]) ? 1u : 0u;
         const uint32_t up = __shfl_up_sync(kFull, L, 1);
         const uint32_t dn = __shfl_down_sync(kFull, L, 1);
-        const uint32_t pbit = lane == 0 ? prevL : ((up >> 15) & 1u);
-        const uint32_t W = L | ((lane == 31 ? (A & 0xFFFFu) : dn) << 16);  // this lane's and the next 16 bytes
-        const uint32_t S = L & ~((L << 1) | pbit) & 0xFFFFu;                // word starts
-        uint32_t x = W;
-        x &= x >> 1; x &= x >> 2; x &= x >> 4; x &= x >> 8; x &= W >> 16;  // starts of 17+ letter runs
+        const uint32_t pbit = lane == 0 ? prevL : (up >> (kLane - 1));
+        uint32_t S = L & ~((L << 1) | pbit);  // word starts
+        uint32_t x;       // starts of 17+ letter runs
+        uint32_t E0, E1;  // last letters of runs, bits 0..31 and (32 bytes a lane) 32..62
+        uint32_t N;
+        if (kLane == 32) {
+            N = lane == 31 ? A : dn;
+            auto ahead = [](uint32_t lo, uint32_t hi, int d) { return __funnelshift_r(lo, hi, d); };
+            uint32_t xn = N & (N >> 1);
+            x = L & ahead(L, N, 1);
+            x &= ahead(x, xn, 2);
+            xn &= xn >> 2;
+            x &= ahead(x, xn, 4);
+            xn &= xn >> 4;
+            x &= ahead(x, xn, 8);
+            x &= ahead(L, N, 16);
+            E0 = L & ~ahead(L, N, 1);
+            E1 = N & ~(N >> 1);
+        } else {
+            N = lane == 31 ? (A & 0xFFFFu) : dn;
+            const uint32_t W = L | (N << 16);
+            S &= 0xFFFFu;
+            x = W;
+            x &= x >> 1; x &= x >> 2; x &= x >> 4; x &= x >> 8; x &= W >> 16;
+            E0 = W & ~(W >> 1);  // bits 0..30 are exact
+            E1 = 0u;
+        }
         uint32_t Ss = S & ~x, Sl = S & x;
-        const uint32_t E = W & ~(W >> 1);  // last letters of runs (bits 0..30 are exact)
+        // a short word's length: it ends within 16 bytes of its start
+        auto short_len = [&](uint32_t j) { return (uint32_t)__ffs((int)(kLane == 32 ? __funnelshift_r(E0, E1, j) : E0 >> j)); };
 
         const uint32_t c1 = __popc(Ss);
         uint32_t incl = c1;
@@ -551,32 +578,34 @@ __global__ void __launch_bounds__(kBlock, 1) k_count3(Count2Args a) {
         // start into the top and its lowest into the bottom (two independent
         // chains; queue order does not matter)
         uint32_t lo = tcount + incl - c1, hi = tcount + incl;
-        const uint32_t tag = ((uint32_t)b << 27) | ((uint32_t)(kLead + 16 * lane) << 5);
+        const uint32_t tag = ((b * kWinB + kLead + (uint32_t)(kLane * lane)) << 4) - 1u;
         const uint32_t nmax = (__reduce_max_sync(kFull, c1) + 1u) >> 1;  // a warp-uniform trip count
         for (uint32_t r = 0; r < nmax; r++) {
             if (Ss) {
                 const uint32_t j = 31u - (uint32_t)__clz(Ss), i = (uint32_t)__ffs(Ss) - 1u;
                 Ss &= ~((1u << j) | (1u << i));
-                // a short word ends within the 32 bits
-                tok[--hi] = tag + (j << 5) + (uint32_t)__ffs(E >> j);
-                if (i != j) tok[lo++] = tag + (i << 5) + (uint32_t)__ffs(E >> i);
+                tok[--hi] = (uint16_t)(tag + (j << 4) + short_len(j));
+                if (i != j) tok[lo++] = (uint16_t)(tag + (i << 4) + short_len(i));
             }
         }
         tcount += total;
         if (MODE != MODE_SAMPLE && __any_sync(kFull, Sl != 0)) {
-            // 48 bits of letter mask from this lane on: runs shorter than 48 - j are measured here
-            const uint32_t dn2 = __shfl_down_sync(kFull, L, 2);
-            const uint32_t third = lane == 31 ? (A >> 16) : (lane == 30 ? (A & 0xFFFFu) : dn2);
-            const unsigned long long W48 = (unsigned long long)W | ((unsigned long long)third << 32);
-            const uintptr_t lbase = win_start(k) + kLead + 16 * (uintptr_t)lane;
+            // 48 or 64 bits of letter mask from this lane on: runs that end within them are measured here
+            constexpr uint32_t kSeen = kLane == 32 ? 64u : 48u;
+            unsigned long long W = (unsigned long long)L | ((unsigned long long)N << kLane);
+            if (kLane == 16) {
+                const uint32_t dn2 = __shfl_down_sync(kFull, L, 2);
+                W |= (unsigned long long)(lane == 31 ? (A >> 16) : (lane == 30 ? (A & 0xFFFFu) : dn2)) << 32;
+            }
+            const uintptr_t lbase = win_start(k) + kLead + kLane * (uintptr_t)lane;
             while (__any_sync(kFull, Sl != 0)) {
                 const bool act = Sl != 0;
                 unsigned long long e = 0;
                 if (act) {
                     const int j = __ffs(Sl) - 1;
                     Sl &= Sl - 1;
-                    const uint32_t run = (uint32_t)__ffsll((long long)~(W48 >> j)) - 1u;
-                    e = ((unsigned long long)(lbase + (uintptr_t)j) << 16) | (run < 48u - (uint32_t)j ? run : 0u);
+                    const uint32_t run = (uint32_t)__ffsll((long long)~(W >> j)) - 1u;
+                    e = ((unsigned long long)(lbase + (uintptr_t)j) << 16) | (run < kSeen - (uint32_t)j ? run : 0u);
                 }
                 const uint32_t lb = __ballot_sync(kFull, act);
                 if (act) longq[longn + __popc(lb & ((1u << lane) - 1u))] = e;
@@ -591,10 +620,22 @@ __global__ void __launch_bounds__(kBlock, 1) k_count3(Count2Args a) {
         }
         __syncwarp();
         // ---- queued words, 32 at a time
+        // the previous strip's buffer is refilled once it holds no queued word any more
+        bool due = k > 0;
+        auto refill = [&]() {
+            if (due) produce();
+            due = false;
+        };
         uint32_t bq = 0;
         if (MODE == MODE_HEAD)
-            for (; bq + 64 <= tcount; bq += 64) process2(tok[bq + lane], tok[bq + 32 + lane]);
-        for (; bq + 32 <= tcount; bq += 32) process(tok[bq + lane], true);
+            for (; bq + 64 <= tcount; bq += 64) {
+                process2(tok[bq + lane], tok[bq + 32 + lane]);
+                refill();
+            }
+        for (; bq + 32 <= tcount; bq += 32) {
+            process(tok[bq + lane], true);
+            if (MODE == MODE_WIDE) refill();
+        }
         uint32_t rem = tcount - bq;
         if (tprev > bq) {  // words of the previous strip still queued: finish them all now
             const uint32_t e = (uint32_t)lane < rem ? tok[bq + lane] : 0u;
@@ -603,13 +644,12 @@ __global__ void __launch_bounds__(kBlock, 1) k_count3(Count2Args a) {
         } else if (bq) {
             const uint32_t e = (uint32_t)lane < rem ? tok[bq + lane] : 0u;
             __syncwarp();
-            if ((uint32_t)lane < rem) tok[lane] = e;
+            if ((uint32_t)lane < rem) tok[lane] = (uint16_t)e;
             __syncwarp();
         }
         tcount = rem;
         tprev = rem;
-        // the previous strip's buffer holds no queued word any more: refill it
-        if (k > 0) produce(k - 1 + kStages);
+        refill();
     }
     // ---- drain: the last strip's queued words, then the long and tail queues
     if (!timed_out) {
@@ -619,15 +659,14 @@ __global__ void __launch_bounds__(kBlock, 1) k_count3(Count2Args a) {
             flush_long(0, longn < 32 ? longn : 32);
             if (longn > 32) flush_long(32, longn - 32);
         }
-        while (tailn > 0 || __any_sync(kFull, tl.st != 0u)) tl.round(tailq, tailn, lane);
+        while (tailn > 0 || __any_sync(kFull, tl.busy)) tl.round(tailq, tailn, lane);
     }
     if (__syncthreads_or(timed_out)) {
         if (lane == 0) {
             if (timed_out) atomicOr(a.g.status, ST_TIMEOUT);
             // let this warp's copies in flight land before the block exits
             // (bounded): strips k .. issued - 1 were staged but not waited for
-            for (unsigned long long j = k; j < issued; j++)
-                mbar_wait(&full[j % kStages], (uint32_t)(j / kStages) & 1u);
+            for (uint32_t j = k; j < issued; j++) mbar_wait(&full[j % kStages], (j / kStages) & 1u);
         }
         return;
     }
@@ -799,39 +838,43 @@ __global__ void k_head_collect(const G8Slot *s, unsigned long long cap, uint32_t
 }
 
 // Places the head candidates into the HEAD image by hash and displace.  The
-// image's regions of 512 slots are independent (a key's region is fixed by
+// image's regions of 128 slots are independent (a key's region is fixed by
 // its bucket), so block r builds region r alone: its eight warps pick out
-// the candidates whose bucket lies in the region and group them by bucket,
-// and its first warp places the buckets in two passes, first those holding one of the sample's
-// kHotMax most frequent words (the region is then nearly empty, so they
-// always find room), then the rest, each pass largest bucket first.  A bucket
-// of at most 8 keys tries 32 displacements at once, one per lane: a lane's
-// displacement qualifies when its keys land on distinct slots that the
-// region's occupancy bitmap shows free, and the lowest qualifying lane takes
-// it.  Larger buckets try one displacement at a time, one key per lane.  A
-// bucket with no displacement in 0..255, or with more than 32 keys, is left
-// out (as are candidates beyond the region's 512 slots): their words are then
-// counted in the global table, never wrongly, because a lookup always
-// compares the whole key.  Empty slots keep key 0, which no word has.
-constexpr int kRegionBuckets = kHeadBuckets / kHeadRegions;  // 128
-static_assert(kRegionBuckets == 128, "four buckets a lane");
+// the candidates whose bucket lies in the region and group them by bucket, and
+// its first warp places the buckets in two passes, first those holding one of
+// the sample's kHotMax most frequent words (the region is then nearly empty, so
+// they always find room), then the rest, each pass largest
+// bucket first.  A bucket of at most 8 keys tries 32 displacements at once, one
+// per lane: a lane's displacement qualifies when its keys land on distinct
+// slots that the region's occupancy bitmap shows free, and the lowest
+// qualifying lane takes it.  Larger buckets try one displacement at a time, one
+// key per lane.  A bucket with no displacement in 0..127, or with more than 32
+// keys, is left out (with 109 candidates a region expected, a few words of the
+// fullest regions): their words are then counted in the global table, never
+// wrongly, because a lookup always compares the whole key.  Empty slots keep key 0, which no word has.  Bound by the chain of
+// buckets, about 700 cycles each: 16 regions of 256 slots 46-50 us, 32 of 128
+// 28 us, 64 of 64 19 us but too many words left out.
+constexpr int kRegionBuckets = kHeadBuckets / kHeadRegions;  // 64
+constexpr int kLaneBuckets = kRegionBuckets / 32;
+constexpr uint32_t kSelMax = 2 * kRegionSlots;
 
 template <int S>
 __device__ __forceinline__ bool chd_place_small(const unsigned long long *bk, uint32_t *used, unsigned long long *rimage,
                                                 uint8_t *disp, uint32_t lane) {
-    unsigned long long key[S], h[S];
+    unsigned long long key[S];
+    uint2 h[S];
 #pragma unroll
     for (int i = 0; i < S; i++) {
         key[i] = bk[i];
         h[i] = l1_mix(key[i]);
     }
-    for (uint32_t dbase = 0; dbase < 256; dbase += 32) {
+    for (uint32_t dbase = 0; dbase < (uint32_t)kRegionSlots; dbase += 32) {
         const uint32_t d = dbase + lane;
         uint32_t slot[S];
         bool ok = true;
 #pragma unroll
         for (int i = 0; i < S; i++) {
-            slot[i] = head_slot(h[i], d) & (uint32_t)(kRegionSlots - 1);
+            slot[i] = head_in_region(h[i], d);
             ok = ok && !((used[slot[i] >> 5] >> (slot[i] & 31u)) & 1u);
 #pragma unroll
             for (int j = 0; j < i; j++) ok = ok && slot[j] != slot[i];
@@ -857,12 +900,12 @@ constexpr int kChdThreads = 256;
 __global__ void __launch_bounds__(kChdThreads) k_head_chd(const unsigned long long *cand, const uint32_t *ccnt,
                                                           const uint32_t *meta, unsigned long long *image,
                                                           uint8_t *disp) {
-    __shared__ unsigned long long sel[kRegionSlots], rkey[kRegionSlots], rimage[kRegionSlots];
+    __shared__ unsigned long long sel[kSelMax], rkey[kSelMax], rimage[kRegionSlots];
     grid_dependency_wait();
     grid_dependency_trigger();
-    __shared__ uint32_t selb[kRegionSlots];  // local bucket, bit 31: hot
+    __shared__ uint32_t selb[kSelMax];  // local bucket, bit 31: hot
     __shared__ uint32_t bsize[kRegionBuckets], bstart[kRegionBuckets], bfill[kRegionBuckets];
-    __shared__ uint32_t used[kRegionSlots / 32];
+    __shared__ uint32_t used[(kRegionSlots + 31) / 32];
     __shared__ uint8_t sdisp[kRegionBuckets];
     __shared__ uint32_t nsel_sh;
     constexpr uint32_t kHot = 1u << 31;
@@ -874,7 +917,7 @@ __global__ void __launch_bounds__(kChdThreads) k_head_chd(const unsigned long lo
         sdisp[i] = 0;
     }
     for (uint32_t i = t; i < kRegionSlots; i += kChdThreads) rimage[i] = 0ull;
-    if (t < kRegionSlots / 32) used[t] = 0;
+    if (t < (kRegionSlots + 31) / 32) used[t] = 0;
     if (t == 0) nsel_sh = 0;
     __syncthreads();
     // ---- this region's candidates (in any order), every thread a share
@@ -883,14 +926,14 @@ __global__ void __launch_bounds__(kChdThreads) k_head_chd(const unsigned long lo
         const uint32_t g = head_bucket(l1_mix(key));
         if ((g & (uint32_t)(kHeadRegions - 1)) == r) {
             const uint32_t pos = atomicAdd(&nsel_sh, 1u);
-            if (pos < (uint32_t)kRegionSlots) {
+            if (pos < kSelMax) {
                 sel[pos] = key;
                 selb[pos] = (g / kHeadRegions) | (ccnt[i] >= hot_min ? kHot : 0u);
             }
         }
     }
     __syncthreads();
-    const uint32_t nsel = nsel_sh < (uint32_t)kRegionSlots ? nsel_sh : (uint32_t)kRegionSlots;
+    const uint32_t nsel = nsel_sh < kSelMax ? nsel_sh : kSelMax;
     for (uint32_t j = t; j < nsel; j += kChdThreads) {
         const uint32_t lb = selb[j] & ~kHot;
         atomicAdd(&bsize[lb], 1u);
@@ -898,10 +941,10 @@ __global__ void __launch_bounds__(kChdThreads) k_head_chd(const unsigned long lo
     }
     __syncthreads();
     if (t >= 32) return;  // grouping and placement: the first warp alone (warp barriers only)
-    // bucket starts: four buckets a lane, then a shuffle scan
+    // bucket starts: two buckets a lane, then a shuffle scan
     uint32_t own = 0;
 #pragma unroll
-    for (int q = 0; q < 4; q++) own += bsize[lane * 4 + q] & 0xFFFFu;
+    for (int q = 0; q < kLaneBuckets; q++) own += bsize[lane * kLaneBuckets + q] & 0xFFFFu;
     uint32_t incl = own;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -910,9 +953,9 @@ __global__ void __launch_bounds__(kChdThreads) k_head_chd(const unsigned long lo
     }
     uint32_t run = incl - own;
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
-        bstart[lane * 4 + q] = run;
-        run += bsize[lane * 4 + q] & 0xFFFFu;
+    for (int q = 0; q < kLaneBuckets; q++) {
+        bstart[lane * kLaneBuckets + q] = run;
+        run += bsize[lane * kLaneBuckets + q] & 0xFFFFu;
     }
     __syncwarp();
     for (uint32_t j = lane; j < nsel; j += 32) {
@@ -922,7 +965,7 @@ __global__ void __launch_bounds__(kChdThreads) k_head_chd(const unsigned long lo
     __syncwarp();
     uint32_t maxsize = 0;
 #pragma unroll
-    for (int q = 0; q < 4; q++) maxsize = max(maxsize, bsize[lane * 4 + q] & 0xFFFFu);
+    for (int q = 0; q < kLaneBuckets; q++) maxsize = max(maxsize, bsize[lane * kLaneBuckets + q] & 0xFFFFu);
     maxsize = __reduce_max_sync(kFull, maxsize);
     // ---- placement
     for (int pass = 0; pass < 2; pass++) {
@@ -947,10 +990,10 @@ __global__ void __launch_bounds__(kChdThreads) k_head_chd(const unsigned long lo
                     }
                     const bool mine = lane < size;
                     const unsigned long long key = mine ? bk[lane] : 0ull;
-                    const unsigned long long h = l1_mix(key);
-                    for (uint32_t d = 0; d < 256; d++) {
+                    const uint2 h = l1_mix(key);
+                    for (uint32_t d = 0; d < (uint32_t)kRegionSlots; d++) {
                         // dummy slots of idle lanes never clash; every lane takes part in the match
-                        const uint32_t slot = mine ? (head_slot(h, d) & (uint32_t)(kRegionSlots - 1)) : 1024u + lane;
+                        const uint32_t slot = mine ? head_in_region(h, d) : 1024u + lane;
                         const uint32_t peers = __match_any_sync(kFull, slot);
                         const bool ok = (!mine || !((used[slot >> 5] >> (slot & 31u)) & 1u)) && peers == (1u << lane);
                         if (!__all_sync(kFull, ok)) continue;
@@ -992,9 +1035,9 @@ static int sm_count_dev() {
     return sms > 0 ? sms : 1;
 }
 
-int count_global_launches(uint64_t nbytes, bool head, bool scratch) {
+int count_global_launches(uint64_t nbytes, bool builds_head, bool scratch) {
     if (!nbytes) return 0;
-    return ((nbytes >= kHeadMinBytes && head) ? 6 : 1) + (scratch ? 1 : 0);
+    return (builds_head ? 6 : 1) + (scratch ? 1 : 0);
 }
 
 cudaError_t ensure_smem_limit(const void *func, int bytes) {
@@ -1012,9 +1055,10 @@ cudaError_t ensure_smem_limit(const void *func, int bytes) {
 }
 
 cudaError_t launch_count_global(const CountLaunch &c, cudaStream_t s) {
-    cudaError_t e = ensure_smem_limit((const void *)k_count3<MODE_HEAD>, (int)kCountSmem);
-    if (e == cudaSuccess) e = ensure_smem_limit((const void *)k_count3<MODE_LOCAL>, (int)kCountSmem);
-    if (e == cudaSuccess) e = ensure_smem_limit((const void *)k_count3<MODE_SAMPLE>, (int)kCountSmem);
+    cudaError_t e = ensure_smem_limit((const void *)k_count3<MODE_HEAD>, (int)Geo<MODE_HEAD>::kSmem);
+    if (e == cudaSuccess) e = ensure_smem_limit((const void *)k_count3<MODE_LOCAL>, (int)Geo<MODE_LOCAL>::kSmem);
+    if (e == cudaSuccess) e = ensure_smem_limit((const void *)k_count3<MODE_WIDE>, (int)Geo<MODE_WIDE>::kSmem);
+    if (e == cudaSuccess) e = ensure_smem_limit((const void *)k_count3<MODE_SAMPLE>, (int)Geo<MODE_SAMPLE>::kSmem);
     if (e == cudaSuccess) e = ensure_smem_limit((const void *)k_long_deferred, (int)kDefSmem);
     if (e != cudaSuccess) return e;
     if (c.hi <= c.lo) return cudaSuccess;
@@ -1026,7 +1070,6 @@ cudaError_t launch_count_global(const CountLaunch &c, cudaStream_t s) {
     a.hi = c.hi;
     a.base_al = (tb + c.lo) & ~(uintptr_t)15;
     const unsigned long long span = tb + c.hi - a.base_al;
-    a.nstrips = (span + kStrip - 1) / kStrip;
     a.piece_strips = 0;
     a.piece_stride = 0;
     a.g = c.g;
@@ -1045,7 +1088,11 @@ cudaError_t launch_count_global(const CountLaunch &c, cudaStream_t s) {
     if (c.no_level1) {  // LOCAL kernel with its table switched off
     } else if (c.head_mode == 1 && hs) {  // the head an earlier launch built
         head = true;
-    } else if (c.head_mode == 0 && n >= kHeadMinBytes && hs) {
+    } else if (hs && (c.head_mode == 3 || (c.head_mode == 0 && n >= kHeadMinBytes))) {
+        // choosing a head (sampling, selection, placement) takes about 90 us; a
+        // table filled as words come counts as fast until it has long been full of
+        // words that came early (count + top 100, us, LOCAL against HEAD: 40 MB
+        // 320, 390; 64 MB 394, 418; 80 MB 435, 443)
         // sampling pass (LOCAL tables per block, spills into the sample table)
         G8Slot *sample = reinterpret_cast<G8Slot *>(hs);
         uint32_t *hist = reinterpret_cast<uint32_t *>(hs + kHsSample);
@@ -1057,10 +1104,10 @@ cudaError_t launch_count_global(const CountLaunch &c, cudaStream_t s) {
         Count2Args sa = a;
         sa.g.slots8 = sample;
         sa.g.mask8 = kSampleSlots - 1;
-        sa.piece_strips = kSamplePieceBytes / kStrip;
+        sa.piece_strips = kSamplePieceBytes / Geo<MODE_SAMPLE>::kStrip;
         sa.piece_stride = (span / kSamplePieces) & ~(unsigned long long)15;
         sa.nstrips = (unsigned long long)sa.piece_strips * kSamplePieces;
-        k_count3<MODE_SAMPLE><<<sms, kBlock, kCountSmem, s>>>(sa);
+        k_count3<MODE_SAMPLE><<<sms, Geo<MODE_SAMPLE>::kBlock, Geo<MODE_SAMPLE>::kSmem, s>>>(sa);
         // each head kernel overlaps its launch with the tail of the one before
         launch_dependent(k_head_hist, dim3(sms), dim3(256), 0, s, (const G8Slot *)sample, kSampleSlots, hist);
         launch_dependent(k_head_threshold, dim3(1), dim3(1024), 0, s, (const uint32_t *)hist, kHeadMax, meta);
@@ -1083,24 +1130,30 @@ cudaError_t launch_count_global(const CountLaunch &c, cudaStream_t s) {
         a.head = image;
         a.head_disp = image_disp;
     }
+    const bool wide = !head && n >= kWideMinBytes;
+    const unsigned kWarps = head ? Geo<MODE_HEAD>::kWarps : Geo<MODE_LOCAL>::kWarps;
+    const unsigned long long strip = head || wide ? Geo<MODE_HEAD>::kStrip : Geo<MODE_LOCAL>::kStrip;
+    static_assert(Geo<MODE_WIDE>::kWarps == Geo<MODE_LOCAL>::kWarps, "one grid rule for both");
+    a.nstrips = (span + strip - 1) / strip;
     // one persistent block per SM (fewer for short texts); each block's
     // level-1 counts stay below 2^32 because a block reads under 2^33 bytes
     unsigned long long grid = c.grid > 0 ? (unsigned long long)c.grid : (unsigned long long)sms;
     const unsigned long long need = (a.nstrips + kWarps - 1) / kWarps;
     if (grid > need) grid = need;
-    while ((a.nstrips + grid * kWarps - 1) / (grid * kWarps) * kWarps * kStrip >= (1ull << 33)) grid *= 2;
+    while ((a.nstrips + grid * kWarps - 1) / (grid * kWarps) * kWarps * strip >= (1ull << 33)) grid *= 2;
     for (cudaEvent_t ev : c.main_ev)
         if (ev) cudaEventRecord(ev, s);
-    if (head) k_count3<MODE_HEAD><<<(unsigned)grid, kBlock, kCountSmem, s>>>(a);
-    else k_count3<MODE_LOCAL><<<(unsigned)grid, kBlock, kCountSmem, s>>>(a);
+    if (head) k_count3<MODE_HEAD><<<(unsigned)grid, Geo<MODE_HEAD>::kBlock, Geo<MODE_HEAD>::kSmem, s>>>(a);
+    else if (wide) k_count3<MODE_WIDE><<<(unsigned)grid, Geo<MODE_WIDE>::kBlock, Geo<MODE_WIDE>::kSmem, s>>>(a);
+    else k_count3<MODE_LOCAL><<<(unsigned)grid, Geo<MODE_LOCAL>::kBlock, Geo<MODE_LOCAL>::kSmem, s>>>(a);
     if (a.lq)
         launch_dependent(k_long_deferred, dim3(sms * 2), dim3(kDefChunk), kDefSmem, s, (const unsigned long long *)a.lq,
                          (const unsigned long long *)a.lqn, a.g, a.lbegin, reinterpret_cast<const uint8_t *>(tb + c.hi));
     return cudaGetLastError();
 }
 
-int count_global_chunk_bytes() { return kStrip; }
 uint64_t count_global_head_min() { return kHeadMinBytes; }
+uint64_t count_global_scratch_min() { return kWideMinBytes; }
 
 // ---------------------------------------------------------------- wait self-test
 // The counting kernel's bounded wait, on a barrier expecting one arrival:

@@ -24,20 +24,21 @@ struct CountLaunch {
     int grid;                // 0 = one persistent block per SM
     void *head_scratch;      // head_scratch_bytes() or null (no shared-memory head)
     cudaEvent_t main_ev[2];  // recorded (when non-null) right before the main counting kernel
-    int head_mode;           // 0: build a head (texts >= count_global_head_min()); 1: reuse the
-                             // head an earlier launch built in head_scratch; 2: no head
+    int head_mode;           // 0: build a head for texts >= count_global_head_min(); 1: reuse the
+                             // head an earlier launch built in head_scratch; 2: no head; 3: build one
     int no_level1;           // 1: no shared-memory level-1 table at all (measurement)
 };
 // Tokenises and counts text[lo, hi) into g (8-byte, 16-byte and long tables).
 cudaError_t launch_count_global(const CountLaunch &c, cudaStream_t s);
-int count_global_chunk_bytes();
 uint64_t count_global_head_min();
+// Head scratch (also where long words wait) pays for itself in texts from here on.
+uint64_t count_global_scratch_min();
 // One block runs the counting kernel's bounded barrier wait (see wc_selftest_wait).
 cudaError_t launch_wait_selftest(uint32_t *d_status, uint32_t polls, int arrive, cudaStream_t s);
-// Kernel launches of one launch_count_global: head selection when `head` and
-// the text is long enough, the counting kernel, and the deferred long-word
+// Kernel launches of one launch_count_global: head selection when it builds a
+// head, the counting kernel, and the deferred long-word
 // inserts when head scratch is given (`scratch`).
-int count_global_launches(uint64_t nbytes, bool head, bool scratch);
+int count_global_launches(uint64_t nbytes, bool builds_head, bool scratch);
 size_t head_scratch_bytes();
 
 // Texts of at most kSmallCountMax bytes: the whole table by one block, no scratch
