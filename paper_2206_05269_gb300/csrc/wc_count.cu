@@ -387,7 +387,6 @@ __global__ void __launch_bounds__(Geo<MODE>::kBlock, 1) k_count3(Count2Args a) {
 
     const uintptr_t vb = reinterpret_cast<uintptr_t>(a.text) + a.lo, ve = reinterpret_cast<uintptr_t>(a.text) + a.hi;
     const uint8_t *end = reinterpret_cast<const uint8_t *>(ve);
-    const unsigned long long policy = policy_evict_first();
     // this warp's strips: s0, s0 + stride, ... (a block reads under 2^33 bytes: 32-bit counts)
     const unsigned long long stride = (unsigned long long)gridDim.x * kWarps;
     const unsigned long long s0 = (unsigned long long)blockIdx.x * kWarps + (unsigned long long)warp;
@@ -412,7 +411,7 @@ __global__ void __launch_bounds__(Geo<MODE>::kBlock, 1) k_count3(Count2Args a) {
         if (w0 >= vb && w0 + kWinB <= ve) {
             if (lane == 0) {
                 fence_proxy_async();
-                tma_load(win, reinterpret_cast<const void *>(w0), kWinB, &full[b], policy);
+                tma_load(win, reinterpret_cast<const void *>(w0), kWinB, &full[b], policy_evict_first());
             }
         } else {  // a document edge: plain loads, the outside read as spaces
             for (int t = lane; t < kWinB / 16; t += 32) {
