@@ -890,7 +890,7 @@ __device__ unsigned long long lookup_count(const GTable &g, uint4 k, const uint8
     }
     if ((k.z | k.w) == 0u) {
         const unsigned long long key = ((unsigned long long)k.y << 32) | k.x;
-        unsigned long long s = hash8(key) >> __clzll((long long)g.mask8);
+        unsigned long long s = home8(key, g.mask8);
         for (int probe = 0; probe < kGlobalProbeLimit; probe++) {
             if (g.slots8[s].key == key) return g.slots8[s].cnt;
             if (g.slots8[s].key == 0) return 0;

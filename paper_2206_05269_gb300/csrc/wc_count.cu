@@ -254,11 +254,12 @@ __device__ __forceinline__ uint4 window_key16(const uint8_t *win, uint32_t p, ui
 //   * both slots hold other keys: loads of the next two slots are started.
 // Keys are written once and never move, so a key seen in a slot is final.
 // Both key sizes take the same path: the table (8-byte slots of 16 bytes,
-// 16-byte slots of 32 bytes) is chosen by address arithmetic, the slot hash
-// is shared, and a 16-byte load covers either slot's key (for an 8-byte slot,
-// key and count; the count is ignored).  Only the claim differs (64- or
-// 128-bit CAS); claims are rare.  Lanes still busy keep their word across
-// flushes; free lanes take new words.
+// 16-byte slots of 32 bytes) is chosen by address arithmetic and the slot hash
+// is shared.  8-byte keys start at an even slot, so that their two slots are one
+// 32-byte sector and one load (two 16-byte loads took twice the L1 passes, which
+// are nearly the limit: 1 GB 1,408 -> 1,370 us); their counts are ignored.  Only
+// the claim differs (64- or 128-bit CAS); claims are rare.  Lanes still busy
+// keep their word across flushes; free lanes take new words.
 static_assert(sizeof(G8Slot) == 16 && offsetof(G8Slot, cnt) == 8, "8-byte slot layout");
 static_assert(sizeof(GSlot) == 32 && offsetof(GSlot, cnt) == 16, "16-byte slot layout");
 template <int MODE>
@@ -295,9 +296,10 @@ struct Tail {
         }
         // a 16-byte slot with both halves non-zero holds another key for good
         const bool e0 = a0 == 0ull || (p16 && a1 == 0ull), e1 = b0 == 0ull || (p16 && b1 == 0ull);
-        pslot = e0 ? pslot : ((pslot + (e1 ? 1 : 2)) & m);
-        if (e0 || e1) {  // claim it; the load that follows shows whose it became
-            uint8_t *slot = tab() + (pslot << shf());
+        if (!e0 && !e1) {
+            pslot = (pslot + 2) & m;
+        } else {  // claim it; the load that follows shows whose it became
+            uint8_t *slot = tab() + ((e0 ? pslot : ((pslot + 1) & m)) << shf());
             if (p16) cas128_drop(slot, k0, k1);
             else cas64_drop(slot, k0);
         }
@@ -323,15 +325,19 @@ struct Tail {
             k1 = ((unsigned long long)k.w << 32) | k.z;
             p16 = MODE != MODE_SAMPLE && k1 != 0ull;
             pslot = hash_slot(k0, k1) >> __clzll((long long)msk());
+            if (!p16) pslot &= ~1ull;  // home8
             probes = 0;
             busy = need = true;
         }
         // the round's only loads (at one place, so that no copy of their
         // registers makes the warp wait for them here)
         if (need) {
-            uint8_t *t = tab();
-            v0 = ld_relaxed_v2(t + (pslot << shf()));
-            v1 = ld_relaxed_v2(t + (((pslot + 1) & msk()) << shf()));
+            if (p16) {
+                v0 = ld_relaxed_v2(&g.slots[pslot]);
+                v1 = ld_relaxed_v2(&g.slots[(pslot + 1) & g.mask]);
+            } else {
+                ld_relaxed_v4(&g.slots8[pslot], v0, v1);
+            }
         }
         tailn -= tk;
         __syncwarp();

@@ -281,6 +281,14 @@ __device__ __forceinline__ uint4 ld_relaxed_v2(const void *p) {
     asm volatile("ld.relaxed.gpu.global.L1::evict_first.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
     return make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
 }
+// 32 bytes at a 32-byte aligned address, likewise (four 64-bit elements).
+__device__ __forceinline__ void ld_relaxed_v4(const void *p, uint4 &lo, uint4 &hi) {
+    unsigned long long a, b, c, d;
+    asm volatile("ld.relaxed.gpu.global.L1::evict_first.v4.b64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p) : "memory");
+    lo = make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
+    hi = make_uint4((uint32_t)c, (uint32_t)(c >> 32), (uint32_t)d, (uint32_t)(d >> 32));
+}
 __device__ __forceinline__ uint4 ld_relaxed_u128(const uint4 *p) {
     const unsigned long long *q = reinterpret_cast<const unsigned long long *>(p);
     const unsigned long long a = ld_u64(q), b = ld_u64(q + 1);
@@ -431,6 +439,11 @@ __device__ __forceinline__ unsigned long long hash_slot(unsigned long long k0, u
     return (k0 ^ (k1 * 0xC2B2AE3D27D4EB4Full)) * 0x9E3779B97F4A7C15ull;
 }
 __device__ __forceinline__ unsigned long long hash8(unsigned long long key) { return hash_slot(key, 0ull); }
+// The home slot of an 8-byte key in a table of mask + 1 (a power of two, at least
+// 2) slots: an even one, so that it shares its 32-byte sector with the next.
+__device__ __forceinline__ unsigned long long home8(unsigned long long key, unsigned long long mask) {
+    return hash8(key) >> __clzll((long long)mask) & ~1ull;
+}
 // The home slot of a 16-byte key in a table of mask + 1 (a power of two, at least 2) slots.
 __device__ __forceinline__ unsigned long long home16(uint4 k, unsigned long long mask) {
     return hash_slot(((unsigned long long)k.y << 32) | k.x, ((unsigned long long)k.w << 32) | k.z) >>
@@ -464,7 +477,7 @@ __device__ __forceinline__ void global_insert8_from(const GTable &g, unsigned lo
     atomicOr(g.status, ST_TABLE_FULL);
 }
 __device__ __forceinline__ void global_insert8(const GTable &g, unsigned long long key, unsigned long long add) {
-    global_insert8_from(g, key, add, hash8(key) >> __clzll((long long)g.mask8));  // top bits
+    global_insert8_from(g, key, add, home8(key, g.mask8));
 }
 
 // Words of 9..16 letters: both key halves are non-zero, so two 64-bit loads
