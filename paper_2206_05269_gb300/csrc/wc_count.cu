@@ -88,7 +88,8 @@ enum : int { MODE_HEAD = 0, MODE_LOCAL = 1, MODE_SAMPLE = 2, MODE_WIDE = 3 };  /
 template <int MODE>
 struct Geo {
     static constexpr bool kWide = MODE == MODE_HEAD || MODE == MODE_WIDE;
-    static constexpr int kWarps = MODE == MODE_HEAD ? 24 : 20;  // each with its own ring
+    static constexpr int kWarps = MODE == MODE_SAMPLE ? 20 : 24;  // each with its own ring (64 MB by WIDE: 20 warps
+                                                                  // 188 us, 24 169)
     static constexpr int kBlock = kWarps * 32;
     static constexpr int kLane = kWide ? 32 : 16;  // bytes a lane classifies per step
     static constexpr int kStrip = 32 * kLane;
