@@ -13,9 +13,13 @@
 // division plus a compensated addition took 14-16 fp64 instructions a term:
 // n = 1e8 took 2.97 ms (sqrt) and 2.60 ms (reciprocals), the FP64 pipe 86 %
 // busy.  Over a short run x0, x0 + 1, ... both functions are, to 64 bits, a
-// cubic in the offset, so a run needs fp64 only at its start (the function
-// value to 80 bits and three differences) and then three multi-word integer
-// additions a term: both series together 5.72 ms -> 0.30 ms at n = 1e8.
+// polynomial in the offset, so a run needs fp64 only at its start (the function
+// value to 80 bits and its differences) and then three or four multi-word
+// integer additions a term.  The shorter the runs, the more fp64: a quartic
+// makes the runs of the small terms eight times as long as a cubic would
+// (n = 1e8, both series: fp64 throughout 5.72 ms, cubics alone 0.212, now 0.173;
+// n = 1e6 0.043 -> 0.034).  Large n is bound by the integer pipe: 0.66 ns per
+// thousand terms.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -25,8 +29,8 @@
 namespace wc {
 
 constexpr int kSeriesThreads = 256;
-constexpr int kSeriesBlocksPerSm = 4;
-constexpr int kRunMax = 256;  // terms a run
+constexpr int kSeriesBlocksPerSm = 6;  // 40 registers; a run's set-up spills a few (5 blocks: 0.181 ms, 8: 0.177)
+constexpr int kRunMax4 = 256, kRunMax3 = 1024;  // terms a run, quartic and cubic
 
 // Fixed point of the sums: sqrt(i) >= 1 is a whole number of 2^-52, a
 // reciprocal of i < 2^53 a whole number of 2^-105.
@@ -34,15 +38,20 @@ constexpr int kUnitSqrt = 52, kUnitRecip = 106;
 
 // Terms are numbered z: x = z for the square roots and x = z + 1 for the
 // reciprocals, so that over z in [2^k, 2^(k+1)) every 1/x has one exponent (as
-// every sqrt(x) has).  A run of m terms from z0 has m <= z0 / 2^kShift.  With
-// t = m / x0 <= 2^-kShift, the first omitted term of the series is at most
-// 5/128 t^4 = 2^-68.7 of the root and t^4 = 2^-68 of the reciprocal, less than
-// 1/16 of the last of 64 bits.  z below 2^(kShift + 2) is computed directly.
+// every sqrt(x) has).  A run of m terms from there has m <= 2^k / 2^kShift4
+// (quartic) or 2^k / 2^kShift3 (cubic).  With t = m / x0, the first omitted term
+// of the series is at most 7/256 t^5 = 2^-70.2 of the root and t^5 = 2^-70 of
+// the reciprocal for a quartic, 5/128 t^4 = 2^-68.7 and t^4 = 2^-68 for a cubic:
+// at most 1/16 of the last of 64 bits.  z below kDirect is computed directly (its
+// differences would need more than the words they have here).
 template <int SERIES>
 struct SeriesCfg {
-    static constexpr int kShift = SERIES ? 17 : 16;
-    static constexpr unsigned long long kDirect = 1ull << (kShift + 2);
-    static constexpr unsigned long long kLongRuns = 1ull << (kShift + 8);  // from here on runs of kRunMax
+    static constexpr int kShift4 = SERIES ? 14 : 13, kShift3 = SERIES ? 17 : 16;
+    static constexpr unsigned long long kDirect = 1ull << (kShift4 + 3);
+    static constexpr int kShort = 5;  // power-of-two intervals with runs shorter than kRunMax4
+    static constexpr unsigned long long kLongRuns = kDirect << kShort;
+    static constexpr int kCubic = kShift3 + 8;  // from 2^kCubic on a cubic serves kRunMax4 terms
+    static_assert(kLongRuns >> kShift4 == kRunMax4, "short runs grow up to kRunMax4");
 };
 
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
@@ -67,44 +76,47 @@ __device__ __noinline__ bool above_boundary(unsigned long long x, int k, unsigne
     return (unsigned __int128)x << (106 - 2 * (k >> 1)) > (unsigned __int128)M * M;
 }
 
-// Sum of the terms z0 .. z0 + m - 1 (one power-of-two interval 2^k.., m <= kRunMax,
-// m / z0 within the bound above), in the series' units.
+// Sum of the terms z0 .. z0 + m - 1 (one power-of-two interval 2^k.., m within
+// the bound above), in the series' units, by a polynomial of degree ORDER.
 //
 // The function f scaled to [2^63, 2^64) is kept as a 64.32-bit number
-// w2:w1.w0, its first difference d1 as e2:e1.e0, its second and third as
-// 64-bit numbers of 2^-32 (d2, d3): per term w +- d1, d1 - d2, d2 - d3.  1024 is
+// w2:w1.w0, its first difference d1 as e2:e1.e0, the others as 64-bit numbers
+// of 2^-32 (d2, d3, d4): per term w +- d1, d1 - d2, d2 - d3, d3 - d4.  1024 is
 // added to w once, so that the 53-bit mantissa rounded to nearest is w >> 11.
-// Errors, in units of 2^-64 of the value: the start 2^-20, d1 is rounded to
-// 2^-17 and carries three fp64 roundings (2^-51 of at most 2^46 / kRunMax ...:
-// below 2^-4 over a run), d2 and d3 2^-33 (2^-11 over a run), the omitted
-// terms 2^-4: together far below 1.  So only when w's low 11 bits are all
-// zeros or all ones may the rounding be off, and those terms (1 in 1,024) are
-// decided exactly.
-template <int SERIES>
-__device__ __forceinline__ __int128 run_sum(unsigned long long z0, int m) {
+// Errors, in units of 2^-64 of the value: the start 2^-20; d1 is rounded to 2^-17
+// and carries up to four (the quartic's reciprocal: two) fp64 roundings of a
+// first difference that adds up to 2^49 (2^50) over a run, so 2^-2; d2 to d4
+// are rounded to 2^-33 (over 256 terms of a quartic 2^-5); the omitted terms
+// 2^-4: together well below 1 (largest found over the intervals: 0.19).  So only
+// when w's low 11 bits are all zeros or all ones may the rounding be off, and
+// those terms (1 in 1,024) are decided exactly.
+// Not inlined: the callers' 128-bit sums would raise the loops' registers.
+template <int SERIES, int ORDER>
+__device__ __noinline__ __int128 run_sum(unsigned long long z0, int m) {
     const int k = 63 - __clzll((long long)z0);
     const unsigned long long x0 = z0 + SERIES;
     const double x = (double)x0;
     const int e = SERIES ? -(k + 1) : k >> 1;  // exponent of the value
     const double S = pow2d(63 - e);
     const double u = 1.0 / x;
-    double y, dl, a1, a2, a3;  // value, its remainder, |first|, second and third differences (unscaled)
+    double y, dl, c1, c2, c3, c4 = 0.0;  // value, its remainder, |Taylor terms| of offset 1 (unscaled)
     if (SERIES) {
         y = u;
         dl = y * fma(-y, x, 1.0);
-        const double c2 = y * u * u, c3 = c2 * u;  // y u^2, y u^3
-        a1 = y * u - c2 + c3;
-        a2 = 2.0 * c2 - 6.0 * c3;
-        a3 = 6.0 * c3;
+        c1 = ORDER == 4 ? fma(y, u, 2.0 * (y * dl)) : y * u;
+        c2 = c1 * u;
+        c3 = c2 * u;
+        if (ORDER == 4) c4 = c3 * u;
     } else {
         y = sqrt(x);
-        const double c1 = 0.5 * (y * u);  // 1 / (2 sqrt(x))
+        c1 = 0.5 * (y * u);  // 1 / (2 sqrt(x))
         dl = fma(-y, y, x) * c1;
-        const double c2 = 0.25 * (c1 * u), c3 = 0.5 * (c2 * u);
-        a1 = c1 - c2 + c3;
-        a2 = 2.0 * c2 - 6.0 * c3;
-        a3 = 6.0 * c3;
+        c2 = 0.25 * (c1 * u);
+        c3 = 0.5 * (c2 * u);
+        if (ORDER == 4) c4 = 0.625 * (c3 * u);
     }
+    // |differences|
+    const double a1 = c1 - (c2 - (c3 - c4)), a2 = 2.0 * c2 - (6.0 * c3 - 14.0 * c4), a3 = 6.0 * c3 - 36.0 * c4;
     const double S32 = S * 4294967296.0;
     const long long dli = __double2ll_rn(dl * S32);
     const unsigned long long f0 = __double2ull_rn(y * S) + 1024ull + (unsigned long long)(dli >> 32);
@@ -114,7 +126,9 @@ __device__ __forceinline__ __int128 run_sum(unsigned long long z0, int m) {
     uint32_t w0 = (uint32_t)dli, w1 = (uint32_t)f0, w2 = (uint32_t)(f0 >> 32);
     uint32_t e0 = (uint32_t)(v1 << 16), e1 = (uint32_t)(v1 >> 16), e2 = (uint32_t)(v1 >> 48);
     uint32_t g0 = (uint32_t)d2i, g1 = (uint32_t)(d2i >> 32);
-    const uint32_t h0 = (uint32_t)d3i, h1 = (uint32_t)(d3i >> 32);
+    uint32_t h0 = (uint32_t)d3i, h1 = (uint32_t)(d3i >> 32);
+    const unsigned long long d4i = ORDER == 4 ? (unsigned long long)__double2ll_rn(24.0 * c4 * S32) : 0ull;
+    const uint32_t i0 = (uint32_t)d4i, i1 = (uint32_t)(d4i >> 32);
     const uint32_t top0 = w2;
     uint32_t lo = 0, hi = 0;  // sums of w1 >> 11 and of w2 (mod 2^32), signed for the reciprocals
     auto term = [&](uint32_t j, bool minus) {
@@ -140,6 +154,8 @@ __device__ __forceinline__ __int128 run_sum(unsigned long long z0, int m) {
             : "+r"(e0), "+r"(e1), "+r"(e2)
             : "r"(g0), "r"(g1));
         asm("sub.cc.u32 %0, %0, %2;\n\tsubc.u32 %1, %1, %3;" : "+r"(g0), "+r"(g1) : "r"(h0), "r"(h1));
+        if (ORDER == 4)
+            asm("sub.cc.u32 %0, %0, %2;\n\tsubc.u32 %1, %1, %3;" : "+r"(h0), "+r"(h1) : "r"(i0), "r"(i1));
     };
     if constexpr (SERIES != 0) {
         // pairs (plus, minus): the sums of differences stay far inside 32 bits
@@ -165,7 +181,7 @@ __device__ __forceinline__ __int128 run_sum(unsigned long long z0, int m) {
             term((uint32_t)j, false);
             advance();
         }
-        // the w2 of a run exceed the first by less than 2^15: their sum is known mod 2^32
+        // the w2 of a run exceed the first by less than 2^18: their sum is known mod 2^32
         const unsigned long long base = (unsigned long long)top0 * (unsigned long long)m;
         const unsigned long long his = base + (uint32_t)(hi - (uint32_t)base);
         return ((__int128)his << (21 + e)) + ((__int128)lo << e);
@@ -179,13 +195,13 @@ __device__ __forceinline__ __int128 shfl_down128(__int128 v, int o) {
 }
 
 // Every thread's terms: a strided share of the directly computed ones; a
-// strided share of the short runs (2^kShift of them in each power-of-two
-// interval up to kLongRuns, m = 1/2^kShift of the interval's start: they cost
-// mostly fp64, so they are spread over all SMs); and one contiguous piece of
-// the rest in equal runs of at most kRunMax, cut at powers of two.  A
-// block's sum goes to part[b].  Sums of n < 2^53 terms stay below 2^80 units
-// of 2^-52 over all blocks and below 2^122 within one (blocks hold at most
-// n / gridDim terms and grids of large n have hundreds of blocks).
+// strided share of the short runs (2^kShift4 of them in each power-of-two
+// interval up to kLongRuns, as long as the bound allows: they cost mostly fp64,
+// so they are spread over all SMs); and one contiguous piece of the rest in runs
+// of about equal length, cut at powers of two.  A block's sum goes to part[b].
+// Sums of n < 2^53 terms stay below 2^80 units of 2^-52 over all blocks and
+// below 2^122 within one (blocks hold at most n / gridDim terms and grids of
+// large n have hundreds of blocks).
 template <int SERIES>
 __global__ void __launch_bounds__(kSeriesThreads, kSeriesBlocksPerSm) k_series_part(unsigned long long n,
                                                                                     ulonglong2 *part) {
@@ -196,24 +212,29 @@ __global__ void __launch_bounds__(kSeriesThreads, kSeriesBlocksPerSm) k_series_p
     const unsigned long long zb = SERIES ? 0ull : 1ull, ze = n + zb;  // terms [zb, ze)
     __int128 acc = 0;
     for (unsigned long long z = zb + t; z < ze && z < C::kDirect; z += T) acc += term_direct<SERIES>(z);
-    for (unsigned long long r = t; r < (6ull << C::kShift); r += T) {
-        const int k = C::kShift + 2 + (int)(r >> C::kShift);
-        const int m = 1 << (k - C::kShift);
-        const unsigned long long z0 = (1ull << k) + (r & ((1ull << C::kShift) - 1ull)) * (unsigned long long)m;
+    for (unsigned long long r = t; r < ((unsigned long long)C::kShort << C::kShift4); r += T) {
+        const int k = C::kShift4 + 3 + (int)(r >> C::kShift4);
+        const int m = 1 << (k - C::kShift4);
+        const unsigned long long z0 = (1ull << k) + (r & ((1ull << C::kShift4) - 1ull)) * (unsigned long long)m;
         if (z0 >= ze) break;  // starts grow with r
-        acc += run_sum<SERIES>(z0, ze - z0 < (unsigned long long)m ? (int)(ze - z0) : m);
+        acc += run_sum<SERIES, 4>(z0, ze - z0 < (unsigned long long)m ? (int)(ze - z0) : m);
     }
     if (ze > C::kLongRuns) {
         const unsigned long long N = ze - C::kLongRuns, per = (N + T - 1) / T;
         unsigned long long z = C::kLongRuns + t * per;
         const unsigned long long end = z + per < ze ? z + per : ze;
-        const unsigned long long runs = (per + kRunMax - 1) / kRunMax, len = (per + runs - 1) / runs;
         while (z < end) {
-            const unsigned long long edge = 2ull << (63 - __clzll((long long)z));
-            unsigned long long stop = z + len < end ? z + len : end;
-            if (stop > edge) stop = edge;
-            acc += run_sum<SERIES>(z, (int)(stop - z));
-            z = stop;
+            const int k = 63 - __clzll((long long)z);
+            const unsigned long long edge = 2ull << k, left = (end < edge ? end : edge) - z;
+            const bool cubic = k >= C::kCubic;
+            const uint32_t most = cubic ? (uint32_t)min((1ull << k) >> C::kShift3, (unsigned long long)kRunMax3) : kRunMax4;
+            uint32_t len = most;
+            if (left < 4ull * most) {  // the last few runs share what is left
+                const uint32_t l = (uint32_t)left, runs = (l + most - 1) / most;
+                len = (l + runs - 1) / runs;
+            }
+            acc += cubic ? run_sum<SERIES, 3>(z, (int)len) : run_sum<SERIES, 4>(z, (int)len);
+            z += len;
         }
     }
     for (int o = 16; o; o >>= 1) acc += shfl_down128(acc, o);
