@@ -3,7 +3,7 @@
 Default workload: the large single-pass count -- 1e9 bytes of Zipf(1.0) text
 over a 1M-word vocabulary (~170M words), one document, 64-bit counts.  A
 step is one whole pass of the path: tokenise + two-level count, compaction
-and the radix sort into (count desc, word asc).  Inputs are resident in HBM
+and the sort into (count desc, word asc).  Inputs are resident in HBM
 when the timed region starts; 1 GB is larger than L2, so no flush is needed.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl gb300|reference]
@@ -626,16 +626,16 @@ def run_served_workload(args, local, print_line: bool = True):
     return line
 
 
-# fp64 thread instructions per term of k_series_part<0> and <1>
-# (sm__inst_executed_pipe_fp64 x 32 / n, n = 1e8)
-FP64_INSTR_PER_TERM = {0: 16.15, 1: 14.15}
+# integer-pipe thread instructions per term of k_series_part
+# (sm__inst_executed_pipe_alu x 32 / n, n = 1e8)
+ALU_INSTR_PER_TERM = 11.0
 
 
 def run_numeric(args, local) -> dict:
     """The paper's numeric MapReduce (Sec. 4.2) at n = 1e8: sum of sqrt(i)
     and the alternating harmonic sum, each term a correctly rounded double,
-    compensated sums (wc_series_sum).  FP64-pipe bound: reported against the
-    nominal FP64 rate of the part (no measured FP64 peak is available)."""
+    the sum exact and rounded once (wc_series_sum).  Bound by the 32-bit integer
+    pipe: reported against its nominal rate (64 instructions a clock and SM)."""
     import torch
     import oracle
     from paper_2206_05269_gb300 import wc
@@ -660,18 +660,17 @@ def run_numeric(args, local) -> dict:
         m = 10_000_000  # the oracle on a tenth of the terms (about a second of CPU work)
         oracle.series_sum(series, m)
         cpu_s = time.perf_counter() - t0
-        # FP64-pipe bound: fp64 instructions per term from the ncu count of
-        # this kernel (sm__inst_executed_pipe_fp64), against the part's
-        # nominal FP64 rate, 1.25 TFLOP/s with an FMA counted twice
-        per_term = FP64_INSTR_PER_TERM[series]
-        ginstr = per_term * n / (ms * 1e-3) / 1e9
+        # integer instructions per term from the ncu count of this kernel
+        # (sm__inst_executed_pipe_alu), against 64 a clock and SM at 2,070 MHz
+        ginstr = ALU_INSTR_PER_TERM * n / (ms * 1e-3) / 1e9
+        peak = 64 * torch.cuda.get_device_properties(local).multi_processor_count * 2.07
         res[name] = {"n": n, "value": got, "oracle": oracle.series_sum(series, n), "ms": ms,
                      "terms_per_s": n / (ms * 1e-3),
-                     "roofline": {"bound": "fp64", "achieved": ginstr, "peak": 625.0,
-                                  "unit": "G fp64 instructions/s", "frac": ginstr / 625.0,
-                                  "peak_kind": "nominal FP64 rate of the part (1.25 TFLOP/s, FMA = 2)",
-                                  "instr_per_term": per_term,
-                                  "instr_source": "ncu sm__inst_executed_pipe_fp64 (profiles/numeric_series_fp64.md)"},
+                     "roofline": {"bound": "int32", "achieved": ginstr, "peak": peak,
+                                  "unit": "G integer instructions/s", "frac": ginstr / peak,
+                                  "peak_kind": "nominal integer rate of the part (64 a clock and SM, 2,070 MHz)",
+                                  "instr_per_term": ALU_INSTR_PER_TERM,
+                                  "instr_source": "ncu sm__inst_executed_pipe_alu (profiles/numeric_series.md)"},
                      "cpu_baseline": {"value": m / cpu_s, "unit": "terms/s", "cores": 1, "kind": "oracle",
                                       "sample": f"first {m} terms, single-threaded compensated sum, {cpu_s:.2f} s"},
                      "paper_v100_ms": 73.372 if series == wc.WC_SERIES_SQRT else 65.323}

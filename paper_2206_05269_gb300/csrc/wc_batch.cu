@@ -6,8 +6,8 @@
 //  - a whole document (sizes up to the split threshold): one block counts it
 //    into a shared-memory table (dynamic inserts, 16-byte keys) with words of
 //    17+ letters in a small shared list, sorts the entries by (count desc,
-//    word asc) with a bitonic network in shared memory and writes them into
-//    the CSR output at an atomically reserved offset;
+//    word asc) in shared memory (order_by_parts) and writes them into the CSR
+//    output at an atomically reserved offset;
 //  - a byte range of a large document: the block counts the range (words
 //    that start in it, read past its end as needed) and adds its table into
 //    global tables keyed by (document, word).
@@ -15,7 +15,7 @@
 // (and, at the end, its shared table) to the same global tables.  Documents
 // counted there are finished by a segmented pass: the bucket sort (wc_bucket.cuh) with the
 // document ordering first, straight into the CSR output; where the document and
-// count need more than 48 bits or the tables more than 2^24 slots, compaction, a
+// count need more than 48 bits or the tables more than 2^26 slots, compaction, a
 // radix sort with the document as most significant key, and a CSR write.
 #include "wc_batch.h"
 
