@@ -201,7 +201,8 @@ struct DocShared {  // per-block scalars
     uint32_t lcount;
     uint32_t nfill;
     uint32_t spilled;
-    uint32_t nent;
+    uint32_t nshort;  // live entries of the table
+    uint32_t nent;    // these and the long words
     uint32_t nlong;
     unsigned long long base, lbase, abase, abytes;
     uint32_t ok;
@@ -445,7 +446,7 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
         // which a fix-up orders below.  The sort then moves 16-bit indices and
         // compares composites.
         if (threadIdx.x == 0) {
-            sh.nent = 0;
+            sh.nshort = 0;
             sh.nlong = 0;
         }
         __syncthreads();
@@ -455,12 +456,12 @@ __global__ void __launch_bounds__(BLOCK, (DocCfg<BLOCK, LOGC1>::MINB)) k_docs(Ba
             const bool live = scnt[i] != 0u;
             const uint32_t m = __ballot_sync(kFull, live);
             uint32_t base = 0;
-            if (lane == 0 && m) base = atomicAdd(&sh.nent, (uint32_t)__popc(m));
+            if (lane == 0 && m) base = atomicAdd(&sh.nshort, (uint32_t)__popc(m));
             base = __shfl_sync(kFull, base, 0);
             if (live) found[base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)i;
         }
         __syncthreads();
-        const uint32_t nshort = sh.nent;
+        const uint32_t nshort = sh.nshort;  // (not written again before the next barrier: a late warp reads it too)
         for (uint32_t e = threadIdx.x; e < nshort; e += BLOCK) {
             const uint32_t i = found[e];
             const uint4 k = unmark_key(skey[i]);
