@@ -81,7 +81,7 @@ __device__ __forceinline__ unsigned long long be_bytes16(const uint8_t *src, int
 // 0xFFFF - count so that a larger count sorts first), the 16-letter prefix
 // packed 5 bits a letter (80 bits, pack5 of the big-endian key halves), a
 // long-word flag and the long word's index.  Documents counted in shared
-// memory hold at most 128,000 bytes, so counts stay below 2^16.
+// memory hold at most 80,000 bytes, so counts stay below 2^16.
 __device__ __forceinline__ ulonglong2 doc_composite(unsigned long long khi, unsigned long long klo, uint32_t cnt,
                                                    bool is_long, uint32_t idx) {
     const unsigned long long ph = pack5(khi), pl = pack5(klo);  // 40 bits each

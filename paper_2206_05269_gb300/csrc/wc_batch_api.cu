@@ -18,7 +18,7 @@ namespace {
 constexpr uint64_t kSmallMax = 8 << 10;     // whole documents up to 8 KB: small shape
 constexpr uint64_t kMediumMax = 32 << 10;   // whole documents up to 32 KB: medium shape; larger: large shape
 constexpr uint64_t kSplitMin = 64 << 10;    // documents above 64 KB may be split into ranges
-constexpr uint64_t kSplitAll = 128000;      // documents above this always are (a composite holds counts below 2^16)
+constexpr uint64_t kSplitAll = 80000;       // documents above this always are
 constexpr uint64_t kRange = 32 << 10;       // byte range per item of a split document
 constexpr uint32_t kMaxDocs = 1u << 24;     // (document, word) keys carry 24 document bits
 
@@ -213,7 +213,12 @@ static wc_status batch_plan(wc_ctx *ctx, const uint64_t *h_offsets, uint32_t ndo
     // A document between the two is split when it would keep one block busy for
     // longer than a sixteenth of an even share of the batch: its words then pass
     // through the global (document, word) tables and the sort after them, which
-    // costs more in all than one block's shared table does.
+    // costs more in all than one block's shared table does where its words fit
+    // there.  Where they do not, the block has worked for nothing, so kSplitAll lies
+    // where that loss is still small.  2,500 documents of one size, ms, whole |
+    // ranges (words of a 200,000-word vocabulary, 4,700 different ones a document
+    // of 79 KB; of a 500,000-word one, 7,200): 79 KB 2.49 | 5.16 and 8.66 | 7.74,
+    // 94 KB 3.03 | 5.87 and 10.7 | 9.05, 125 KB 8.30 | 7.97 and 15.2 | 12.2.
     const uint64_t bytes = ndocs ? h_offsets[ndocs] - h_offsets[0] : 0;
     const uint64_t split = std::min(kSplitAll, std::max(kSplitMin, bytes / (16 * (uint64_t)ctx->sms)));
     std::vector<DocItem> small, medium, large;
@@ -226,11 +231,11 @@ static wc_status batch_plan(wc_ctx *ctx, const uint64_t *h_offsets, uint32_t ndo
         long_est += exact ? s / 18 + 1 : std::min<uint64_t>(s / 18 + 1, e / 8 + 2);
         total += s;
         b->max_doc_bytes = std::max(b->max_doc_bytes, s);
+        if (s > kSplitMin) glob_est += e;
         if (s <= kSmallMax) small.push_back({lo, hi, d, 0});
         else if (s <= kMediumMax) medium.push_back({lo, hi, d, 0});
         else if (s <= split) large.push_back({lo, hi, d, 0});
         else {
-            glob_est += e;
             for (uint64_t r = lo; r < hi; r += kRange) large.push_back({r, std::min(hi, r + kRange), d, 1});
         }
     }
@@ -247,8 +252,10 @@ static wc_status batch_plan(wc_ctx *ctx, const uint64_t *h_offsets, uint32_t ndo
     b->args.out_cap = out_est + 1024;
     b->args.lcap = long_est + 1024;
     b->args.arena_cap = exact ? total + b->args.lcap + 65536 : b->args.lcap * 24 + 65536;
-    // planned: split documents; reserve: documents whose shared table fills
-    // up (exact: every (document, word) pair may spill)
+    // planned: documents above kSplitMin, split or not (a block's shared tables
+    // hold 6,144 words and 64 long ones, fewer than many texts of that size have:
+    // all of such a document's words then spill); reserve: shorter documents
+    // whose shared table fills up (exact: every (document, word) pair may spill)
     b->exact = exact;
     b->cap8 = pow2_ge(exact ? 2 * out_est + (1u << 18) : 2 * glob_est + out_est / 32 + (1u << 18));
     b->cap16 = pow2_ge(exact ? out_est + out_est / 4 + (1u << 17) : glob_est + out_est / 64 + (1u << 17));
