@@ -192,11 +192,14 @@ constexpr int kBktMean = 384;    // entries a bucket is meant to hold
 constexpr int kBktStride = 8;    // words between two buckets' counters
 constexpr int kBktSplits = 0, kBktRoom = 1, kBktSpilled = 2, kBktTied = 3, kBktBig = 4, kBktTicket = 5;  // BucketScratch::state
 // Tables of more slots are radix sorted.  There are at most 2,730 splitters (54 KB
-// of shared memory in the scatter kernels); buckets of more than 2,560 entries
-// are sorted in global memory, which at 10,000 entries a bucket still takes a
-// quarter of the radix passes' time; past that the radix sort's cost an entry is
-// the smaller one.
-constexpr uint64_t kBktMaxCap = 1ull << 26;
+// of shared memory in the scatter kernels); past 1,500 entries a bucket more and
+// more buckets hold over 2,560 and are sorted in global memory, while the radix
+// passes' cost an entry stays the same.  Finish of N words, ms, bucket | radix:
+// 1 M 0.13 | 0.20-0.25; 2 M (8.5 M slots) 0.31-0.33 | 0.34-0.41; 4 M (16.8 M
+// slots) 0.74-0.79 | 0.67-0.80; 8 M 2.3-2.4 | 1.4-1.7; 12 M (2 x 2^24 slots) 4.0-4.3 |
+// 2.2-2.5.  Plans of documents split into ranges: 2.2 M rows (6.8 M slots) 0.77 |
+// 1.00, 4.5 M (13.1 M slots) 2.13 | 1.98, 18 M 11.3 | 8.65.
+constexpr uint64_t kBktMaxCap = 10ull << 20;
 struct BucketScratch {
     uint32_t groups;              // sample blocks
     unsigned long long slots;     // entries `key` and `lref` hold, shared out evenly to the buckets
