@@ -285,10 +285,10 @@ struct SortJob {
     LongView v;
     DevTable out;
 };
-// finish_table for n tables at once by the bucket sort: every step as one launch over all
-// n tables (grid.y).  d_jobs: device memory of finish_tables_job_bytes(n), alive
-// until the stream has run the launches.  Tables without bucket scratch are
-// finished one by one.
+// finish_table for n tables at once: every step of those with bucket scratch as
+// one launch over them all (grid.y), the others one by one.  d_jobs: device
+// memory of finish_tables_job_bytes(n), alive until the stream has run the
+// launches.
 struct FinishSpec {
     GTable g;
     uint64_t gcap8, gcap, glcap;

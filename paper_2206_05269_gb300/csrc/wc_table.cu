@@ -1175,42 +1175,36 @@ cudaError_t finish_table(const GTable &g, uint64_t gcap8, uint64_t gcap, uint64_
 
 size_t finish_tables_job_bytes(int n) { return sizeof(FinishJob) * (size_t)(n > 0 ? n : 1); }
 
-static bool all_by_buckets(const FinishSpec *spec, int n, uint32_t skip) {
-    for (int t = 0; t < n; t++)
-        if (!finish_by_buckets(*spec[t].bs, skip)) return false;
-    return true;
-}
-
 int finish_tables_launches(const FinishSpec *spec, int n, uint32_t skip) {
-    if (all_by_buckets(spec, n, skip)) return kBucketLaunches;
     int k = 0;
-    for (int t = 0; t < n; t++) k += finish_table_launches(*spec[t].ss, *spec[t].bs, skip);
-    return k;
+    bool buckets = false;
+    for (int t = 0; t < n; t++) {
+        if (finish_by_buckets(*spec[t].bs, skip)) buckets = true;
+        else k += finish_table_launches(*spec[t].ss, *spec[t].bs, skip);
+    }
+    return k + (buckets ? kBucketLaunches : 0);
 }
 
 cudaError_t finish_tables(const FinishSpec *spec, int n, void *d_jobs, cudaStream_t st, uint32_t skip) {
-    if (n <= 0) return cudaSuccess;
-    if (!all_by_buckets(spec, n, skip)) {
-        for (int t = 0; t < n; t++) {
-            const FinishSpec &f = spec[t];
-            const cudaError_t e = finish_table(f.g, f.gcap8, f.gcap, f.glcap, *f.ss, *f.bs, *f.out, st, skip);
-            if (e != cudaSuccess) return e;
-        }
-        return cudaSuccess;
-    }
-    std::vector<FinishJob> jobs((size_t)n);
+    std::vector<FinishJob> jobs;
     uint64_t cap = 0;
-    const BucketScratch *most = spec[0].bs;
+    const BucketScratch *most = nullptr;
     for (int t = 0; t < n; t++) {
         const FinishSpec &f = spec[t];
-        jobs[t] = FinishJob{f.g, f.gcap8, f.gcap, f.glcap, *f.bs, *f.out};
+        if (!finish_by_buckets(*f.bs, skip)) {
+            const cudaError_t e = finish_table(f.g, f.gcap8, f.gcap, f.glcap, *f.ss, *f.bs, *f.out, st, skip);
+            if (e != cudaSuccess) return e;
+            continue;
+        }
+        jobs.push_back(FinishJob{f.g, f.gcap8, f.gcap, f.glcap, *f.bs, *f.out});
         cap = std::max<uint64_t>(cap, f.gcap8 + f.gcap + f.glcap);
-        if (f.bs->groups > most->groups) most = f.bs;
+        if (!most || f.bs->groups > most->groups) most = f.bs;
     }
+    if (jobs.empty()) return cudaSuccess;
     const cudaError_t e =
         cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(FinishJob) * jobs.size(), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return e;
-    return launch_buckets(FinishList{static_cast<const FinishJob *>(d_jobs)}, *most, cap, n, st);
+    return launch_buckets(FinishList{static_cast<const FinishJob *>(d_jobs)}, *most, cap, (int)jobs.size(), st);
 }
 
 // ---------------------------------------------------------------- merge
