@@ -103,24 +103,33 @@ void wc_ctx::release(void *p, size_t bytes, cudaStream_t s) {
     used -= bytes;
 }
 
+// In a thread (or beside one) with a stream capture under way an event query
+// would invalidate the capture, although none of these events was recorded in
+// one: the relaxed mode allows it.  Only an event that has been seen to pass is
+// taken off the charge and used again.
 void wc_ctx::collect(bool all) {
+    if (freed.empty()) return;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
     auto passed = [&](const Freed &f) {
-        const cudaError_t e = cudaEventQuery(f.ev);
-        if (e == cudaErrorNotReady) {
+        if (cudaEventQuery(f.ev) != cudaSuccess) {  // not yet, or the device failed
             cudaGetLastError();
             return false;
         }
-        if (e != cudaSuccess) cudaGetLastError();  // the stream or device failed: nothing will use the bytes
         used -= f.bytes;
         spare_events.push_back(f.ev);
         return true;
     };
     while (!freed.empty() && passed(freed.front())) freed.pop_front();
-    if (!all) return;
-    for (size_t i = 0; i < freed.size();) {
-        if (passed(freed[i])) freed.erase(freed.begin() + (long)i);
-        else i++;
-    }
+    if (all)
+        for (size_t i = 0; i < freed.size();) {
+            if (passed(freed[i])) freed.erase(freed.begin() + (long)i);
+            else i++;
+        }
+    cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
 void wc_ctx::prof_mark(std::vector<cudaEvent_t> &v, cudaStream_t s) {
