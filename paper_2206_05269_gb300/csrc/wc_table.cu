@@ -1263,11 +1263,16 @@ __global__ void k_topk_copy(DevTable in, unsigned long long k, DevTable out) {
         out.d_meta[2] = ab;
         *out.d_status = *in.d_status;
     }
-    unsigned long long tok = 0, bytes = 0;
+    // meta[1] keeps the length of the long words' list, all of which is copied; the
+    // rows' own kinds are counted (a merge sizes its tables by them)
+    unsigned long long tok = 0, bytes = 0, n8 = 0, n16 = 0;
     for (unsigned long long i = t; i < m; i += stride) {
+        const unsigned long long klo = in.klo[i];
         out.khi[i] = in.khi[i];
-        out.klo[i] = in.klo[i];
+        out.klo[i] = klo;
         uint32_t r = in.lref[i];
+        n8 += !r && !klo ? 1u : 0u;
+        n16 += !r && klo ? 1u : 0u;
         out.lref[i] = r;
         unsigned long long c;
         if (in.count_bits == 32) c = static_cast<const uint32_t *>(in.cnt)[i];
@@ -1275,7 +1280,7 @@ __global__ void k_topk_copy(DevTable in, unsigned long long k, DevTable out) {
         if (out.count_bits == 32) static_cast<uint32_t *>(out.cnt)[i] = (uint32_t)c;
         else static_cast<unsigned long long *>(out.cnt)[i] = c;
         tok += c;
-        bytes += r ? in.llen[r - 1] : short_len(in.khi[i], in.klo[i]);
+        bytes += r ? in.llen[r - 1] : short_len(in.khi[i], klo);
     }
     for (unsigned long long i = t; i < nl; i += stride) {
         out.loff[i] = in.loff[i];
@@ -1285,10 +1290,14 @@ __global__ void k_topk_copy(DevTable in, unsigned long long k, DevTable out) {
     for (int d = 16; d; d >>= 1) {
         tok += __shfl_xor_sync(kFull, tok, d);
         bytes += __shfl_xor_sync(kFull, bytes, d);
+        n8 += __shfl_xor_sync(kFull, n8, d);
+        n16 += __shfl_xor_sync(kFull, n16, d);
     }
     if ((threadIdx.x & 31) == 0) {
         if (tok) atomicAdd(&out.d_meta[3], tok);
         if (bytes) atomicAdd(&out.d_meta[4], bytes);
+        if (n8) atomicAdd(&out.d_meta[5], n8);
+        if (n16) atomicAdd(&out.d_meta[6], n16);
     }
 }
 
