@@ -398,6 +398,15 @@ def _stream_handle(stream) -> int:
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
 
+def _free_once(obj, free) -> None:
+    """Frees an owned object's handle, unless its Counter has: in a reference
+    cycle's end the collector runs the finalizers in any order."""
+    handle, held = getattr(obj, "handle", None), getattr(obj, "_held", None)
+    obj.handle = None
+    if handle and (held is None or held.pop(handle, None)):
+        free(handle)
+
+
 class Table:
     """Owns a wc_table handle (or borrows one from a batch, which it keeps
     alive).  An owned table registers with its Counter, which frees it before
@@ -411,13 +420,14 @@ class Table:
         self._owner = owner  # the batch a borrowed table reads from
         if owned and counter is not None:
             counter._track(self)
+            self._held = counter._hold(handle, wc_table_free)
 
     def __del__(self):
         self.free()
 
     def free(self):
-        if getattr(self, "handle", None) and self.owned:
-            wc_table_free(self.handle)
+        if getattr(self, "owned", False):
+            _free_once(self, wc_table_free)
         self.handle = None
 
     def status(self) -> int:
@@ -458,6 +468,7 @@ class Batch:
         self._owner = owner
         if owned and counter is not None:
             counter._track(self)
+            self._held = counter._hold(handle, wc_batch_free)
 
     def status(self) -> int:
         return wc_batch_status(self.handle)
@@ -516,8 +527,8 @@ class Batch:
         return out
 
     def free(self):
-        if getattr(self, "handle", None) and self.owned:
-            wc_batch_free(self.handle)
+        if getattr(self, "owned", False):
+            _free_once(self, wc_batch_free)
         self.handle = None
 
     def __del__(self):
@@ -561,15 +572,24 @@ class Counter:
     def __init__(self, device: int = 0, budget: int = 0, count_bits: int = 64, autotune: bool = False,
                  tune_cache_path: str | None = None):
         self._live = weakref.WeakSet()  # owned tables, batches and plans of this context
+        self._held = {}  # and what frees their handles: the set forgets objects that the cyclic collector has found
         self.ctx = wc_create(device, budget, count_bits, int(autotune), tune_cache_path)
 
     def _track(self, obj) -> None:
         self._live.add(obj)
 
+    def _hold(self, handle, free) -> dict:
+        self._held[handle] = free
+        return self._held
+
     def close(self):
         """Frees every table, batch and plan still alive, then the context."""
         for obj in list(getattr(self, "_live", ())):
             obj.free()
+        held = getattr(self, "_held", {})
+        while held:
+            handle, free = held.popitem()
+            free(handle)
         if getattr(self, "ctx", None):
             wc_destroy(self.ctx)
             self.ctx = None
@@ -680,6 +700,7 @@ class Plan:
         self.ndocs = int(np.asarray(h_offsets).size - 1)
         self.handle = wc_plan_create(counter.ctx, h_offsets, nclasses, _stream_handle(stream))
         counter._track(self)
+        self._held = counter._hold(self.handle, wc_plan_free)
 
     def run(self, text, offsets, classes=None, stream=None) -> Batch:
         h = wc_plan_run(self.counter.ctx, self.handle, text.data_ptr(), offsets.data_ptr(),
@@ -687,9 +708,7 @@ class Plan:
         return Batch(h, self.ndocs, owned=False, owner=self)
 
     def free(self):
-        if getattr(self, "handle", None):
-            wc_plan_free(self.handle)
-        self.handle = None
+        _free_once(self, wc_plan_free)
 
     def __del__(self):
         self.free()
