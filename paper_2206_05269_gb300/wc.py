@@ -403,7 +403,7 @@ def _free_once(obj, free) -> None:
     cycle's end the collector runs the finalizers in any order."""
     handle, held = getattr(obj, "handle", None), getattr(obj, "_held", None)
     obj.handle = None
-    if handle and (held is None or held.pop(handle, None)):
+    if handle and (held is None or held.pop(handle.value, None)):
         free(handle)
 
 
@@ -579,7 +579,7 @@ class Counter:
         self._live.add(obj)
 
     def _hold(self, handle, free) -> dict:
-        self._held[handle] = free
+        self._held[handle.value] = (handle, free)
         return self._held
 
     def close(self):
@@ -588,7 +588,7 @@ class Counter:
             obj.free()
         held = getattr(self, "_held", {})
         while held:
-            handle, free = held.popitem()
+            _, (handle, free) = held.popitem()
             free(handle)
         if getattr(self, "ctx", None):
             wc_destroy(self.ctx)
