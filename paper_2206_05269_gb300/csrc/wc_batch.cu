@@ -900,7 +900,7 @@ struct SegSource {
         const LSlot &l = j.g.lslots[i];
         if (l.h == 0ull && l.addr == 0ull) return false;
         k = j.keylong(reinterpret_cast<const uint8_t *>(l.addr), l.cnt);
-        tie = (uint32_t)i;
+        tie = (uint32_t)i + 1u;  // 0: the short words'
         return true;
     }
 };
@@ -971,7 +971,7 @@ __global__ void __launch_bounds__(kSegThreads, 2) k_seg_scatter(SegJob j) {
         if (!occ) return;
         n++;
         nl++;
-        bucket_put(j.s, sp, j.keylong(src, c), (uint32_t)slot, lref);
+        bucket_put(j.s, sp, j.keylong(src, c), (uint32_t)slot + 1u, lref);
     });
     n = __reduce_add_sync(kFull, n);
     nl = __reduce_add_sync(kFull, nl);

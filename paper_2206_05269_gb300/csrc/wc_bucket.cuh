@@ -76,7 +76,8 @@ constexpr int kBktThreads = 256;
 constexpr int kBktProbes = 512;  // slots a sample block reads
 
 // Source: cap slots; get(i, key, tie): whether slot i holds an entry, its key
-// and a number that tells entries of equal keys apart.
+// and a number that tells entries of equal keys apart (all of them: two equal
+// samples would take one rank and leave the next, maybe a splitter, unwritten).
 template <class Source>
 __device__ __forceinline__ void bucket_sample(const BucketScratch &s, const Source &src) {
     __shared__ uint32_t nv;

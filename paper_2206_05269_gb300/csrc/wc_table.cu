@@ -957,7 +957,7 @@ struct TableSource {
         if (l.h == 0ull && l.addr == 0ull) return false;
         const uint4 f = (l.len & kLongReady) ? l.f : load_run16(reinterpret_cast<const uint8_t *>(l.addr), 16);
         k = count_key(l.cnt, be_half(f.x, f.y), be_half(f.z, f.w));
-        tie = (uint32_t)i;
+        tie = (uint32_t)i + 1u;  // 0: the short words'
         return true;
     }
 };
@@ -1042,7 +1042,7 @@ __global__ void __launch_bounds__(kScatterThreads, kScatterPerSm) k_bucket_scatt
                         nl++;
                         tok += c;
                         bytes += len;
-                        bucket_put(j.s, sp, count_key(c, khi, klo), (uint32_t)slot, lref);
+                        bucket_put(j.s, sp, count_key(c, khi, klo), (uint32_t)slot + 1u, lref);
                     });
     for (int d = 16; d; d >>= 1) {
         n8 += __shfl_xor_sync(kFull, n8, d);
