@@ -49,9 +49,12 @@ wc_status wc_ctx::alloc(void **p, size_t bytes, cudaStream_t s) {
     *p = nullptr;
     if (bytes == 0) bytes = 256;
     bytes = (bytes + 255) & ~(size_t)255;
+    // what streams have passed is off the charge before it could refuse these
+    // bytes or count in a new peak
+    const uint64_t want = used.load() + bytes;
+    collect((budget && want > budget) || want > peak.load());
     // reserve the bytes against the budget first (compare-and-swap: two
     // callers can never both pass a budget that holds only one of them)
-    collect(budget && used.load() + bytes > budget);
     uint64_t cur = used.load();
     do {
         if (budget && cur + bytes > budget) return fail(WC_ERR_BUDGET, "allocation over the context budget");
