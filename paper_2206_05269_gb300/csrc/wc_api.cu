@@ -89,15 +89,22 @@ void wc_ctx::release(void *p, size_t bytes, cudaStream_t s) {
     }
     if (cap == cudaStreamCaptureStatusNone) {
         cudaEvent_t ev = nullptr;
-        if (!spare_events.empty()) {
-            ev = spare_events.back();
-            spare_events.pop_back();
-        } else if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
-            ev = nullptr;
+        {
+            std::lock_guard<std::mutex> g(freed_mu);
+            if (!spare_events.empty()) {
+                ev = spare_events.back();
+                spare_events.pop_back();
+            }
         }
+        if (!ev && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) ev = nullptr;
         if (ev && cudaEventRecord(ev, s) == cudaSuccess) {
-            freed.push_back(Freed{ev, bytes});
-            if (freed.size() > 1024) collect(true);
+            size_t n = 0;
+            {
+                std::lock_guard<std::mutex> g(freed_mu);
+                freed.push_back(Freed{ev, bytes});
+                n = freed.size();
+            }
+            if (n > 1024) collect(true);
             return;
         }
         cudaGetLastError();
@@ -111,6 +118,7 @@ void wc_ctx::release(void *p, size_t bytes, cudaStream_t s) {
 // one: the relaxed mode allows it.  Only an event that has been seen to pass is
 // taken off the charge and used again.
 void wc_ctx::collect(bool all) {
+    std::lock_guard<std::mutex> g(freed_mu);
     if (freed.empty()) return;
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {

@@ -55,11 +55,14 @@ struct wc_ctx {
     void release(void *p, size_t bytes, cudaStream_t s);
     // Stream-ordered frees still charged to `used`: each with an event recorded
     // behind it.  collect(all) takes those whose event has passed off the charge,
-    // from the oldest to the first that has not (all: every one).
+    // from the oldest to the first that has not (all: every one).  Under a lock:
+    // objects may be freed by another thread (a garbage collector's) than the one
+    // that uses the context.
     struct Freed {
         cudaEvent_t ev;
         size_t bytes;
     };
+    std::mutex freed_mu;
     std::deque<Freed> freed;
     std::vector<cudaEvent_t> spare_events;
     void collect(bool all);
