@@ -52,7 +52,7 @@ wc_status wc_ctx::alloc(void **p, size_t bytes, cudaStream_t s) {
     // what streams have passed is off the charge before it could refuse these
     // bytes or count in a new peak
     const uint64_t want = used.load() + bytes;
-    collect((budget && want > budget) || want > peak.load());
+    collect(s, (budget && want > budget) || want > peak.load());
     // reserve the bytes against the budget first (compare-and-swap: two
     // callers can never both pass a budget that holds only one of them)
     uint64_t cur = used.load();
@@ -98,13 +98,15 @@ void wc_ctx::release(void *p, size_t bytes, cudaStream_t s) {
         }
         if (!ev && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) ev = nullptr;
         if (ev && cudaEventRecord(ev, s) == cudaSuccess) {
-            size_t n = 0;
+            bool many = false;
             {
                 std::lock_guard<std::mutex> g(freed_mu);
-                freed.push_back(Freed{ev, bytes});
-                n = freed.size();
+                auto q = std::find_if(freed.begin(), freed.end(), [&](const FreedOn &f) { return f.stream == s; });
+                if (q == freed.end()) q = freed.insert(q, FreedOn{s, {}});
+                q->waiting.push_back(Freed{ev, bytes});
+                many = ++nfreed > freed_limit;
             }
-            if (n > 1024) collect(true);
+            if (many) collect(s, true);
             return;
         }
         cudaGetLastError();
@@ -117,29 +119,33 @@ void wc_ctx::release(void *p, size_t bytes, cudaStream_t s) {
 // would invalidate the capture, although none of these events was recorded in
 // one: the relaxed mode allows it.  Only an event that has been seen to pass is
 // taken off the charge and used again.
-void wc_ctx::collect(bool all) {
+void wc_ctx::collect(cudaStream_t s, bool all) {
     std::lock_guard<std::mutex> g(freed_mu);
-    if (freed.empty()) return;
+    if (!nfreed) return;
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
         cudaGetLastError();
         return;
     }
-    auto passed = [&](const Freed &f) {
-        if (cudaEventQuery(f.ev) != cudaSuccess) {  // not yet, or the device failed
-            cudaGetLastError();
-            return false;
+    for (FreedOn &f : freed) {
+        if (!all && f.stream != s) continue;
+        while (!f.waiting.empty()) {
+            const Freed x = f.waiting.front();
+            if (cudaEventQuery(x.ev) != cudaSuccess) {  // not yet, or the device failed
+                cudaGetLastError();
+                break;
+            }
+            used -= x.bytes;
+            nfreed--;
+            if (spare_events.size() < 1024) spare_events.push_back(x.ev);
+            else cudaEventDestroy(x.ev);
+            f.waiting.pop_front();
         }
-        used -= f.bytes;
-        spare_events.push_back(f.ev);
-        return true;
-    };
-    while (!freed.empty() && passed(freed.front())) freed.pop_front();
-    if (all)
-        for (size_t i = 0; i < freed.size();) {
-            if (passed(freed[i])) freed.erase(freed.begin() + (long)i);
-            else i++;
-        }
+    }
+    if (all) {
+        freed.erase(std::remove_if(freed.begin(), freed.end(), [](const FreedOn &f) { return f.waiting.empty(); }), freed.end());
+        freed_limit = std::max<size_t>(1024, 2 * nfreed);
+    }
     cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
@@ -286,8 +292,9 @@ void wc_destroy(wc_ctx *ctx) {
     cudaSetDevice(ctx->device);
     cudaDeviceSynchronize();
     prof_clear(ctx);
-    ctx->collect(true);
-    for (auto &f : ctx->freed) cudaEventDestroy(f.ev);
+    ctx->collect(nullptr, true);
+    for (auto &f : ctx->freed)
+        for (auto &x : f.waiting) cudaEventDestroy(x.ev);
     for (auto e : ctx->spare_events) cudaEventDestroy(e);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     if (ctx->meta_host) cudaFreeHost(ctx->meta_host);
@@ -344,7 +351,7 @@ wc_status wc_buffer_free(wc_ctx *ctx, void *p, uint64_t bytes, cudaStream_t stre
 wc_status wc_mem_usage(wc_ctx *ctx, uint64_t *used, uint64_t *peak, int reset) {
     if (!ctx) return WC_ERR_INVALID_ARG;
     cudaSetDevice(ctx->device);
-    ctx->collect(true);
+    ctx->collect(nullptr, true);
     const uint64_t u = ctx->used.load();
     if (used) *used = u;
     if (peak) *peak = ctx->peak.load();

@@ -54,18 +54,25 @@ struct wc_ctx {
     wc_status alloc(void **p, size_t bytes, cudaStream_t s);
     void release(void *p, size_t bytes, cudaStream_t s);
     // Stream-ordered frees still charged to `used`: each with an event recorded
-    // behind it.  collect(all) takes those whose event has passed off the charge,
-    // from the oldest to the first that has not (all: every one).  Under a lock:
-    // objects may be freed by another thread (a garbage collector's) than the one
-    // that uses the context.
+    // behind it, by stream, oldest first.  collect(s, all) takes those that stream
+    // s (all: every stream) has passed off the charge: one query a stream beyond
+    // them, however many wait.  A release looks at all from freed_limit entries
+    // on, at least twice what the last look left.  Under a lock: objects may be
+    // freed by another thread (a garbage collector's) than the one that uses the
+    // context.
     struct Freed {
         cudaEvent_t ev;
         size_t bytes;
     };
+    struct FreedOn {
+        cudaStream_t stream;
+        std::deque<Freed> waiting;
+    };
     std::mutex freed_mu;
-    std::deque<Freed> freed;
+    std::vector<FreedOn> freed;
+    size_t nfreed = 0, freed_limit = 1024;
     std::vector<cudaEvent_t> spare_events;
-    void collect(bool all);
+    void collect(cudaStream_t s, bool all);
 };
 
 struct wc_table {

@@ -1,5 +1,6 @@
 """The peak of wc_mem_usage leaves out memory whose free its stream has passed,
-also while another stream's older free waits."""
+also while another stream's older free waits; thousands of waiting frees do not
+hold up the host."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -31,3 +32,38 @@ def test_peak_beside_a_waiting_stream():
     torch.cuda.synchronize()
     assert ctr.mem_usage()[0] == 0
     ctr.close()
+
+
+def test_thousands_of_waiting_frees():
+    """Giving memory back takes microseconds; looking at every waiting free on
+    every release took tenths of a millisecond."""
+    import time
+
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2206_05269_gb300 import wc
+    ctr = wc.Counter(0)
+    streams = [torch.cuda.Stream() for _ in range(8)]
+
+    def host_seconds(n):
+        t0 = time.perf_counter()
+        for _ in range(n):
+            for s in streams:
+                p = wc.wc_buffer_alloc(ctr.ctx, 4096, s.cuda_stream)
+                wc.wc_buffer_free(ctr.ctx, p, 4096, s.cuda_stream)
+        return time.perf_counter() - t0
+
+    host_seconds(350)  # pools and events made
+    torch.cuda.synchronize()
+    idle = host_seconds(350)
+    torch.cuda.synchronize()
+    for s in streams:
+        with torch.cuda.stream(s):
+            torch.cuda._sleep(2_000_000_000)  # about a second
+    waiting = host_seconds(350)  # 2,800 frees
+    assert not streams[0].query(), f"the streams' work ended before the host's ({waiting:.3f} s)"
+    torch.cuda.synchronize()
+    assert ctr.mem_usage()[0] == 0
+    ctr.close()
+    assert waiting < 4 * idle + 0.02, (waiting, idle)
