@@ -567,7 +567,7 @@ wc_status wc_table_export(const wc_table *t, uint8_t *h_words, uint64_t *h_word_
         if ((s = ctx->alloc(&mem, sb + wb + ob, stream)) != WC_OK) return abandon(s);
         uint8_t *dwords = static_cast<uint8_t *>(mem) + sb;
         unsigned long long *doffs = reinterpret_cast<unsigned long long *>(dwords + wb);
-        e = launch_export(d, n, mem, dwords, doffs, stream);
+        e = launch_export(d, n, t->word_bytes, mem, dwords, doffs, stream);
         if (e == cudaSuccess && h_words && t->word_bytes)
             e = cudaMemcpyAsync(h_words, dwords, t->word_bytes, cudaMemcpyDeviceToHost, stream);
         if (e == cudaSuccess && h_word_offsets)

@@ -318,9 +318,9 @@ constexpr int kMergeChunk = 256;  // rows a merge block inserts, one a thread
 
 cudaError_t launch_topk_copy(const DevTable &in, uint64_t k, DevTable &out, cudaStream_t s);
 
-// Export of a table's n rows: word lengths -> offsets -> bytes, on the device.
+// Export of a table's n rows of word_bytes letters: word lengths -> offsets -> bytes, on the device.
 size_t export_scratch_bytes(uint64_t n);
-cudaError_t launch_export(const DevTable &t, uint64_t n, void *scratch, uint8_t *d_words, unsigned long long *d_offs,
-                          cudaStream_t s);
+cudaError_t launch_export(const DevTable &t, uint64_t n, uint64_t word_bytes, void *scratch, uint8_t *d_words,
+                          unsigned long long *d_offs, cudaStream_t s);
 
 }  // namespace wc

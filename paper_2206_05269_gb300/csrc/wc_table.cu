@@ -1401,7 +1401,12 @@ __global__ void k_export_write(DevTable t, unsigned long long *offs, const unsig
 }
 
 // A table of at most kExportSmall rows in one block: lengths, their scan and the
-// bytes (three launches for a top-100 answer were most of its device time).
+// bytes, a thread its rows' words of up to 64 letters, the whole warp each longer
+// one.  One launch for three, but one block writes slowly: tables of more than
+// 16 KB of letters, or of more than 24 a row, go to the grid.  Export, us, one
+// block | grid: 100 words of 8 letters 36 | 44, of 30 40 | 43, of 40 50 | 44; 1,000 of
+// 14 39 | 44, of 20 50 | 44; 2,000 of 7 38 | 44, of 14 51 | 44; 4,000 of 4 38 | 43, of 7
+// 50 | 43.
 constexpr int kExportSmall = 4096, kExportSmallThreads = 1024;
 __global__ void __launch_bounds__(kExportSmallThreads) k_export_small(DevTable t, uint32_t n, unsigned long long *offs,
                                                                       uint8_t *words) {
@@ -1435,25 +1440,31 @@ __global__ void __launch_bounds__(kExportSmallThreads) k_export_small(DevTable t
 #pragma unroll
     for (int q = 0; q < kPer; q++) {
         const uint32_t i = i0 + q;
-        if (i < n) {
-            offs[i] = run;
-            const uint8_t *p = r[q] ? t.arena + t.loff[r[q] - 1] : nullptr;
+        const bool have = i < n, warp_word = have && len[q] > 64;  // (such words by the whole warp)
+        const uint8_t *p = r[q] ? t.arena + t.loff[r[q] - 1] : nullptr;
+        if (have) offs[i] = run;
+        if (have && !warp_word)
             for (unsigned long long j = 0; j < len[q]; j++)
                 words[run + j] = p ? p[j] : (uint8_t)((j < 8 ? hi[q] >> (56 - 8 * j) : lo[q] >> (56 - 8 * (j - 8))) & 0xFF);
+        for (uint32_t m = __ballot_sync(kFull, warp_word); m; m &= m - 1u) {
+            const int l = __ffs((int)m) - 1;
+            const unsigned long long src = __shfl_sync(kFull, (unsigned long long)reinterpret_cast<uintptr_t>(p), l);
+            const unsigned long long to = __shfl_sync(kFull, run, l), letters = __shfl_sync(kFull, len[q], l);
+            for (unsigned long long j = lane; j < letters; j += 32) words[to + j] = reinterpret_cast<const uint8_t *>(src)[j];
         }
         run += len[q];
     }
     if (threadIdx.x == kExportSmallThreads - 1) offs[n] = run;
 }
 
-cudaError_t launch_export(const DevTable &t, uint64_t n, void *scratch, uint8_t *d_words, unsigned long long *d_offs,
-                          cudaStream_t s) {
-    if (n <= (uint64_t)kExportSmall) {
+cudaError_t launch_export(const DevTable &t, uint64_t n, uint64_t word_bytes, void *scratch, uint8_t *d_words,
+                          unsigned long long *d_offs, cudaStream_t s) {
+    if (n <= (uint64_t)kExportSmall && word_bytes <= (16u << 10) && word_bytes <= 24 * n) {
         k_export_small<<<1, kExportSmallThreads, 0, s>>>(t, (uint32_t)n, d_offs, d_words);
         return cudaGetLastError();
     }
     unsigned long long *blocksum = static_cast<unsigned long long *>(scratch);
-    const int nb = (int)((n + kScanBlock - 1) / kScanBlock);
+    const int nb = (int)((n + kScanBlock - 1) / kScanBlock);  // (n = 0 has no letters: above)
     k_export_lens<<<nb, 256, 0, s>>>(t, d_offs, blocksum);
     k_export_blocksums<<<1, kBlockSumThreads, 0, s>>>(t, blocksum, d_offs);
     k_export_write<<<grid_for(n, 256, sm_count() * 8), 256, 0, s>>>(t, d_offs, blocksum, d_words);
