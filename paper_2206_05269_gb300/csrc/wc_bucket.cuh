@@ -486,7 +486,7 @@ __device__ __forceinline__ void bucket_sort(const BucketScratch &s, BucketShared
     if (t + 1 < (uint32_t)kBktCoarse) sh.cand[t] = key[(t + 1) * m / kBktCoarse];
     for (uint32_t i = t; i < parts; i += kBktSortThreads) sh.pstart[i] = 0u;
     __syncthreads();
-    {   // the coarse splitters in order: eight threads rank one
+    {   // the coarse splitters in order: sixteen threads rank one
         constexpr uint32_t kLanes = kBktSortThreads / kBktCoarse;
         const uint32_t i = t / kLanes;
         uint32_t r = 0;
