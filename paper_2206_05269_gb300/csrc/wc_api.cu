@@ -49,10 +49,10 @@ wc_status wc_ctx::alloc(void **p, size_t bytes, cudaStream_t s) {
     *p = nullptr;
     if (bytes == 0) bytes = 256;
     bytes = (bytes + 255) & ~(size_t)255;
-    // what streams have passed is off the charge before it could refuse these
+    // what streams have passed is taken off the charge where it could refuse these
     // bytes or count in a new peak
     const uint64_t want = used.load() + bytes;
-    collect(s, (budget && want > budget) || want > peak.load());
+    if ((budget && want > budget) || want > peak.load()) collect();
     // reserve the bytes against the budget first (compare-and-swap: two
     // callers can never both pass a budget that holds only one of them)
     uint64_t cur = used.load();
@@ -88,25 +88,20 @@ void wc_ctx::release(void *p, size_t bytes, cudaStream_t s) {
         cap = cudaStreamCaptureStatusActive;  // unknown: do not defer
     }
     if (cap == cudaStreamCaptureStatusNone) {
-        cudaEvent_t ev = nullptr;
-        {
-            std::lock_guard<std::mutex> g(freed_mu);
-            if (!spare_events.empty()) {
-                ev = spare_events.back();
-                spare_events.pop_back();
-            }
+        cudaEvent_t ev = take_event();
+        if (!ev) {  // those of passed frees
+            collect();
+            ev = take_event();
         }
         if (!ev && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) ev = nullptr;
         if (ev && cudaEventRecord(ev, s) == cudaSuccess) {
-            bool many = false;
             {
                 std::lock_guard<std::mutex> g(freed_mu);
                 auto q = std::find_if(freed.begin(), freed.end(), [&](const FreedOn &f) { return f.stream == s; });
                 if (q == freed.end()) q = freed.insert(q, FreedOn{s, {}});
                 q->waiting.push_back(Freed{ev, bytes});
-                many = ++nfreed > freed_limit;
+                nfreed++;
             }
-            if (many) collect(s, true);
             return;
         }
         cudaGetLastError();
@@ -115,11 +110,19 @@ void wc_ctx::release(void *p, size_t bytes, cudaStream_t s) {
     used -= bytes;
 }
 
+cudaEvent_t wc_ctx::take_event() {
+    std::lock_guard<std::mutex> g(freed_mu);
+    if (spare_events.empty()) return nullptr;
+    const cudaEvent_t ev = spare_events.back();
+    spare_events.pop_back();
+    return ev;
+}
+
 // In a thread (or beside one) with a stream capture under way an event query
 // would invalidate the capture, although none of these events was recorded in
 // one: the relaxed mode allows it.  Only an event that has been seen to pass is
 // taken off the charge and used again.
-void wc_ctx::collect(cudaStream_t s, bool all) {
+void wc_ctx::collect() {
     std::lock_guard<std::mutex> g(freed_mu);
     if (!nfreed) return;
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -127,8 +130,7 @@ void wc_ctx::collect(cudaStream_t s, bool all) {
         cudaGetLastError();
         return;
     }
-    for (FreedOn &f : freed) {
-        if (!all && f.stream != s) continue;
+    for (FreedOn &f : freed)
         while (!f.waiting.empty()) {
             const Freed x = f.waiting.front();
             if (cudaEventQuery(x.ev) != cudaSuccess) {  // not yet, or the device failed
@@ -141,11 +143,9 @@ void wc_ctx::collect(cudaStream_t s, bool all) {
             else cudaEventDestroy(x.ev);
             f.waiting.pop_front();
         }
-    }
-    if (all) {
-        freed.erase(std::remove_if(freed.begin(), freed.end(), [](const FreedOn &f) { return f.waiting.empty(); }), freed.end());
-        freed_limit = std::max<size_t>(1024, 2 * nfreed);
-    }
+    if (freed.size() > 64)  // streams come and go
+        freed.erase(std::remove_if(freed.begin(), freed.end(), [](const FreedOn &f) { return f.waiting.empty(); }),
+                    freed.end());
     cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
@@ -292,7 +292,7 @@ void wc_destroy(wc_ctx *ctx) {
     cudaSetDevice(ctx->device);
     cudaDeviceSynchronize();
     prof_clear(ctx);
-    ctx->collect(nullptr, true);
+    ctx->collect();
     for (auto &f : ctx->freed)
         for (auto &x : f.waiting) cudaEventDestroy(x.ev);
     for (auto e : ctx->spare_events) cudaEventDestroy(e);
@@ -351,7 +351,7 @@ wc_status wc_buffer_free(wc_ctx *ctx, void *p, uint64_t bytes, cudaStream_t stre
 wc_status wc_mem_usage(wc_ctx *ctx, uint64_t *used, uint64_t *peak, int reset) {
     if (!ctx) return WC_ERR_INVALID_ARG;
     cudaSetDevice(ctx->device);
-    ctx->collect(nullptr, true);
+    ctx->collect();
     const uint64_t u = ctx->used.load();
     if (used) *used = u;
     if (peak) *peak = ctx->peak.load();

@@ -54,12 +54,11 @@ struct wc_ctx {
     wc_status alloc(void **p, size_t bytes, cudaStream_t s);
     void release(void *p, size_t bytes, cudaStream_t s);
     // Stream-ordered frees still charged to `used`: each with an event recorded
-    // behind it, by stream, oldest first.  collect(s, all) takes those that stream
-    // s (all: every stream) has passed off the charge: one query a stream beyond
-    // them, however many wait.  A release looks at all from freed_limit entries
-    // on, at least twice what the last look left.  Under a lock: objects may be
-    // freed by another thread (a garbage collector's) than the one that uses the
-    // context.
+    // behind it, by stream, oldest first.  collect() takes those that their stream
+    // has passed off the charge: one query a stream beyond them, however many
+    // wait.  A release does it when no spare event is left, so about as often as
+    // the waiting frees are passed.  Under a lock: objects may be freed by another
+    // thread (a garbage collector's) than the one that uses the context.
     struct Freed {
         cudaEvent_t ev;
         size_t bytes;
@@ -70,9 +69,10 @@ struct wc_ctx {
     };
     std::mutex freed_mu;
     std::vector<FreedOn> freed;
-    size_t nfreed = 0, freed_limit = 1024;
+    size_t nfreed = 0;
     std::vector<cudaEvent_t> spare_events;
-    void collect(cudaStream_t s, bool all);
+    void collect();
+    cudaEvent_t take_event();
 };
 
 struct wc_table {
