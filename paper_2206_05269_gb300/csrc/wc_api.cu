@@ -641,7 +641,8 @@ CapPlan plan_capacity(const wc_ctx *ctx, uint64_t nbytes, const wc_count_opts *o
 }
 
 // Allocates the hash tables (+ head-selection scratch) + sort scratch in one block.
-wc_status scratch_create(wc_ctx *ctx, const CapPlan &p, bool head, cudaStream_t s, CountScratch &cs, bool radix) {
+wc_status scratch_create(wc_ctx *ctx, const CapPlan &p, bool head, cudaStream_t s, CountScratch &cs, bool radix,
+                         uint64_t rows) {
     cs.gcap8 = p.cap8;
     cs.gcap = p.cap16;
     cs.glcap = p.caplong;
@@ -649,7 +650,7 @@ wc_status scratch_create(wc_ctx *ctx, const CapPlan &p, bool head, cudaStream_t 
     const size_t b8 = r(p.cap8 * sizeof(G8Slot)), b16 = r(p.cap16 * sizeof(GSlot)), bl = r(p.caplong * sizeof(LSlot));
     const size_t hb = b8 + b16 + bl;
     const size_t bh = head ? r(head_scratch_bytes()) : 0;
-    if (cs.entries() > kBktMaxCap) radix = true;
+    if (rows ? rows > kBktMaxRows || cs.entries() > kBktMaxSparse : cs.entries() > kBktMaxCap) radix = true;
     cs.bytes = hb + bh + (radix ? sort_scratch_bytes(cs.entries()) : bucket_scratch_bytes(cs.entries())) + 512;
     wc_status st = ctx->alloc(&cs.mem, cs.bytes, s);
     if (st != WC_OK) return st;

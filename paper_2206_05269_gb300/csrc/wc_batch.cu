@@ -15,7 +15,7 @@
 // (and, at the end, its shared table) to the same global tables.  Documents
 // counted there are finished by a segmented pass: the bucket sort (wc_bucket.cuh) with the
 // document ordering first, straight into the CSR output; where the document and
-// count need more than 48 bits or the tables more than kBktMaxCap slots, compaction, a
+// count need more than 48 bits or more than kBktMaxRows rows are expected, compaction, a
 // radix sort with the document as most significant key, and a CSR write.
 #include "wc_batch.h"
 

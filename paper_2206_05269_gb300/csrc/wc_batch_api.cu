@@ -73,6 +73,7 @@ struct wc_batch {
     // lazily built
     bool tables_built = false;
     bool exact = false;  // capacities at the exact bounds
+    uint64_t seg_rows = 0;  // (document, word) rows to expect in the global tables, or 0
     uint64_t max_doc_bytes = 0, total_bytes = 0;  // bounds on counts: no count exceeds half of these
     int count_bits() const {  // bits of the largest count of a document
         return 64 - __builtin_clzll(max_doc_bytes / 2 + 1);
@@ -257,6 +258,7 @@ static wc_status batch_plan(wc_ctx *ctx, const uint64_t *h_offsets, uint32_t ndo
     // all of such a document's words then spill); reserve: shorter documents
     // whose shared table fills up (exact: every (document, word) pair may spill)
     b->exact = exact;
+    b->seg_rows = exact ? 0 : std::max<uint64_t>(1, glob_est);
     b->cap8 = pow2_ge(exact ? 2 * out_est + (1u << 18) : 2 * glob_est + out_est / 32 + (1u << 18));
     b->cap16 = pow2_ge(exact ? out_est + out_est / 4 + (1u << 17) : glob_est + out_est / 64 + (1u << 17));
     b->caplong = pow2_ge(exact ? 2 * long_est + (1u << 14) : glob_est / 8 + (1u << 14));
@@ -296,7 +298,7 @@ static wc_status batch_alloc(wc_batch *b, cudaStream_t stream) {
     a.ndocs = b->ndocs;
     // scratch: items + queue cursors, (document, word) tables, sort scratch
     CapPlan plan{b->cap8, b->cap16, b->caplong, 0};
-    st = scratch_create(ctx, plan, false, stream, b->scr.cs, b->seg_radix());
+    st = scratch_create(ctx, plan, false, stream, b->scr.cs, b->seg_radix(), b->seg_rows);
     b->scr.ibytes = sizeof(DocItem) * std::max<size_t>(b->items.size(), 1) + 256 + 16 * 8;
     void *ib = nullptr;
     if (st == WC_OK) st = ctx->alloc(&ib, b->scr.ibytes, stream);

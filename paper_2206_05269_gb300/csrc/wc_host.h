@@ -123,4 +123,6 @@ void table_mark_done(wc_table *t, cudaStream_t s);
 wc_status table_sync(const wc_table *t);
 CapPlan plan_capacity(const wc_ctx *ctx, uint64_t nbytes, const wc_count_opts *o);
 // radix: sort scratch for the radix sort even where the bucket sort would serve.
-wc_status scratch_create(wc_ctx *ctx, const CapPlan &p, bool head, cudaStream_t s, CountScratch &cs, bool radix = false);
+// rows: the entries to expect, where the slots say little about them (0: not known).
+wc_status scratch_create(wc_ctx *ctx, const CapPlan &p, bool head, cudaStream_t s, CountScratch &cs, bool radix = false,
+                         uint64_t rows = 0);

@@ -197,9 +197,15 @@ constexpr int kBktSplits = 0, kBktRoom = 1, kBktSpilled = 2, kBktTied = 3, kBktB
 // passes' cost an entry stays the same.  Finish of N words, ms, bucket | radix:
 // 1 M 0.13 | 0.20-0.25; 2 M (8.5 M slots) 0.31-0.33 | 0.34-0.41; 4 M (16.8 M
 // slots) 0.74-0.79 | 0.67-0.80; 8 M 2.3-2.4 | 1.4-1.7; 12 M (2 x 2^24 slots) 4.0-4.3 |
-// 2.2-2.5.  Plans of documents split into ranges: 2.2 M rows (6.8 M slots) 0.77 |
-// 1.00, 4.5 M (13.1 M slots) 2.13 | 1.98, 18 M 11.3 | 8.65.
+// 2.2-2.5.
+//   Batches: the (document, word) tables have several times the slots of their rows
+// where documents are large, so the rows to expect decide, up to the slots that the
+// scratch is meant for.  Plans, ms: documents of 94 KB of a 500,000-word vocabulary,
+// 2.5 M rows (1.8 M expected) 0.77 | 1.00, 5 M (3.6 M) 2.13 | 1.98, 10 M (7.2 M)
+// 5.1-5.4 | 4.12; log-normal documents, 20,000 (1.5 M expected) 1.37 | 1.62, 60,000
+// (5.0 M) 3.95 | 4.21.
 constexpr uint64_t kBktMaxCap = 10ull << 20;
+constexpr uint64_t kBktMaxRows = 5000000, kBktMaxSparse = 1ull << 26;
 struct BucketScratch {
     uint32_t groups;              // sample blocks
     unsigned long long slots;     // entries `key` and `lref` hold, shared out evenly to the buckets

@@ -896,8 +896,9 @@ void bucket_scratch_carve(BucketScratch &s, void *base, uint64_t cap) {
     while (s.tree <= s.splits()) s.tree *= 2;
     const size_t keep = (size_t)s.groups * kBktKeep, split = s.splits();
     // twice the slots: tables are at most about half full, so a bucket may
-    // hold four times its share before entries spill
-    s.slots = kOneSlot ? cap / 16 : 2 * cap;  // (the one-slot test build spills)
+    // hold four times its share before entries spill; batches' large tables,
+    // mostly sized by estimates, are emptier still and make do with their slots
+    s.slots = kOneSlot ? cap / 16 : (cap <= (1ull << 24) ? 2 * cap : cap);  // (the one-slot test build spills)
     s.kept = static_cast<ulonglong2 *>(take(keep * 16));
     s.split = static_cast<ulonglong2 *>(take(split * 16));
     s.kept_tie = static_cast<uint32_t *>(take(keep * 4));
