@@ -659,6 +659,8 @@ wc_status scratch_create(wc_ctx *ctx, const CapPlan &p, bool head, cudaStream_t 
     cs.slots = reinterpret_cast<GSlot *>(q + b8);
     cs.lslots = reinterpret_cast<LSlot *>(q + b8 + b16);
     cs.head = head ? q + hb : nullptr;
+    cs.ss = SortScratch{};  // (an earlier scratch of this object may have held the other)
+    cs.bs = BucketScratch{};
     if (radix) sort_scratch_carve(cs.ss, q + hb + bh, cs.entries());
     else bucket_scratch_carve(cs.bs, q + hb + bh, cs.entries());
     cudaMemsetAsync(cs.mem, 0, hb, s);
