@@ -659,7 +659,7 @@ static wc_status build_tables_at(wc_batch *b, const std::vector<uint64_t> &est, 
         plan.caplong = pow2_ge(std::max<uint64_t>(256, 2 * std::min<uint64_t>(d, b->nlong)));
         plan.arena = std::max<uint64_t>(4096, b->args.arena_cap);
         CountScratch &cs = c < b->nclasses ? scr[c] : b->gscratch;
-        if ((st = scratch_create(ctx, plan, false, s, cs)) != WC_OK) break;
+        if ((st = scratch_create(ctx, plan, false, s, cs, false, d)) != WC_OK) break;
         if ((st = table_create(ctx, cs.entries(), plan.caplong, plan.arena, c < b->nclasses ? 32 : ctx->count_bits,
                                s, &tabs[c])) != WC_OK)
             break;

@@ -199,7 +199,8 @@ constexpr int kBktSplits = 0, kBktRoom = 1, kBktSpilled = 2, kBktTied = 3, kBktB
 // slots) 0.74-0.79 | 0.67-0.80; 8 M 2.3-2.4 | 1.4-1.7; 12 M (2 x 2^24 slots) 4.0-4.3 |
 // 2.2-2.5.
 //   Batches: the (document, word) tables have several times the slots of their rows
-// where documents are large, so the rows to expect decide, up to the slots that the
+// where documents are large, and class and global tables are sized for a quarter of
+// the documents' rows, so the rows to expect decide, up to the slots that the
 // scratch is meant for.  Plans, ms: documents of 94 KB of a 500,000-word vocabulary,
 // 2.5 M rows (1.8 M expected) 0.77 | 1.00, 5 M (3.6 M) 2.13 | 1.98, 10 M (7.2 M)
 // 5.1-5.4 | 4.12; log-normal documents, 20,000 (1.5 M expected) 1.37 | 1.62, 60,000
